@@ -274,28 +274,47 @@ __global__ void __launch_bounds__(512, 2) ws_temporal_kernel(const TopoDev<float
     }
 }
 
-constexpr int kTile = 64;
+constexpr int kTile = 64;      // samples per tile
+constexpr int kGradThreads = 512;
+constexpr int kRow = kTile + 4;  // row stride of the [neuron][sample] arrays: 16-byte accesses to
+                                 // consecutive rows fall in different banks
+constexpr int kGradSmall = kMlpTrainable - kMlpH * kMlpH;  // gradient entries outside W2
 
 // Mean squared error of the normalised output, sum_c (o_c - t_c / s_out_c)^2 averaged
-// over n samples, and its gradient (added into grad, which the caller zeroes).
-__global__ void __launch_bounds__(256) mlp_grad_kernel(const float* __restrict__ P, const float* __restrict__ feat,
-                                                      const float* __restrict__ target, const int* __restrict__ idx,
-                                                      int n, float inv_n, float* grad, float* loss)
+// over n samples, and its gradient (added into grad, which the caller zeroes).  A block
+// works on 64 samples at a time with the activations as [neuron][sample]: each of the
+// three 64 x 64 x 64 products gives a thread a register tile of 4 x 2 outputs (three
+// shared loads per 8 or 32 multiply-adds), the gradient stays in registers over the
+// block's tiles and leaves by 16-byte reductions.  vec: grad is 16-byte aligned.
+__global__ void __launch_bounds__(kGradThreads) mlp_grad_kernel(const float* __restrict__ P, const float* __restrict__ feat,
+                                                                const float* __restrict__ target, const int* __restrict__ idx,
+                                                                int n, float inv_n, float* grad, float* loss, int vec)
 {
     extern __shared__ __align__(16) float sm[];
     float* W = sm;                         // parameters, weights rounded to BF16
-    float* G = W + kMlpParams;             // gradient accumulator
-    float* X = G + kMlpTrainable + 4;      // [tile][9] normalised inputs (pads to 16 B)
-    float* H1 = X + kTile * 12;            // [tile][64]
-    float* H2 = H1 + kTile * kMlpH;        // [tile][64]
-    float* D2 = H2 + kTile * kMlpH;        // [tile][64]
-    float* D1 = D2 + kTile * kMlpH;        // [tile][64]
-    float* DO = D1 + kTile * kMlpH;        // [tile][3]
+    float* W2T = W + kMlpParams;           // W2 transposed [i][j]
+    float* X = W2T + kMlpH * kMlpH;        // [9][sample] normalised inputs
+    float* H1 = X + kMlpIn * kRow;         // [neuron][sample]
+    float* H1r = H1 + kMlpH * kRow;        // rounded to BF16
+    float* H2 = H1r + kMlpH * kRow;
+    float* D2 = H2 + kMlpH * kRow;
+    float* D1 = D2 + kMlpH * kRow;
+    float* DO = D1 + kMlpH * kRow;         // [3][sample]
     __shared__ float red[32];
     const int tid = threadIdx.x, NT = blockDim.x;
-    for (int q = tid; q < kMlpParams; q += NT) W[q] = q < kMlpTrainable && (q < kPB1 || (q >= kPW2 && q < kPB2) || (q >= kPW3 && q < kPB3)) ? bf16_round(P[q]) : P[q];
-    for (int q = tid; q < kMlpTrainable; q += NT) G[q] = 0.f;
+    for (int q = tid; q < kMlpParams; q += NT) {
+        const bool weight = q < kPB1 || (q >= kPW2 && q < kPB2) || (q >= kPW3 && q < kPB3);
+        const float w = weight ? bf16_round(P[q]) : P[q];
+        W[q] = w;
+        if (q >= kPW2 && q < kPB2) W2T[((q - kPW2) & (kMlpH - 1)) * kMlpH + ((q - kPW2) >> 6)] = w;
+    }
     float lsum = 0.f;
+    // register tiles: neurons 4 jq .. 4 jq + 3 of samples s0, s0 + 1 (products); W2 entries
+    // (jq + 16 k, ig + 32 m) and up to two of the other gradient entries
+    const int jq = tid & 15, ig = tid >> 4, s0 = 2 * ig, j0 = 4 * jq;
+    float g2[4][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+    float gs[2] = {0.f, 0.f};
+    static_assert(kGradSmall <= 2 * kGradThreads && kMlpH == 64, "the register tiles cover the gradient");
     __syncthreads();
     const int ntiles = (n + kTile - 1) / kTile;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -307,82 +326,168 @@ __global__ void __launch_bounds__(256) mlp_grad_kernel(const float* __restrict__
                 const long long smp = idx ? idx[base + s] : base + s;
                 xv = bf16_round((feat[smp * kMlpIn + i] - W[kPMu + i]) / W[kPSig + i]);
             }
-            X[s * 12 + i] = xv;
+            X[i * kRow + s] = xv;
         }
         __syncthreads();
-        for (int e = tid; e < kTile * kMlpH; e += NT) {
-            const int s = e / kMlpH, j = e - s * kMlpH;
-            float a = W[kPB1 + j];
+        {
+            float a[4][2];
 #pragma unroll
-            for (int i = 0; i < kMlpIn; ++i) a += W[kPW1 + j * kMlpIn + i] * X[s * 12 + i];
-            H1[e] = tanhf(a);
+            for (int k = 0; k < 4; ++k) a[k][0] = a[k][1] = W[kPB1 + j0 + k];
+#pragma unroll
+            for (int i = 0; i < kMlpIn; ++i) {
+                const float2 x = *reinterpret_cast<const float2*>(X + i * kRow + s0);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float w = W[kPW1 + (j0 + k) * kMlpIn + i];
+                    a[k][0] += w * x.x;
+                    a[k][1] += w * x.y;
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float2 h = make_float2(tanhf(a[k][0]), tanhf(a[k][1]));
+                *reinterpret_cast<float2*>(H1 + (j0 + k) * kRow + s0) = h;
+                *reinterpret_cast<float2*>(H1r + (j0 + k) * kRow + s0) = make_float2(bf16_round(h.x), bf16_round(h.y));
+            }
         }
         __syncthreads();
-        for (int e = tid; e < kTile * kMlpH; e += NT) {
-            const int s = e / kMlpH, j = e - s * kMlpH;
-            float a = W[kPB2 + j];
-            for (int i = 0; i < kMlpH; ++i) a += W[kPW2 + j * kMlpH + i] * bf16_round(H1[s * kMlpH + i]);
-            H2[e] = tanhf(a);
+        {
+            float a[4][2];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) a[k][0] = a[k][1] = W[kPB2 + j0 + k];
+#pragma unroll 8
+            for (int i = 0; i < kMlpH; ++i) {
+                const float4 w = *reinterpret_cast<const float4*>(W2T + i * kMlpH + j0);
+                const float2 x = *reinterpret_cast<const float2*>(H1r + i * kRow + s0);
+                a[0][0] += w.x * x.x; a[0][1] += w.x * x.y;
+                a[1][0] += w.y * x.x; a[1][1] += w.y * x.y;
+                a[2][0] += w.z * x.x; a[2][1] += w.z * x.y;
+                a[3][0] += w.w * x.x; a[3][1] += w.w * x.y;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                *reinterpret_cast<float2*>(H2 + (j0 + k) * kRow + s0) = make_float2(tanhf(a[k][0]), tanhf(a[k][1]));
         }
         __syncthreads();
         for (int e = tid; e < kTile * kMlpOut; e += NT) {
-            const int s = e / kMlpOut, c = e - s * kMlpOut;
+            const int c = e / kTile, s = e - c * kTile;
             float d = 0.f;
             if (s < cnt) {
                 float a = W[kPB3 + c];
-                for (int i = 0; i < kMlpH; ++i) a += W[kPW3 + c * kMlpH + i] * H2[s * kMlpH + i];
+#pragma unroll 16
+                for (int i = 0; i < kMlpH; ++i) a += W[kPW3 + c * kMlpH + i] * H2[i * kRow + s];
                 const long long smp = idx ? idx[base + s] : base + s;
                 const float r = a - target[smp * kMlpOut + c] / W[kPSout + c];
                 lsum += r * r;
                 d = 2.f * r * inv_n;
             }
-            DO[e] = d;
+            DO[c * kRow + s] = d;
         }
         __syncthreads();
-        for (int e = tid; e < kTile * kMlpH; e += NT) {
-            const int s = e / kMlpH, i = e - s * kMlpH;
-            float a = 0.f;
+        {
+            float2 dout[kMlpOut];
 #pragma unroll
-            for (int c = 0; c < kMlpOut; ++c) a += DO[s * kMlpOut + c] * W[kPW3 + c * kMlpH + i];
-            const float h2 = H2[e];
-            D2[e] = a * (1.f - h2 * h2);
-        }
-        __syncthreads();
-        for (int e = tid; e < kTile * kMlpH; e += NT) {
-            const int s = e / kMlpH, i = e - s * kMlpH;
-            float a = 0.f;
-            for (int j = 0; j < kMlpH; ++j) a += D2[s * kMlpH + j] * W[kPW2 + j * kMlpH + i];
-            const float h1 = H1[e];
-            D1[e] = a * (1.f - h1 * h1);
-        }
-        __syncthreads();
-        // gradient entries, each owned by one thread
-        for (int q = tid; q < kMlpTrainable; q += NT) {
-            float a = 0.f;
-            if (q < kPB1) {
-                const int j = q / kMlpIn, i = q - j * kMlpIn;
-                for (int s = 0; s < kTile; ++s) a += D1[s * kMlpH + j] * X[s * 12 + i];
-            } else if (q < kPW2) {
-                const int j = q - kPB1;
-                for (int s = 0; s < kTile; ++s) a += D1[s * kMlpH + j];
-            } else if (q < kPB2) {
-                const int j = (q - kPW2) / kMlpH, i = (q - kPW2) - j * kMlpH;
-                for (int s = 0; s < kTile; ++s) a += D2[s * kMlpH + j] * bf16_round(H1[s * kMlpH + i]);
-            } else if (q < kPW3) {
-                const int j = q - kPB2;
-                for (int s = 0; s < kTile; ++s) a += D2[s * kMlpH + j];
-            } else if (q < kPB3) {
-                const int c = (q - kPW3) / kMlpH, i = (q - kPW3) - c * kMlpH;
-                for (int s = 0; s < kTile; ++s) a += DO[s * kMlpOut + c] * H2[s * kMlpH + i];
-            } else {
-                const int c = q - kPB3;
-                for (int s = 0; s < kTile; ++s) a += DO[s * kMlpOut + c];
+            for (int c = 0; c < kMlpOut; ++c) dout[c] = *reinterpret_cast<const float2*>(DO + c * kRow + s0);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                float ax = 0.f, ay = 0.f;
+#pragma unroll
+                for (int c = 0; c < kMlpOut; ++c) {
+                    const float w = W[kPW3 + c * kMlpH + j0 + k];
+                    ax += dout[c].x * w;
+                    ay += dout[c].y * w;
+                }
+                const float2 h = *reinterpret_cast<const float2*>(H2 + (j0 + k) * kRow + s0);
+                *reinterpret_cast<float2*>(D2 + (j0 + k) * kRow + s0) = make_float2(ax * (1.f - h.x * h.x), ay * (1.f - h.y * h.y));
             }
-            G[q] += a;
+        }
+        __syncthreads();
+        {
+            float a[4][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll 8
+            for (int j = 0; j < kMlpH; ++j) {
+                const float4 w = *reinterpret_cast<const float4*>(W + kPW2 + j * kMlpH + j0);
+                const float2 d = *reinterpret_cast<const float2*>(D2 + j * kRow + s0);
+                a[0][0] += d.x * w.x; a[0][1] += d.y * w.x;
+                a[1][0] += d.x * w.y; a[1][1] += d.y * w.y;
+                a[2][0] += d.x * w.z; a[2][1] += d.y * w.z;
+                a[3][0] += d.x * w.w; a[3][1] += d.y * w.w;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float2 h = *reinterpret_cast<const float2*>(H1 + (j0 + k) * kRow + s0);
+                *reinterpret_cast<float2*>(D1 + (j0 + k) * kRow + s0) =
+                    make_float2(a[k][0] * (1.f - h.x * h.x), a[k][1] * (1.f - h.y * h.y));
+            }
+        }
+        __syncthreads();
+        // gradient: dW2[j][i] = sum_s D2[j][s] H1r[i][s] in the register tile
+#pragma unroll 4
+        for (int s = 0; s < kTile; s += 4) {
+            float4 d[4], h[2];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) d[k] = *reinterpret_cast<const float4*>(D2 + (jq + 16 * k) * kRow + s);
+#pragma unroll
+            for (int m = 0; m < 2; ++m) h[m] = *reinterpret_cast<const float4*>(H1r + (ig + 32 * m) * kRow + s);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int m = 0; m < 2; ++m)
+                    g2[k][m] += (d[k].x * h[m].x + d[k].y * h[m].y) + (d[k].z * h[m].z + d[k].w * h[m].w);
+        }
+        // the other entries: W1, b1, b2, W3, b3 (a row of one array times a row of another, or
+        // alone)
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const int q = tid + t * kGradThreads;
+            if (q >= kGradSmall) break;
+            const float *ra = nullptr, *rb = nullptr;
+            int p = q;
+            if (p < kMlpH * kMlpIn) {
+                ra = D1 + (p / kMlpIn) * kRow;
+                rb = X + (p % kMlpIn) * kRow;
+            } else if ((p -= kMlpH * kMlpIn) < kMlpH) {
+                ra = D1 + p * kRow;
+            } else if ((p -= kMlpH) < kMlpH) {
+                ra = D2 + p * kRow;
+            } else if ((p -= kMlpH) < kMlpOut * kMlpH) {
+                ra = DO + (p / kMlpH) * kRow;
+                rb = H2 + (p % kMlpH) * kRow;
+            } else {
+                ra = DO + (p - kMlpOut * kMlpH) * kRow;
+            }
+            float a = 0.f;
+#pragma unroll 4
+            for (int s = 0; s < kTile; s += 4) {
+                const float4 u = *reinterpret_cast<const float4*>(ra + s);
+                const float4 v = rb ? *reinterpret_cast<const float4*>(rb + s) : make_float4(1.f, 1.f, 1.f, 1.f);
+                a += (u.x * v.x + u.y * v.y) + (u.z * v.z + u.w * v.w);
+            }
+            gs[t] += a;
         }
         __syncthreads();
     }
-    for (int q = tid; q < kMlpTrainable; q += NT) atomicAdd(&grad[q], G[q]);
+    // the block's gradient in the parameters' order (over the activations), then into grad
+    float* G = H1;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int m = 0; m < 2; ++m) G[kPW2 + (jq + 16 * k) * kMlpH + ig + 32 * m] = g2[k][m];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        const int q = tid + t * kGradThreads;
+        if (q < kGradSmall) G[q < kPW2 ? q : q + kMlpH * kMlpH] = gs[t];
+    }
+    __syncthreads();
+    if (vec) {
+        for (int q = 4 * tid; q + 4 <= kMlpTrainable; q += 4 * NT)
+            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(grad + q)), "f"(G[q]),
+                         "f"(G[q + 1]), "f"(G[q + 2]), "f"(G[q + 3])
+                         : "memory");
+        for (int q = (kMlpTrainable & ~3) + tid; q < kMlpTrainable; q += NT) atomicAdd(&grad[q], G[q]);
+    } else {
+        for (int q = tid; q < kMlpTrainable; q += NT) atomicAdd(&grad[q], G[q]);
+    }
     for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(kFull, lsum, o);
     if ((tid & 31) == 0) red[tid >> 5] = lsum;
     __syncthreads();
@@ -391,6 +496,14 @@ __global__ void __launch_bounds__(256) mlp_grad_kernel(const float* __restrict__
         for (int w = 0; w < NT / 32; ++w) t += red[w];
         atomicAdd(loss, t * inv_n);
     }
+}
+
+// grad and loss to zero in one launch.
+__global__ void mlp_zero_kernel(float* grad, float* loss)
+{
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < kMlpParams) grad[q] = 0.f;
+    if (q == 0) *loss = 0.f;
 }
 
 // Adam (Kingma & Ba) on the trainable parameters.
@@ -453,7 +566,7 @@ __global__ void __launch_bounds__(128) mlp_predict_kernel(const float* Pr, const
     }
 }
 
-constexpr size_t kGradSmem = sizeof(float) * (kMlpParams + kMlpTrainable + 4 + kTile * 12 + 4 * kTile * kMlpH + kTile * kMlpOut);
+constexpr size_t kGradSmem = sizeof(float) * (kMlpParams + kMlpH * kMlpH + kRow * (kMlpIn + 5 * kMlpH + kMlpOut));
 
 }  // namespace
 
@@ -503,16 +616,18 @@ int npfem_mlp_loss_grad(const float* params, const float* feat, const float* tar
     if (!params || !feat || !target || !grad || !loss || n < 1)
         return set_error(NPFEM_ERR_INVALID_ARG, "npfem_mlp_loss_grad: null pointer or n < 1");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t e = cudaMemsetAsync(grad, 0, sizeof(float) * kMlpParams, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(loss, 0, sizeof(float), s);
+    mlp_zero_kernel<<<(kMlpParams + 255) / 256, 256, 0, s>>>(grad, loss);
+    count_launch();
+    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradSmem);
     if (e != cudaSuccess) return set_error(NPFEM_ERR_CUDA, std::string("npfem_mlp_loss_grad: ") + cudaGetErrorString(e));
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int tiles = (n + kTile - 1) / kTile;
-    const int grid = std::max(1, std::min(tiles, 2 * sms));
-    mlp_grad_kernel<<<grid, 256, kGradSmem, s>>>(params, feat, target, idx, n, 1.f / n, grad, loss);
+    const int grid = std::max(1, std::min(tiles, sms));
+    mlp_grad_kernel<<<grid, kGradThreads, kGradSmem, s>>>(params, feat, target, idx, n, 1.f / n, grad, loss,
+                                                          (reinterpret_cast<uintptr_t>(grad) & 15) == 0);
     count_launch();
     e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(NPFEM_ERR_CUDA, std::string("npfem_mlp_loss_grad: ") + cudaGetErrorString(e));
