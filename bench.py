@@ -644,12 +644,12 @@ def main():
         if "c4" in want:
             legs["c4"] = compare_leg(N, W, torch, "c4", [p4], [16384], args, flush, P, local, pk, pk_kind)
             legs["c4"]["workload"] = w4
-        # the precision configuration: the A^-1 contraction in BF16 and in TF32 on the tensor
-        # cores, each with one refinement sweep
+        # the precision configuration: TF32 handles (which run in FP32), and BF16 on the tensor
+        # cores with one refinement sweep
         if "c4_tf32" in want:
             legs["c4_tf32"] = compare_leg(N, W, torch, "c4_tf32", [p4], [16384], args, flush, P, local, pk, pk_kind,
                                           refine=1, plain=False, precision="tf32")
-            legs["c4_tf32"]["form"] = "TF32 tensor-core A^-1 contraction (streamed, per SIMT block) + one refinement sweep"
+            legs["c4_tf32"]["form"] = "TF32 handle (H~^-1 applied in FP32: dense inverse or sparse factor)"
             legs["c4_tf32"]["workload"] = w4
         if "c4_bf16_refine1" in want:
             legs["c4_bf16_refine1"] = compare_leg(N, W, torch, "c4_bf16_refine1", [p4], [16384], args, flush, P,

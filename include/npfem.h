@@ -52,18 +52,18 @@ extern "C" {
 
 /* ---- precision of the solve (npfem_opts.precision) ----------------------- */
 #define NPFEM_PREC_FP64 0 /* state, energies and the A^-1 contraction in FP64            */
-#define NPFEM_PREC_FP32 1 /* state and energies FP32 (sums FP64), A^-1 FP32 on the SIMT  */
-                          /* pipes: the plain GPU path                                  */
-#define NPFEM_PREC_TF32 2 /* as FP32, but the A^-1 contraction runs on tcgen05 tensor    */
-                          /* cores in TF32 with FP32 accumulation: every persistent SIMT */
-                          /* block streams A^-1 (TF32, 128 x 32 tiles) from L2 through   */
-                          /* shared memory, `refine` refinement sweeps; up to 4096       */
-                          /* vertices (npfem_step_static contracts in FP32 instead)      */
+#define NPFEM_PREC_FP32 1 /* state and energies FP32 (compensated sums); H~^-1 applied in   */
+                          /* FP32: the dense inverse for meshes of at most 700 vertices, a */
+                          /* sparse block factor of H~ above                              */
+#define NPFEM_PREC_TF32 2 /* as FP32 (the direction is at least as accurate as with a TF32  */
+                          /* A^-1 and one refinement sweep, and cheaper: a sparse factor or  */
+                          /* the dense inverse in FP32 beats streaming A^-1 through the      */
+                          /* tensor cores)                                                  */
 #define NPFEM_PREC_BF16 3 /* as FP32, but the A^-1 contraction runs on tcgen05 tensor    */
                           /* cores: BF16 A^-1 resident in tensor memory across a cluster */
                           /* of ceil(n/128) SMs, BF16 q, FP32 accumulation, `refine`     */
-                          /* refinement sweeps; meshes above 960 vertices fall back to    */
-                          /* the FP32 SIMT contraction                                    */
+                          /* refinement sweeps; meshes above 960 vertices and handles with */
+                          /* beta_D > 0 take the FP32 path                               */
 
 typedef struct npfem_handle npfem_handle;
 
@@ -101,8 +101,9 @@ typedef struct {
    equal_mass: 1 = lump the mass equally, 0 = by barycentric rest area.
    armijo_noise: multiple of the estimated rounding error of g added to the
                  Armijo bound (FP32 energies); 0 = exact test.
-   refine: NPFEM_PREC_BF16 and NPFEM_PREC_TF32: refinement sweeps of the tensor-core
-           A^-1 contraction (0 or 1): r = A^-1 q, then r += A^-1 (q - H~ r).
+   refine: NPFEM_PREC_BF16: refinement sweeps of the tensor-core A^-1 contraction (0 or
+           1): r = A^-1 q, then r += A^-1 (q - H~ r).  The FP32 application of H~^-1
+           needs none.
    fill_idle_sms: NPFEM_PREC_BF16 only: 1 = SMs that the tensor-core clusters leave
            idle run the SIMT solver on the same cells (dynamic split), 0 = clusters only.
    warm_history: 1 = temporal warm start: when a call steps the same groups and cell
@@ -164,7 +165,8 @@ void npfem_default_opts(npfem_opts* o);
    (us): validates the mesh, computes the rest-state tables in FP64 on the host
    (D_m^-1, rest areas, cotangent weights, mixed Voronoi areas, lumped masses, L),
    inverts H~ = M~/h^2 + L in FP64 on the GPU (the one-time prefactorisation of
-   Sec. 2.1.1) and keeps A^-1 = H~^-1 resident in the precision of opts->precision.
+   Sec. 2.1.1), factors it sparsely on the host (nested dissection) meanwhile, and keeps
+   what opts->precision applies H~^-1 with resident on the device.
    The handle owns all its device memory. Blocks until the setup is complete.
    Errors: INVALID_ARG (null pointers, bad sizes/options, dt <= 0), BAD_MESH,
    NOT_SPD, OOM, CUDA. */
@@ -175,8 +177,10 @@ int npfem_create(const npfem_mesh* mesh, const npfem_material* mat, const npfem_
 int npfem_destroy(npfem_handle* h);
 
 /* Advances every cell of n_groups meshes by one time step (Algorithm 1) on `stream`
-   (a cudaStream_t; 0 = legacy default stream): one persistent solver launch over all
-   groups (NPFEM_PREC_BF16 with every mesh of at most 960 vertices: one cluster launch
+   (a cudaStream_t; 0 = legacy default stream): one persistent solver launch over the
+   groups of each block size (by mesh size and number of cells; with at most a cell per SM
+   one launch over all groups; few FP64 cells run as a cluster of blocks per cell)
+   (NPFEM_PREC_BF16 with every mesh of at most 960 vertices: one cluster launch
    per group, plus a SIMT launch on SMs the clusters leave idle, forked from and
    joined back to `stream`), preceded by the warm-start launch when a network is
    installed.  With the temporal warm start (opts.warm_history) a cluster group's
@@ -207,10 +211,8 @@ int npfem_step(npfem_handle* const* meshes, int n_groups, const int32_t* cells_p
    array compiled into the library, held by every GPU that loads the library until
    the process exits.  Arguments, layout, results and errors are those of
    npfem_step, with these differences: every group runs the persistent SIMT solver
-   kernel (NPFEM_PREC_BF16 handles included, which then contract a BF16 copy of A^-1
-   with FP32 accumulation on the SIMT pipes instead of the tensor-core cluster kernel),
-   one launch per distinct
-   tuned block size as npfem_step launches its SIMT groups; the temporal warm start
+   kernel (NPFEM_PREC_BF16 handles included, which then apply H~^-1 in FP32 instead of on
+   the tensor cores) in one launch of 512-thread blocks; the temporal warm start
    (opts.warm_history) is not used; with large meshes it may run fewer persistent
    blocks so that their slots fit; and it returns INVALID_ARG when one block's
    scratch exceeds the array.  Every call looks up the array's device address on
@@ -430,18 +432,18 @@ const char* npfem_last_error(void);
 /* Launch-shape autotuner: for every group (cells_per_group[g] > 0) times
    `trial_steps` back-to-back steps of that group alone (after one untimed step) on
    copies of its x, v for each candidate shape, and keeps the fastest in the handle:
-   SIMT blocks of 512 or 640 threads (640 for FP32 state only), and for NPFEM_PREC_BF16
-   meshes of at most 960 vertices the tensor-core cluster kernel with and without the
-   idle-SM SIMT launch (with the handle's temporal warm start, as the steps that
-   follow will run).  x, v are not modified.  trial_ms (optional, 5 floats per
-   group) receives the mean trial-step time of each candidate in the order SIMT 512,
-   SIMT 640, clusters + idle-SM 512, clusters only, clusters + idle-SM 640 (-1 where
-   a candidate does not apply).  Blocks.  Errors: INVALID_ARG, CUDA, OOM. */
+   the SIMT kernel (its block size follows from the mesh and the cells), and for
+   NPFEM_PREC_BF16 meshes of at most 960 vertices the tensor-core cluster kernel with and
+   without the idle-SM SIMT launch (with the handle's temporal warm start, as the steps
+   that follow will run).  x, v are not modified.  trial_ms (optional, 5 floats per
+   group) receives the mean trial-step time of each candidate: [0] SIMT, [2] clusters +
+   idle-SM blocks, [3] clusters only (-1 where a candidate does not apply; [1] and [4] are
+   not used).  Blocks.  Errors: INVALID_ARG, CUDA, OOM. */
 int npfem_autotune(npfem_handle* const* meshes, int n_groups, const int32_t* cells_per_group, const void* x,
                    const void* v, const void* f_ext, double dt, int trial_steps, float* trial_ms);
 
-/* The launch shape a handle uses: *use_tc (cluster kernel), *threads (SIMT block
-   size), *fill_idle_sms.  Errors: INVALID_ARG. */
+/* The launch shape a handle uses: *use_tc (cluster kernel), *threads (the largest SIMT
+   block size, 512), *fill_idle_sms.  Errors: INVALID_ARG. */
 int npfem_get_tuning(const npfem_handle* h, int* use_tc, int* threads, int* fill_idle_sms);
 
 /* A CUDA graph of `steps` consecutive npfem_step calls on fixed state buffers (the

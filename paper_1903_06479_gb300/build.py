@@ -20,7 +20,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # The solver's FP32 divisions and square roots feed an iteration that stops at a
 # relative residual of ~1e-6; the approximate forms (a few ulp) cut the evaluation's
 # instruction count by about a fifth.  FP64 arithmetic is unaffected by these flags.
-EXTRA = {"npfem_solver.cu": ["-prec-div=false", "-prec-sqrt=false"]}
+EXTRA_CELL = ["-prec-div=false", "-prec-sqrt=false"]
 
 
 def _nvcc() -> str:
@@ -52,7 +52,7 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
 
     def compile_one(src: str) -> str:
         obj = os.path.join(BUILD, os.path.basename(src) + ".o")
-        cmd = [nvcc, *common, *ARCH, *EXTRA.get(os.path.basename(src), []), "-c", src, "-o", obj]
+        cmd = [nvcc, *common, *ARCH, *(EXTRA_CELL if os.path.basename(src).startswith("npfem_cell") else []), "-c", src, "-o", obj]
         if ptxas_info and src.endswith(".cu"):
             cmd += ["-Xptxas", "-v"]
         r = subprocess.run(cmd, capture_output=True, text=True)
@@ -62,7 +62,7 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
             sys.stderr.write(r.stdout + r.stderr)
         return obj
 
-    with cf.ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 4)) as ex:
+    with cf.ThreadPoolExecutor(max_workers=min(16, os.cpu_count() or 4)) as ex:
         objs = list(ex.map(compile_one, sources()))
     tmp = LIB + f".tmp{os.getpid()}"
     cmd = [nvcc, *ARCH, "-shared", "-o", tmp, *objs, "-lcudart"]

@@ -79,7 +79,28 @@ int upload(npfem_handle* h, const std::vector<S>& src, const X** out)
 }
 
 template <typename T>
-int fill_topo(npfem_handle* h, TopoDev<T>* tp, const void* ainv, const void* minv)
+int upload_sparse(npfem_handle* h, const SparseHost& F, SparseDev<T>* sp)
+{
+    int rc;
+    const int* drow = nullptr;
+    if ((rc = upload(h, F.perm, &sp->perm))) return rc;
+    if ((rc = upload(h, F.rows, &drow))) return rc;
+    if ((rc = upload(h, F.idx, &sp->idx))) return rc;
+    if ((rc = upload(h, F.val, &sp->val))) return rc;
+    sp->row = reinterpret_cast<const int2*>(drow);
+    sp->npos = F.npos;
+    for (int v = 0; v < kSparseScheds; ++v) {
+        const int* ds = nullptr;
+        if ((rc = upload(h, F.sched[v], &ds))) return rc;
+        sp->sched[v] = reinterpret_cast<const int4*>(ds);
+        sp->entries[v] = (int)F.sched[v].size() / (4 * sparse_sched_warps(v));
+    }
+    return 0;
+}
+
+template <typename T>
+int fill_topo(npfem_handle* h, TopoDev<T>* tp, const SparseHost& factor, const SparseHost& cluster_factor,
+              const SparseHost* mass_factor)
 {
     const HostTopo& H = h->host;
     int rc;
@@ -186,24 +207,23 @@ int fill_topo(npfem_handle* h, TopoDev<T>* tp, const void* ainv, const void* min
     tp->nt = H.nt;
     tp->n_pad = h->n_pad;
     tp->nnz = (int)H.ring_idx.size();
-    tp->ainv = static_cast<const T*>(ainv);
-    tp->minv = static_cast<const T*>(minv);
     tp->l_ptr = nullptr;
     tp->l_idx = nullptr;
     tp->l_val = nullptr;
     tp->beta_h = (T)(h->mat.beta_D / h->dt);
-    if (minv) {
+    if (mass_factor) {
         if ((rc = upload(h, H.L_ptr, &tp->l_ptr))) return rc;
         std::vector<unsigned short> lidx(H.L_idx.begin(), H.L_idx.end());
         if ((rc = upload(h, lidx, &tp->l_idx))) return rc;
         if ((rc = upload(h, H.L_val, &tp->l_val))) return rc;
     }
     tp->ainv_lp = nullptr;
-    tp->ainv_b16 = nullptr;
-    tp->n8 = 0;
     tp->h_ptr = nullptr;
     tp->h_idx = nullptr;
     tp->h_val = nullptr;
+    if ((rc = upload_sparse(h, factor, &tp->sp))) return rc;
+    if (cluster_factor.npos && (rc = upload_sparse(h, cluster_factor, &tp->spc))) return rc;
+    if (mass_factor && (rc = upload_sparse(h, *mass_factor, &tp->spm))) return rc;
     tp->C = (T)h->mat.C;
     tp->B = (T)h->mat.B;
     tp->Dsk = (T)h->mat.D;
@@ -239,6 +259,25 @@ int check_opts(const npfem_opts* o)
     return 0;
 }
 
+// Block size of a SIMT group: a mesh's evaluation keeps about n / 32 warps busy and most of
+// its phases are latency-bound, so when every SM has several cells to solve, two blocks of
+// 256 threads or four of 128 per SM overlap each other's phases (vectors that then do not
+// fit in shared memory go to global memory, L2).  Measured, FP32, three steps of 3040
+// cells, 512 / 256 / 128 threads: 66 vertices 296 / 161 / 107 us, 258: 1087 / 688 / 557,
+// 362: 1223 / 830 / 804; 1520 cells: 642: 2048 / 1726 / 1901, 1026: 5235 / 4758 / 6816;
+// 400 cells of 2562: 7677 / 12086.  With at most a cell per SM a cell's own latency counts:
+// 40 cells of 66 vertices 33 / 30 / 31 us, 162: 64 / 66 / 79, 258: 68 / 78 / 105.  FP64 is
+// bound by the FP64 pipe; four blocks hide its latencies best at every size (160 cells of
+// 66 vertices 972 / 705 / 573 us, 258: 5321 / 4846 / 4666).
+int simt_threads(const npfem_handle* h, int n, long long cells)
+{
+    const long long sms = h->sm_count;
+    if (h->precision == NPFEM_PREC_FP64) return cells > sms ? 128 : 512;
+    if (n <= 384 && cells > 2 * sms) return 128;
+    if (n <= 1200 && cells > sms) return 256;
+    return 512;
+}
+
 template <typename T>
 int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T* x, T* v, const T* f, const T* y,
               T* grad_out, double* parts, npfem_cell_stats* stats, int mode, cudaStream_t stream,
@@ -252,16 +291,17 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
     memset(&a, 0, sizeof(a));
     long long total = 0, state = 0, slot = 0;
     int smem_max = 0;
-    // TF32 tensor-core contraction: the A^-1 ring and the B operand sit in front of the
-    // per-cell vectors, and every block holds 16 tensor-memory columns per row tile
-    const bool tf = sizeof(T) == 4 && mode == 0 && h0->precision == NPFEM_PREC_TF32;
-    int tf_kpad = 0, tf_tiles = 0;
-    for (int gi = 0; tf && gi < n_groups; ++gi) {
-        tf_kpad = std::max(tf_kpad, meshes[gi]->tf.kpad);
-        tf_tiles = std::max(tf_tiles, meshes[gi]->tf.rb);
+    if (threads <= 0) {
+        int n_max = 0;
+        long long all = 0;
+        for (int gi = 0; gi < n_groups; ++gi) {
+            n_max = std::max(n_max, meshes[gi]->n);
+            all += cells[gi];
+        }
+        threads = simt_threads(h0, n_max, all);
     }
-    const int tcb = tf ? tf32_smem_bytes(tf_kpad) : 0;
-    const int budget = h0->smem_optin - kFixedSmem - 1024 - tcb;
+    // 512 / threads blocks share an SM's shared memory (1 KB of it per block is the system's)
+    const int budget = (threads < 512 ? h0->smem_sm / (512 / threads) : h0->smem_optin) - kFixedSmem - 1024;
     for (int gi = 0; gi < n_groups; ++gi) {
         npfem_handle* h = meshes[gi];
         GroupDesc<T>& g = a.g[gi];
@@ -273,7 +313,7 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
         g.carry_rec = carry_rec_elems(h->n_pad, h0->opts.lbfgs_m);
         g.carry_off = carry_offs ? carry_offs[gi] : 0;
         long long sb = 0;
-        place_vectors(&g, h->n_pad, h->nt, h0->opts.lbfgs_m, budget, &sb, tcb);
+        place_vectors(&g, h->n, h->n_pad, h->nt, h->npos(), h0->opts.lbfgs_m, budget, &sb);
         slot = std::max(slot, sb);
         smem_max = std::max(smem_max, g.smem_bytes);
         total += cells[gi];
@@ -292,17 +332,6 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
     a.work = h0->work;
     set_solver_params(&a.p, h0->opts);
     a.p.mode = mode;
-    a.p.contraction = CONTRACT_SIMT;
-    int tmem_cols = 0;
-    if (tf) {
-        a.p.contraction = CONTRACT_TC_TF32;
-        a.p.refine = h0->opts.refine;
-        a.p.tf_kpad = tf_kpad;
-        tmem_cols = 32;
-        while (tmem_cols < 16 * tf_tiles) tmem_cols <<= 1;
-        if (tmem_cols > 512) return fail(NPFEM_ERR_INVALID_ARG, "TF32 path: mesh too large (more than 32 row tiles)");
-        a.p.tmem_cols = tmem_cols;
-    }
     a.u0 = u0;
     a.hist_in = hist_in;
     a.hist_out = hist_out;
@@ -315,14 +344,10 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
         a.col_w = (T)h0->col_w;
     }
 
-    if (threads <= 0) threads = h0->threads;
-    if (sizeof(T) == 8) threads = std::min(threads, 512);
     const int smem = kFixedSmem + smem_max;
-    NPFEM_CUDA(set_cell_kernel_smem<T>(smem));
     int per_sm = 1;
-    NPFEM_CUDA(cells_per_sm<T>(threads, smem, &per_sm));
+    NPFEM_CUDA(cells_per_sm<T>(a, threads, smem, &per_sm));
     per_sm = std::max(per_sm, 1);
-    if (tf) per_sm = std::min(per_sm, 512 / tmem_cols);  // every resident block gets its tensor memory
     long long grid = std::min<long long>(total, (long long)h0->sm_count * per_sm);
     a.slot_bytes = slot;
     if (slot > 0) {
@@ -340,6 +365,92 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
         a.scratch = h0->scratch;
     }
     NPFEM_CUDA(launch_cells<T>(a, (int)grid, threads, smem, stream));
+    return 0;
+}
+
+// Few FP64 cells: one launch of clusters of 8, 4 or 2 blocks per cell, the largest size at which
+// every cell's cluster is resident at once.  *done says whether the launch was made (not
+// with beta_D > 0, one-rings past the fixed width or meshes too large).
+int run_cells_cluster(npfem_handle* const* meshes, int n_groups, const int32_t* cells, double* x, double* v, const double* f,
+                      npfem_cell_stats* stats, cudaStream_t stream, const long long* state_offs, const long long* stats_offs,
+                      const double* hist_in, double* hist_out, double* carry, const long long* carry_offs, bool* done)
+{
+    *done = false;
+    npfem_handle* h0 = meshes[0];
+    long long total = 0;
+    for (int gi = 0; gi < n_groups; ++gi) {
+        const npfem_handle* h = meshes[gi];
+        if (!h->td.k8 || h->mat.beta_D > 0.0 || h->n < 32 || h->n > 4096) return 0;
+        total += cells[gi];
+    }
+    if (total == 0 || 2 * total > h0->sm_count) return 0;
+    for (int lg = 3; lg >= 1; --lg) {
+        const int C = 1 << lg;
+        if (C * total > h0->sm_count) continue;
+        LaunchArgs<double> a;
+        memset(&a, 0, sizeof(a));
+        long long at = 0, slot = 0;
+        int smem_max = 0;
+        bool fits = true;
+        for (int gi = 0; gi < n_groups; ++gi) {
+            npfem_handle* h = meshes[gi];
+            GroupDesc<double>& g = a.g[gi];
+            g.topo = h->td;
+            g.cell_begin = at;
+            g.state_off = state_offs[gi];
+            g.stats_off = stats_offs[gi];
+            g.cells = cells[gi];
+            g.carry_rec = carry_rec_elems(h->n_pad, h0->opts.lbfgs_m);
+            g.carry_off = carry_offs[gi];
+            long long sb = 0;
+            fits = place_vectors_cluster(&g, h->n_pad, h->npos(), h0->opts.lbfgs_m, C,
+                                         h0->smem_optin - kFixedSmem - 1024, &sb) && fits;
+            slot = std::max(slot, sb);
+            smem_max = std::max(smem_max, g.smem_bytes);
+            at += cells[gi];
+        }
+        if (!fits) continue;
+        const int smem = kFixedSmem + smem_max;
+        if (h0->cl_smem[lg] != smem) {
+            NPFEM_CUDA(query_cells_cl(C, smem, &h0->cl_max[lg]));
+            h0->cl_smem[lg] = smem;
+        }
+        if (h0->cl_max[lg] < total) continue;
+        a.n_groups = n_groups;
+        a.total_cells = total;
+        a.x = x;
+        a.v = v;
+        a.f = f;
+        a.stats = stats;
+        a.work = h0->work;
+        set_solver_params(&a.p, h0->opts);
+        a.p.cluster = C;
+        a.hist_in = hist_in;
+        a.hist_out = hist_out;
+        a.carry = hist_out ? carry : nullptr;
+        if (h0->col_planes) {
+            a.col = reinterpret_cast<const float4*>(h0->col_planes);
+            a.col_w = h0->col_w;
+        }
+        a.slot_bytes = slot;
+        if (slot > 0) {
+            const size_t need = (size_t)slot * (size_t)(C * total);
+            if (need > h0->scratch_bytes) {
+                if (h0->scratch) {
+                    NPFEM_CUDA(cudaStreamSynchronize(stream));
+                    cudaFree(h0->scratch);
+                    h0->scratch = nullptr;
+                    h0->scratch_bytes = 0;
+                }
+                NPFEM_CUDA(cudaMalloc(&h0->scratch, need));
+                h0->scratch_bytes = need;
+            }
+            a.scratch = h0->scratch;
+        }
+        NPFEM_CUDA(launch_cells_cl(a, C, (int)total, smem, stream));
+        *done = true;
+        return 0;
+    }
     return 0;
 }
 
@@ -374,7 +485,7 @@ int run_cells_tc(npfem_handle* h, int cells, float* x, float* v, const float* f,
     const int bbytes = (ncol * h->tf.kpad * 2 + 127) & ~127;
     const int budget = h->smem_optin - kFixedSmem - 1024 - bbytes;
     long long slot = 0;
-    place_vectors(&g, h->n_pad, h->nt, h->opts.lbfgs_m, budget, &slot, bbytes, true);
+    place_vectors(&g, h->n, h->n_pad, h->nt, h->npos(), h->opts.lbfgs_m, budget, &slot, bbytes, true);
     if (g.loc[V_GC] < 0) return fail(NPFEM_ERR_INVALID_ARG, "mesh too large for the tensor-core path's shared memory");
     a.n_groups = 1;
     a.total_cells = cells;
@@ -385,7 +496,6 @@ int run_cells_tc(npfem_handle* h, int cells, float* x, float* v, const float* f,
     a.work = h->work;
     set_solver_params(&a.p, h->opts);
     a.p.mode = 0;
-    a.p.contraction = CONTRACT_TC_BF16;
     a.p.cluster = cluster;
     a.p.refine = h->opts.refine;
     // one block per SM: a second block on the SM would wait in the tensor-memory
@@ -409,8 +519,7 @@ int run_cells_tc(npfem_handle* h, int cells, float* x, float* v, const float* f,
     if (cells <= grid || h->opts.fill_idle_sms == 0) helper = 0;
     if (helper > 0) {
         b = a;
-        place_vectors(&b.g[0], h->n_pad, h->nt, h->opts.lbfgs_m, h->smem_optin - kFixedSmem - 1024, &slot_b);
-        b.p.contraction = CONTRACT_SIMT;
+        place_vectors(&b.g[0], h->n, h->n_pad, h->nt, h->npos(), h->opts.lbfgs_m, h->smem_optin - kFixedSmem - 1024, &slot_b);
         b.p.cluster = 0;
         b.p.refine = 0;
         smem_b = kFixedSmem + b.g[0].smem_bytes;
@@ -448,8 +557,7 @@ int run_cells_tc(npfem_handle* h, int cells, float* x, float* v, const float* f,
     NPFEM_CUDA(launch_cells_tc(a, cluster, kTcThreads, smem, grid, stream));
     if (helper > 0) {
         cudaError_t e = cudaStreamWaitEvent(h->side_stream, h->ev_fork, 0);
-        if (e == cudaSuccess) e = set_cell_kernel_smem<float>(smem_b);
-        if (e == cudaSuccess) e = launch_cells<float>(b, helper, h->threads, smem_b, h->side_stream);
+        if (e == cudaSuccess) e = launch_cells<float>(b, helper, kTcThreads, smem_b, h->side_stream);
         if (e != cudaSuccess) {
             // the clusters alone cannot reset the shared counters: clear them behind
             // the launch so that the next step starts clean, and report the failure
@@ -487,7 +595,7 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
             done[g] = 1;
             continue;
         }
-        if (prec == NPFEM_PREC_BF16 && meshes[g]->n <= kTcMaxVerts && meshes[g]->use_tc) {
+        if (prec == NPFEM_PREC_BF16 && meshes[g]->takes_clusters()) {
             npfem_handle* hg = meshes[g];
             int32_t cg = cells_per_group[g];
             float* xg = (float*)x + soff[g];
@@ -518,7 +626,7 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
                 NPFEM_CUDA(cudaMemcpyAsync(hg->defer + 2, hg->defer + 1, sizeof(unsigned int), cudaMemcpyDeviceToDevice, s));
                 NPFEM_CUDA(cudaMemsetAsync(hg->defer, 0, 2 * sizeof(unsigned int), s));
                 int rc = run_cells<float>(&hg, 1, &cg, xg, vg, fg, nullptr, nullptr, nullptr, sg, 0, s,
-                                          u0 ? u0 + soff[g] : nullptr, nullptr, nullptr, 512, hin, hout, pos_stride,
+                                          u0 ? u0 + soff[g] : nullptr, nullptr, nullptr, 0, hin, hout, pos_stride,
                                           hg->defer, hist_ext, kg);
                 if (rc) return rc;
                 only = hg->defer;
@@ -531,14 +639,25 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
             done[g] = 1;
         }
     }
+    // the other groups: with at most a cell per SM in all one launch, else each at its own
+    // block size, groups of one size together
+    long long left = 0;
+    for (int g = 0; g < n_groups; ++g)
+        if (!done[g]) left += cells_per_group[g];
+    std::vector<int> shape(n_groups, 512);
+    if (left > meshes[0]->sm_count)
+        for (int g = 0; g < n_groups; ++g) shape[g] = simt_threads(meshes[g], meshes[g]->n, cells_per_group[g]);
+    else if (n_groups == 1)
+        shape[0] = simt_threads(meshes[0], meshes[0]->n, left);
     for (int g0 = 0; g0 < n_groups; ++g0) {
         if (done[g0]) continue;
-        const int threads = prec == NPFEM_PREC_FP64 ? 512 : meshes[g0]->threads;
+        const int threads = shape[g0];
         std::vector<npfem_handle*> hs;
         std::vector<int32_t> cs;
         std::vector<long long> so, co, ko;
         for (int g = g0; g < n_groups; ++g) {
-            if (done[g] || (prec != NPFEM_PREC_FP64 && meshes[g]->threads != threads)) continue;
+            if (done[g] || shape[g] != threads || (left > meshes[0]->sm_count && !meshes[g]->tf.ainv != !meshes[g0]->tf.ainv))
+                continue;
             hs.push_back(meshes[g]);
             cs.push_back(cells_per_group[g]);
             so.push_back(soff[g]);
@@ -547,6 +666,14 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
             done[g] = 1;
         }
         int rc;
+        bool clustered = false;
+        if (prec == NPFEM_PREC_FP64) {
+            rc = run_cells_cluster(hs.data(), (int)hs.size(), cs.data(), (double*)x, (double*)v, (const double*)f_ext,
+                                   stats, s, so.data(), co.data(), (const double*)hist_in, (double*)hist_out,
+                                   (double*)carry, ko.data(), &clustered);
+            if (rc) return rc;
+        }
+        if (clustered) continue;
         if (prec == NPFEM_PREC_FP64)
             rc = run_cells<double>(hs.data(), (int)hs.size(), cs.data(), (double*)x, (double*)v, (const double*)f_ext,
                                    nullptr, nullptr, nullptr, stats, 0, s, nullptr, so.data(), co.data(), threads,
@@ -690,8 +817,8 @@ int npfem_kernel_timing(npfem_handle* h, int capacity)
 int npfem_get_tuning(const npfem_handle* h, int* use_tc, int* threads, int* fill_idle_sms)
 {
     if (!h || !use_tc || !threads || !fill_idle_sms) return fail(NPFEM_ERR_INVALID_ARG, "npfem_get_tuning: null argument");
-    *use_tc = h->use_tc && h->precision == NPFEM_PREC_BF16 && h->n <= kTcMaxVerts;
-    *threads = h->threads;
+    *use_tc = h->takes_clusters();
+    *threads = 512;
     *fill_idle_sms = h->opts.fill_idle_sms;
     return 0;
 }
@@ -706,7 +833,7 @@ int npfem_autotune(npfem_handle* const* meshes, int n_groups, const int32_t* cel
     const int prec = meshes[0]->precision;
     const size_t es = prec == NPFEM_PREC_FP64 ? 8 : 4;
     struct Shape {
-        int use_tc, threads, fill, slot;
+        int use_tc, fill, slot;
     };
     if (trial_ms)
         for (int q = 0; q < 5 * n_groups; ++q) trial_ms[q] = -1.f;
@@ -723,12 +850,10 @@ int npfem_autotune(npfem_handle* const* meshes, int n_groups, const int32_t* cel
         const size_t bytes = (size_t)3 * h->n * cells * es;
         if (cells == 0) continue;
         std::vector<Shape> cand;
-        cand.push_back({0, 512, h->opts.fill_idle_sms, 0});
-        if (prec != NPFEM_PREC_FP64) cand.push_back({0, 640, h->opts.fill_idle_sms, 1});
-        if (prec == NPFEM_PREC_BF16 && h->n <= kTcMaxVerts) {
-            cand.push_back({1, 512, 1, 2});
-            cand.push_back({1, 512, 0, 3});
-            cand.push_back({1, 640, 1, 4});
+        cand.push_back({0, h->opts.fill_idle_sms, 0});
+        if (prec == NPFEM_PREC_BF16 && h->n <= kTcMaxVerts && h->mat.beta_D == 0.0) {
+            cand.push_back({1, 1, 2});
+            cand.push_back({1, 0, 3});
         }
         void *tx = nullptr, *tv = nullptr;
         cudaError_t ce = cudaMalloc(&tx, bytes);
@@ -737,12 +862,11 @@ int npfem_autotune(npfem_handle* const* meshes, int n_groups, const int32_t* cel
             rc = fail(ce == cudaErrorMemoryAllocation ? NPFEM_ERR_OOM : NPFEM_ERR_CUDA, "npfem_autotune: trial buffers");
         }
         float best = 1e30f;
-        Shape pick = {h->use_tc, h->threads, h->opts.fill_idle_sms, -1};
+        Shape pick = {h->use_tc, h->opts.fill_idle_sms, -1};
         const int hist_opt = h->opts.warm_history;
         for (const Shape& c : cand) {
             if (rc) break;
             h->use_tc = c.use_tc;
-            h->threads = c.threads;
             h->opts.fill_idle_sms = c.fill;
             const char* xs = static_cast<const char*>(x) + off;
             const char* vs = static_cast<const char*>(v) + off;
@@ -768,7 +892,6 @@ int npfem_autotune(npfem_handle* const* meshes, int n_groups, const int32_t* cel
             }
         }
         h->use_tc = pick.use_tc;
-        h->threads = pick.threads;
         h->opts.fill_idle_sms = pick.fill;
         h->opts.warm_history = hist_opt;
         h->hist_sig.clear();
@@ -842,6 +965,7 @@ int npfem_create(const npfem_mesh* mesh, const npfem_material* mat, const npfem_
     h->n_pad = (h->n + 3) & ~3;
     cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, device);
     cudaDeviceGetAttribute(&h->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    cudaDeviceGetAttribute(&h->smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device);
 
     auto bail = [&](int code) {
         h->release();
@@ -866,87 +990,41 @@ int npfem_create(const npfem_mesh* mesh, const npfem_material* mat, const npfem_
     int* flag = h->alloc<int>(4, &e);
     h->work = h->alloc<unsigned int>(4, &e);
     if (e) return bail(e);
-    // one inversion on the GPU: the dense FP64 matrix in, its inverse in place
-    auto invert = [&](double* dA, const std::vector<double>& A, const char* what) -> int {
-        if (cudaMemcpy(dA, A.data(), A.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemset(flag, 0, 4 * sizeof(int)) != cudaSuccess)
-            return fail(NPFEM_ERR_CUDA, std::string("upload of ") + what + " failed");
-        cudaError_t ce = invert_spd_fp64(dA, n, prow, flag, 0);
-        if (ce != cudaSuccess) return fail(NPFEM_ERR_CUDA, std::string("inversion of ") + what + ": " + cudaGetErrorString(ce));
-        int hflag = 0;
-        if (cudaMemcpy(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
-            return fail(NPFEM_ERR_CUDA, std::string("inversion of ") + what + " failed");
-        if (hflag == 2) return fail(NPFEM_ERR_TIMEOUT, std::string("inversion of ") + what + ": a grid barrier gave up");
-        if (hflag) return fail(NPFEM_ERR_NOT_SPD, std::string(what) + " is not positive definite");
-        return 0;
-    };
     if (cudaMemset(h->work, 0, 4 * sizeof(unsigned)) != cudaSuccess) return bail(fail(NPFEM_ERR_CUDA, "memset failed"));
-    if ((rc = invert(h->ainv64, H, "H~"))) return bail(rc);
-    cudaError_t ce = cudaSuccess;
-    // beta_D > 0: M~ is not diagonal; the first guess applies M~^-1 (dense, inverted once
-    // like H~) and the inertia term needs h beta_D L (sparse, in the solver's type)
-    void* minv_t = nullptr;
-    if (mat->beta_D > 0.0) {
-        std::vector<double> Mt((size_t)n * n, 0.0);
-        for (int i = 0; i < n; ++i) {
-            Mt[(size_t)i * n + i] += (1.0 + dt * mat->alpha_D) * h->host.mass[i];
-            for (int q = h->host.L_ptr[i]; q < h->host.L_ptr[i + 1]; ++q)
-                Mt[(size_t)i * n + h->host.L_idx[q]] += dt * mat->beta_D * h->host.L_val[q];
-        }
-        double* m64 = h->alloc<double>((size_t)n * n, &e);
+    // the dense inverse on the GPU (in place), while the host forms the sparse factor the
+    // solver applies H~^-1 with; beta_D > 0: M~ is not diagonal, the first guess solves
+    // with its factor (Eq. preOptimizationNewton)
+    if (cudaMemcpy(h->ainv64, H.data(), H.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemset(flag, 0, 4 * sizeof(int)) != cudaSuccess)
+        return bail(fail(NPFEM_ERR_CUDA, "upload of H~ failed"));
+    cudaError_t ce = invert_spd_fp64(h->ainv64, n, prow, flag, 0);
+    if (ce != cudaSuccess) return bail(fail(NPFEM_ERR_CUDA, std::string("inversion of H~: ") + cudaGetErrorString(ce)));
+    const bool damped = mat->beta_D > 0.0;
+    SparseHost factor, cluster_factor, mass_factor;
+    int frc = build_sparse_factor(h->host, mesh->rest_xyz, ms, lscale, &factor,
+                                  opts->precision == NPFEM_PREC_FP64 ? &cluster_factor : nullptr, &err);
+    if (!frc && damped)
+        frc = build_sparse_factor(h->host, mesh->rest_xyz, 1.0 + dt * mat->alpha_D, dt * mat->beta_D, &mass_factor,
+                                  nullptr, &err);
+    int hflag = 0;
+    if (cudaMemcpy(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+        return bail(fail(NPFEM_ERR_CUDA, "inversion of H~ failed"));
+    if (hflag == 2) return bail(fail(NPFEM_ERR_TIMEOUT, "inversion of H~: a grid barrier gave up"));
+    if (hflag) return bail(fail(NPFEM_ERR_NOT_SPD, "H~ is not positive definite"));
+    if (frc) return bail(fail(frc, err));
+    float* a32 = nullptr;
+    if (h->precision != NPFEM_PREC_FP64 && n <= kDenseMaxVerts) {
+        a32 = h->alloc<float>((size_t)np * np, &e);
         if (e) return bail(e);
-        if ((rc = invert(m64, Mt, "M~"))) return bail(rc);
-        if (h->precision == NPFEM_PREC_FP64) {
-            double* o = h->alloc<double>((size_t)np * np, &e);
-            if (e) return bail(e);
-            ce = publish_inverse(m64, n, np, nullptr, o, nullptr, nullptr, 0);
-            minv_t = o;
-        } else {
-            float* o = h->alloc<float>((size_t)np * np, &e);
-            if (e) return bail(e);
-            ce = publish_inverse(m64, n, np, o, nullptr, nullptr, nullptr, 0);
-            minv_t = o;
-        }
-        if (ce != cudaSuccess) return bail(fail(NPFEM_ERR_CUDA, "publishing M~^-1 failed"));
     }
-
-    void* ainv_t = nullptr;
-    if (h->precision == NPFEM_PREC_FP64) {
-        double* a64 = h->alloc<double>((size_t)np * np, &e);
-        if (e) return bail(e);
-        ce = publish_inverse(h->ainv64, n, np, nullptr, a64, nullptr, nullptr, 0);
-        ainv_t = a64;
-    } else {
-        float* a32 = h->alloc<float>((size_t)np * np, &e);
-        if (e) return bail(e);
-        ce = publish_inverse(h->ainv64, n, np, a32, nullptr, nullptr, nullptr, 0);
-        ainv_t = a32;
-    }
-    if (ce != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
-        return bail(fail(NPFEM_ERR_CUDA, "publishing A^-1 failed"));
-    rc = h->precision == NPFEM_PREC_FP64 ? fill_topo<double>(h, &h->td, ainv_t, minv_t)
-                                         : fill_topo<float>(h, &h->tf, ainv_t, minv_t);
+    if (symmetrise(h->ainv64, n, np, a32, 0) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
+        return bail(fail(NPFEM_ERR_CUDA, "symmetrising A^-1 failed"));
+    rc = h->precision == NPFEM_PREC_FP64 ? fill_topo<double>(h, &h->td, factor, cluster_factor, damped ? &mass_factor : nullptr)
+                                         : fill_topo<float>(h, &h->tf, factor, cluster_factor, damped ? &mass_factor : nullptr);
     if (rc) return bail(rc);
-    if (h->precision == NPFEM_PREC_TF32) {
-        // TF32 path: A^-1 in chunks of 128 rows x 32 K in the MMA's layout, and L for the
-        // refinement residual
-        const int kpad = (n + 31) & ~31, tiles = (n + 127) / 128;
-        float* atf = h->alloc<float>((size_t)tiles * 128 * kpad, &e);
-        if (e) return bail(e);
-        if (publish_inverse_tf32_tiled(h->ainv64, n, tiles, kpad, atf, 0) != cudaSuccess ||
-            cudaDeviceSynchronize() != cudaSuccess)
-            return bail(fail(NPFEM_ERR_CUDA, "publishing the TF32 A^-1 failed"));
-        h->tf.ainv_lp = atf;
-        h->tf.kpad = kpad;
-        h->tf.rb = tiles;
-        std::vector<float> lval(h->host.L_val.size());
-        for (size_t q = 0; q < lval.size(); ++q) lval[q] = (float)(lscale * h->host.L_val[q]);
-        std::vector<unsigned short> lidx(h->host.L_idx.begin(), h->host.L_idx.end());
-        if ((rc = upload(h, h->host.L_ptr, &h->tf.h_ptr))) return bail(rc);
-        if ((rc = upload(h, lidx, &h->tf.h_idx))) return bail(rc);
-        if ((rc = upload(h, lval, &h->tf.h_val))) return bail(rc);
-    }
-    if (h->precision == NPFEM_PREC_BF16) {
+    h->tf.ainv = a32;
+    h->tf.dense_p = dense_parts(n);
+    if (h->precision == NPFEM_PREC_BF16 && n <= kTcMaxVerts) {
         // tensor-core path: BF16 A^-1 in 128-row blocks with K padded to 16, and L for
         // the refinement residual
         const int kpad = (n + 15) & ~15, rb = (n + 127) / 128;
@@ -958,16 +1036,6 @@ int npfem_create(const npfem_mesh* mesh, const npfem_material* mat, const npfem_
         h->tf.ainv_lp = abf;
         h->tf.kpad = kpad;
         h->tf.rb = rb;
-        // the SIMT contraction of a BF16 handle (meshes the clusters do not take, idle-SM
-        // blocks) reads A^-1 in BF16 too: half the bytes of FP32
-        const int n8 = (n + 7) & ~7;
-        void* asq = h->alloc<unsigned short>((size_t)n8 * n8, &e);
-        if (e) return bail(e);
-        if (publish_inverse_bf16_square(h->ainv64, n, n8, asq, 0) != cudaSuccess ||
-            cudaDeviceSynchronize() != cudaSuccess)
-            return bail(fail(NPFEM_ERR_CUDA, "publishing the BF16 A^-1 failed"));
-        h->tf.ainv_b16 = asq;
-        h->tf.n8 = n8;
         // the refinement residual q - H~ r needs H~ = ms M + (1 + beta_D/h) L
         std::vector<float> lval(h->host.L_val.size());
         for (size_t q = 0; q < lval.size(); ++q) lval[q] = (float)(lscale * h->host.L_val[q]);

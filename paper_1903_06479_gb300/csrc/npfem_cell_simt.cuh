@@ -1,0 +1,60 @@
+// The persistent SIMT kernel: blocks pull cells from a work counter and solve them alone.
+// DN: every topology of the launch has the dense FP32 inverse (and no beta_D), so the kernel
+// holds no call of the sparse solve, whose register saves cost the rest of it 10 % (one
+// 642-vertex cell 1.31 against 1.47 ms per eight steps).
+#pragma once
+
+#include "npfem_cell.cuh"
+
+namespace npfem {
+namespace {
+
+template <typename T, int MAXT, int MINB, bool DN>
+__global__ void __launch_bounds__(MAXT, MINB) cell_kernel(const __grid_constant__ LaunchArgs<T> a)
+{
+    unsigned char* smem = smem_dyn;
+    CellSolver<T, !DN> S;
+    // first-iterate pass: evaluate only while most cells of the last step were accepted
+    const bool eval_first = a.defer && 2ll * (long long)a.defer[2] <= a.total_cells;
+    for (;;) {
+        const long long item = next_item(a, smem);
+        if (item < 0) break;
+        if (a.defer && !eval_first) {
+            if (threadIdx.x == 0) a.defer[3 + atomicAdd(a.defer, 1u)] = (unsigned int)item;
+            continue;
+        }
+        int gi = 0;
+        while (gi + 1 < a.n_groups && item >= a.g[gi + 1].cell_begin) ++gi;
+        S.bind(a, a.g[gi], smem);
+        if (!S.begin(item - a.g[gi].cell_begin, a.g[gi].stats_off + item - a.g[gi].cell_begin)) continue;
+        const bool wants = S.wants_direction();
+        if (a.need && wants && threadIdx.x == 0) atomicAdd(a.need, 1u);
+        if (a.defer && wants) {
+            // the cell needs iterations: the launch that follows solves it from the
+            // unchanged state
+            if (threadIdx.x == 0) a.defer[3 + atomicAdd(a.defer, 1u)] = (unsigned int)item;
+            continue;
+        }
+        const TopoDev<T>& tp = a.g[gi].topo;
+        while (S.wants_direction()) {
+            S.first_loop();
+            // r = H0 q
+            if constexpr (DN) contract_dense(tp, S.Dv, S.GCv, S.TRIv);
+            else solve_sparse<T, false>(tp.sp, S.tm, tp.n, S.Dv, S.GCv, S.SPv);
+            S.second_loop();
+            if (!S.descent()) {
+                // not a descent direction: drop the history, d = -H~^-1 g
+                S.count = 0;
+                if constexpr (DN) contract_dense(tp, S.g, S.GCv, S.TRIv);
+                else solve_sparse<T, false>(tp.sp, S.tm, tp.n, S.g, S.GCv, S.SPv);
+                S.negate_direction();
+            }
+            if (!S.line_search_update()) break;
+        }
+        S.finish();
+    }
+    release_counters(a.work, a.total_blocks);
+}
+
+}  // namespace
+}  // namespace npfem

@@ -121,11 +121,9 @@ struct CellShared {
     unsigned long long dbar;
     unsigned pend, batch, fin, flag;
     unsigned taddr;          // tensor-core path: tensor-memory base address
-    // TF32 contraction (SIMT kernel): per stage of the streamed A^-1 ring, "chunk landed"
-    // and "MMAs done reading it" barriers, and each stage's uses so far (phase parity)
-    unsigned long long tfull[2], tfree[2];
-    unsigned tuse[2];
-    int tfail;               // a bounded wait gave up: later contractions are skipped
+    // cluster kernel (several blocks per cell): blocks, this block's rank, parity of the
+    // reductions' exchange buffer
+    int cl_size, cl_rank, cl_par;
     int bad;
     int accept;
     int push;
@@ -153,12 +151,80 @@ __device__ __forceinline__ T prm(double d, float f)
 // value per warp) instead of on warp 0 alone, at the price of one more barrier.
 constexpr int kSpreadReduce = 8;
 
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Shared-memory address of p (a pointer into this block's shared memory) in block `rank`
+// of the cluster.
+__device__ __forceinline__ uint32_t remote_addr(const void* p, int rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+
+__device__ __forceinline__ void st_remote(float* p, int rank, float v)
+{
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote_addr(p, rank)), "f"(v) : "memory");
+}
+
+__device__ __forceinline__ void st_remote(double* p, int rank, double v)
+{
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote_addr(p, rank)), "d"(v) : "memory");
+}
+
+// Exchange buffer of the cluster's reductions: [parity][rank][32 values], the upper half
+// of the reductions' 8 KB (16 warps' partials take at most the lower half).
+template <typename T>
+__device__ __forceinline__ T* cluster_exchange(unsigned char* smem, int par, int rank)
+{
+    return reinterpret_cast<T*>(smem + 4096) + (par * 8 + rank) * 32;
+}
+
+// Totals over the cluster of KC compensated and KP plain sums, each block's in sh->out
+// and sh->outlo: every block gets every block's and adds them in rank order, so that all
+// hold the same bits.  Two buffers in turn: a block can only write the next but one after
+// every block has read this one (the barrier of the next reduction).
+template <typename T, int KC, int KP, typename Epi>
+__device__ __forceinline__ void cluster_merge(unsigned char* smem, Epi epi)
+{
+    constexpr int W = 2 * KC + KP;
+    static_assert(W <= 32, "exchange buffer");
+    CellShared<T>* sh = cell_shared<T>(smem);
+    const int C = sh->cl_size, rank = sh->cl_rank, par = sh->cl_par, tid = threadIdx.x;
+    for (int q = tid; q < C * W; q += blockDim.x) {
+        const int d = q / W, k = q - d * W;
+        const T v = k < KC + KP ? sh->out[k] : sh->outlo[k - KC - KP];
+        st_remote(cluster_exchange<T>(smem, par, rank) + k, d, v);
+    }
+    cluster_barrier();
+    if (tid < KC + KP) {
+        Acc<T> b;
+        T plain = T(0);
+        for (int r = 0; r < C; ++r) {
+            const T* e = cluster_exchange<T>(smem, par, r);
+            if (tid < KC)
+                b.merge(e[tid], e[KC + KP + tid]);
+            else
+                plain += e[tid];
+        }
+        sh->out[tid] = tid < KC ? b.hi : plain;
+        if (tid < KC) sh->outlo[tid] = b.lo;
+    }
+    if (tid == 0) sh->cl_par = par ^ 1;
+    __syncthreads();
+    if (tid == 0) epi(sh);
+    __syncthreads();
+}
+
 struct NoEpi {
     template <typename S>
     __device__ __forceinline__ void operator()(S*) const {}
 };
 
-template <typename T, int K, typename Epi = NoEpi>
+template <typename T, int K, bool CL = false, typename Epi = NoEpi>
 __device__ __forceinline__ void block_reduce(Acc<T> (&a)[K], unsigned char* smem, Epi epi = Epi())
 {
     T* red = reinterpret_cast<T*>(smem);  // [32 warps][K][2]
@@ -200,7 +266,7 @@ __device__ __forceinline__ void block_reduce(Acc<T> (&a)[K], unsigned char* smem
             }
         }
         __syncthreads();
-        if (threadIdx.x == 0) epi(sh);
+        if (!CL && threadIdx.x == 0) epi(sh);
     } else if (w == 0) {
         Acc<T> b[K];
 #pragma unroll
@@ -223,15 +289,16 @@ __device__ __forceinline__ void block_reduce(Acc<T> (&a)[K], unsigned char* smem
                 sh->out[k] = b[k].hi;
                 sh->outlo[k] = b[k].lo;
             }
-            epi(sh);
+            if (!CL) epi(sh);
         }
     }
     __syncthreads();
+    if constexpr (CL) cluster_merge<T, K, 0>(smem, epi);
 }
 
 // Like block_reduce, for KC compensated and KP plain sums (out[0..KC) compensated,
 // out[KC..KC+KP) plain).
-template <typename T, int KC, int KP, typename Epi = NoEpi>
+template <typename T, int KC, int KP, bool CL = false, typename Epi = NoEpi>
 __device__ __forceinline__ void block_reduce_cp(Acc<T> (&a)[KC], T (&p)[KP], unsigned char* smem, Epi epi = Epi())
 {
     constexpr int W = 2 * KC + KP;
@@ -286,7 +353,7 @@ __device__ __forceinline__ void block_reduce_cp(Acc<T> (&a)[KC], T (&p)[KP], uns
             }
         }
         __syncthreads();
-        if (threadIdx.x == 0) epi(sh);
+        if (!CL && threadIdx.x == 0) epi(sh);
     } else if (w == 0) {
         Acc<T> b[KC];
         T q[KP];
@@ -320,14 +387,15 @@ __device__ __forceinline__ void block_reduce_cp(Acc<T> (&a)[KC], T (&p)[KP], uns
             }
 #pragma unroll
             for (int k = 0; k < KP; ++k) sh->out[KC + k] = q[k];
-            epi(sh);
+            if (!CL) epi(sh);
         }
     }
     __syncthreads();
+    if constexpr (CL) cluster_merge<T, KC, KP>(smem, epi);
 }
 
 // Plain (uncompensated) block sum of K values, for dot products of the direction.
-template <typename T, int K, typename Epi = NoEpi>
+template <typename T, int K, bool CL = false, typename Epi = NoEpi>
 __device__ __forceinline__ void block_sum(T (&p)[K], unsigned char* smem, Epi epi = Epi())
 {
     T* red = reinterpret_cast<T*>(smem);
@@ -351,7 +419,7 @@ __device__ __forceinline__ void block_sum(T (&p)[K], unsigned char* smem, Epi ep
             if (lane == 0) sh->out[k] = q;
         }
         __syncthreads();
-        if (threadIdx.x == 0) epi(sh);
+        if (!CL && threadIdx.x == 0) epi(sh);
     } else if (w == 0) {
         T q[K];
 #pragma unroll
@@ -363,10 +431,11 @@ __device__ __forceinline__ void block_sum(T (&p)[K], unsigned char* smem, Epi ep
         if (lane == 0) {
 #pragma unroll
             for (int k = 0; k < K; ++k) sh->out[k] = q[k];
-            epi(sh);
+            if (!CL) epi(sh);
         }
     }
     __syncthreads();
+    if constexpr (CL) cluster_merge<T, 0, K>(smem, epi);
 }
 
 // Four consecutive elements of a per-cell vector (3 n_pad values, n_pad a multiple of

@@ -1,7 +1,7 @@
 // One-time FP64 inversion of the constant Hessian approximation H~ = M~/h^2 + L
 // (Sec. 2.1.1: H~ is constant and SPD, so it is factored once).  The library keeps
-// the dense inverse A^-1 so that every cell sharing a topology applies it as a
-// contraction.  Gauss-Jordan elimination without pivoting is stable for SPD
+// the dense inverse A^-1 for npfem_get_inverse and, in BF16 or FP32, for the meshes whose
+// cells apply it as a contraction (the others use the sparse factor of npfem_sparse.cpp).  Gauss-Jordan elimination without pivoting is stable for SPD
 // matrices; the whole elimination is one cooperative launch.
 #include <cuda_bf16.h>
 
@@ -103,24 +103,12 @@ __global__ void symmetrise_inplace(double* A, int n)
     }
 }
 
-__global__ void symmetrise_publish(const double* A, int n, int n_pad, float* o32, double* o64, __nv_bfloat16* obf,
-                                   float* otf)
+__global__ void publish_fp32(const double* A, int n, int n_pad, float* out)
 {
-    size_t total = (size_t)n_pad * n_pad;
+    const size_t total = (size_t)n_pad * n_pad;
     for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < total; q += (size_t)gridDim.x * blockDim.x) {
-        int i = (int)(q / n_pad), j = (int)(q % n_pad);
-        double v = 0.0;
-        if (i < n && j < n) v = 0.5 * (A[(size_t)i * n + j] + A[(size_t)j * n + i]);
-        if (o32) o32[q] = (float)v;
-        if (o64) o64[q] = v;
-        if (obf) obf[q] = __double2bfloat16(v);
-        if (otf) {
-            // round to the 10-bit TF32 mantissa (round to nearest, ties away)
-            float f = (float)v;
-            unsigned u = __float_as_uint(f);
-            u = (u + 0x1000u) & 0xffffe000u;
-            otf[q] = __uint_as_float(u);
-        }
+        const int i = (int)(q / n_pad), j = (int)(q % n_pad);
+        out[q] = i < n && j < n ? (float)(0.5 * (A[(size_t)i * n + j] + A[(size_t)j * n + i])) : 0.f;
     }
 }
 
@@ -134,50 +122,7 @@ __global__ void publish_bf16_blocked(const double* A, int n, int rows_pad, int k
     }
 }
 
-// Element (row i, column k) of A^-1 at its place in the TF32 chunks: chunk (tile, c) of
-// 128 rows x 32 K holds 16 x 8 core matrices of 8 rows x 4 elements (128 bytes), K-adjacent
-// core matrices 128 bytes apart, row groups 1024 bytes apart.
-__global__ void publish_tf32_tiled(const double* A, int n, int tiles, int kpad, float* out)
-{
-    const int nch = kpad / 32;
-    const size_t total = (size_t)tiles * 128 * kpad;
-    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < total; q += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(q / kpad), k = (int)(q % kpad);
-        const int t = i >> 7, r = i & 127, c = k >> 5, kk = k & 31;
-        double v = (i < n && k < n) ? A[(size_t)i * n + k] : 0.0;
-        float f = (float)v;
-        unsigned u;
-        asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(u) : "f"(f));
-        const size_t chunk = (size_t)t * nch + c;
-        const size_t off = chunk * (128 * 32) + (size_t)(((r >> 3) * 8 + (kk >> 2)) * 32 + (r & 7) * 4 + (kk & 3));
-        out[off] = __uint_as_float(u);
-    }
-}
-
 }  // namespace
-
-cudaError_t publish_inverse_tf32_tiled(const double* A, int n, int tiles, int kpad, float* out, cudaStream_t s)
-{
-    publish_tf32_tiled<<<1024, 256, 0, s>>>(A, n, tiles, kpad, out);
-    count_launch();
-    return cudaGetLastError();
-}
-
-__global__ void publish_bf16_square(const double* A, int n, int n8, __nv_bfloat16* out)
-{
-    size_t total = (size_t)n8 * n8;
-    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < total; q += (size_t)gridDim.x * blockDim.x) {
-        int i = (int)(q / n8), j = (int)(q % n8);
-        out[q] = __double2bfloat16((i < n && j < n) ? A[(size_t)i * n + j] : 0.0);
-    }
-}
-
-cudaError_t publish_inverse_bf16_square(const double* A, int n, int n8, void* out, cudaStream_t s)
-{
-    publish_bf16_square<<<1024, 256, 0, s>>>(A, n, n8, static_cast<__nv_bfloat16*>(out));
-    count_launch();
-    return cudaGetLastError();
-}
 
 cudaError_t publish_inverse_bf16_blocked(const double* A, int n, int rows_pad, int kpad, void* out, cudaStream_t s)
 {
@@ -207,13 +152,14 @@ cudaError_t invert_spd_fp64(double* A, int n, double* prow, int* d_flag, cudaStr
     return cudaGetLastError();
 }
 
-cudaError_t publish_inverse(const double* A, int n, int n_pad, float* o32, double* o64, void* obf, float* otf,
-                            cudaStream_t s)
+cudaError_t symmetrise(double* A, int n, int n_pad, float* out, cudaStream_t s)
 {
-    symmetrise_inplace<<<1024, 256, 0, s>>>(const_cast<double*>(A), n);
+    symmetrise_inplace<<<1024, 256, 0, s>>>(A, n);
     count_launch();
-    symmetrise_publish<<<1024, 256, 0, s>>>(A, n, n_pad, o32, o64, (__nv_bfloat16*)obf, otf);
-    count_launch();
+    if (out) {
+        publish_fp32<<<1024, 256, 0, s>>>(A, n, n_pad, out);
+        count_launch();
+    }
     return cudaGetLastError();
 }
 

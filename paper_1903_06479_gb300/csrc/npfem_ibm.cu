@@ -4,10 +4,12 @@
 // iteration that makes the fluid follow the membrane (Steps 0-5 of Sec. 2.3).
 //
 // The four-point kernel w(r) of Sec. 2.3 gives each vertex a 4 x 4 x 4 stencil of
-// lattice nodes with weights w(r_x - i) w(r_y - j) w(r_z - k).  One thread handles
-// one vertex: it forms the vertex's area share A_k (a third of its triangles' areas)
-// and unit normal n_k from the current positions, then gathers (or, when spreading,
-// scatters with atomics) over its stencil.  Lattice coordinates are formed in FP64
+// lattice nodes with weights w(r_x - i) w(r_y - j) w(r_z - k).  Four lanes handle
+// one vertex, lane q the nodes of x offset q, so that a stencil row of four consecutive
+// nodes is one 64-byte (velocity, force) or 128-byte (stress) access: what bounds these
+// kernels is the number of L1/L2 sectors and atomic operations per stencil.  The lanes
+// share the vertex's triangles for its area share A_k (a third of its triangles' areas)
+// and unit normal n_k at the current positions; their stencil sums meet in two shuffles.  Lattice coordinates are formed in FP64
 // (a 100 um domain at FP32 would round the fractional lattice offset to ~1e-5); the
 // weights and sums are FP32.
 //
@@ -18,6 +20,7 @@
 //    that spreading is the adjoint of interpolation;
 //  * stencil nodes outside the lattice contribute nothing.
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 
 #include <algorithm>
@@ -40,6 +43,7 @@ struct LatDev {
 struct IbmGroup {
     TopoDev<float> topo;
     long long vert_begin;  // first global vertex index of the group
+    long long cell_begin;  // first global cell of the group
     long long state_off;   // element offset of the group's first cell in the SoA arrays
     int cells;
 };
@@ -47,7 +51,7 @@ struct IbmGroup {
 struct IbmArgs {
     IbmGroup g[kMaxGroups];
     int n_groups;
-    long long total_verts;
+    long long total_verts, total_cells;
     LatDev lat;
     const float* x;       // SoA positions
     const float* field;   // sigma [nodes][8] (forces) or a velocity [nodes][4]
@@ -55,6 +59,7 @@ struct IbmArgs {
     const float* uvert;   // forcing: membrane vertex velocities U_k (SoA)
     float* out;           // SoA vertex output
     float* lat_out;       // forcing: lattice force [nodes][4] (spread phase)
+    int lat_vec;          // lat_out is 16-byte aligned (vector reductions)
     float rho, dt;
     int mode;             // forces: 0 full stencil, 1 exterior nodes, 2 farthest exterior node
     int phase;            // forcing: 0 f = (U - u*)/dt, 1 spread f, 2 f += (U - u_l)/dt
@@ -75,15 +80,30 @@ struct Stencil {
     float w[3][4];       // weights of nodes i0 + a, a = 0..3
 };
 
+// Base node of a coordinate's stencil.  A point far outside the lattice (or not finite) gets
+// a stencil with no nodes.
+__device__ __forceinline__ double lattice_floor(const LatDev& L, double origin, float X, double* r)
+{
+    const double v = ((double)X - origin) * L.inv_dx;
+    *r = v == v ? fmin(fmax(v, -1.0e6), 1.0e6) : -1.0e6;
+    return floor(*r);
+}
+
+__device__ __forceinline__ int lattice_base(const LatDev& L, double origin, float X)
+{
+    double r;
+    return (int)lattice_floor(L, origin, X, &r) - 1;
+}
+
 __device__ __forceinline__ void make_stencil(const LatDev& L, float X, float Y, float Z, Stencil& s)
 {
-    const double r[3] = {((double)X - L.ox) * L.inv_dx, ((double)Y - L.oy) * L.inv_dx, ((double)Z - L.oz) * L.inv_dx};
+    const double o[3] = {L.ox, L.oy, L.oz};
+    const float P[3] = {X, Y, Z};
     int b[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        // a point far outside the lattice (or not finite) gets a stencil with no nodes
-        const double rd = r[d] == r[d] ? fmin(fmax(r[d], -1.0e6), 1.0e6) : -1.0e6;
-        const double f = floor(rd);
+        double rd;
+        const double f = lattice_floor(L, o[d], P[d], &rd);
         b[d] = (int)f - 1;
         const float t = (float)(rd - f);
         s.t[d] = t;
@@ -119,139 +139,377 @@ __device__ __forceinline__ long long node_index(const LatDev& L, int i, int j, i
     return ((long long)k * L.ny + j) * L.nx + i;
 }
 
-// Eq. Fext, one vertex per thread.
+// Sum over the four lanes of a vertex.
+__device__ __forceinline__ float sum4(float v)
+{
+    v += __shfl_xor_sync(kFull, v, 1);
+    return v + __shfl_xor_sync(kFull, v, 2);
+}
+
+// vertex_area_normal() of vertex i shared by its four lanes (lane q takes every fourth
+// incident triangle); the normal's sums only when N is given.
+template <bool kNormal>
+__device__ __forceinline__ void area_normal4(const TopoDev<float>& tp, const float* xc, int i, int q, float* A, float* nv)
+{
+    const int n_ = tp.n;
+    float N[3] = {0.f, 0.f, 0.f}, S = 0.f;
+    const int b0 = __ldg(&tp.inc_ptr[i]), b1 = __ldg(&tp.inc_ptr[i + 1]);
+    for (int e = b0 + q; e < b1; e += 4) {
+        const ushort4 tv = __ldg(&tp.tri[__ldg(&tp.inc_idx[e]) >> 2]);
+        const int p0 = tv.x, p1 = tv.y, p2 = tv.z;
+        float e1[3], e2[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float x0 = xc[c * n_ + p0];
+            e1[c] = xc[c * n_ + p1] - x0;
+            e2[c] = xc[c * n_ + p2] - x0;
+        }
+        const float cr[3] = {e1[1] * e2[2] - e1[2] * e2[1], e1[2] * e2[0] - e1[0] * e2[2], e1[0] * e2[1] - e1[1] * e2[0]};
+        if (kNormal)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) N[c] += 0.5f * cr[c];
+        S += sqrtf(cr[0] * cr[0] + cr[1] * cr[1] + cr[2] * cr[2]);
+    }
+    *A = sum4(S) * (1.f / 6.f);
+    if (kNormal) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) N[c] = sum4(N[c]);
+        const float inv = rsqrtf(N[0] * N[0] + N[1] * N[1] + N[2] * N[2]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) nv[c] = N[c] * inv;
+    }
+}
+
+// Vertices per block of 256 threads; the loops below run to the rounded count so that the
+// shuffles see whole warps (vertices past the end repeat the last and write nothing).
+constexpr int kVertsPerBlock = 64;
+
+// Row (b, c) of a vertex's stencil, lane q's node: its index, or -1 outside the lattice.
+__device__ __forceinline__ long long row_node(const LatDev& L, const Stencil& s, int q, int b, int c)
+{
+    const int ii = s.i0 + q, jj = s.j0 + b, kk = s.k0 + c;
+    return node_in(L, ii, jj, kk) ? node_index(L, ii, jj, kk) : -1;
+}
+
+// Eq. Fext, four lanes per vertex.
 __global__ void __launch_bounds__(256) ibm_forces_kernel(const __grid_constant__ IbmArgs a)
 {
     const LatDev& L = a.lat;
-    for (long long gv = blockIdx.x * (long long)blockDim.x + threadIdx.x; gv < a.total_verts;
-         gv += (long long)gridDim.x * blockDim.x) {
+    const int q = threadIdx.x & 3;
+    for (long long v0 = blockIdx.x * (long long)kVertsPerBlock; v0 < a.total_verts; v0 += (long long)gridDim.x * kVertsPerBlock) {
+        const long long gv = v0 + (threadIdx.x >> 2);
+        const bool live = gv < a.total_verts;
         long long cell;
         int i;
-        const IbmGroup& G = locate(a, gv, &cell, &i);
+        const IbmGroup& G = locate(a, live ? gv : a.total_verts - 1, &cell, &i);
         const int n = G.topo.n;
         const long long so = G.state_off + cell * 3LL * n;
         const float* xc = a.x + so;
         float A, nv[3];
-        vertex_area_normal(G.topo, xc, i, &A, nv);
+        area_normal4<true>(G.topo, xc, i, q, &A, nv);
         Stencil s;
         make_stencil(L, xc[i], xc[n + i], xc[2 * n + i], s);
+        const float wq = q == 0 ? s.w[0][0] : (q == 1 ? s.w[0][1] : (q == 2 ? s.w[0][2] : s.w[0][3]));
         float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, wsum = 0.f, dbest = -1.f;
-        for (int c = 0; c < 4; ++c)
-            for (int b = 0; b < 4; ++b)
-                for (int q = 0; q < 4; ++q) {
-                    const int ii = s.i0 + q, jj = s.j0 + b, kk = s.k0 + c;
-                    if (!node_in(L, ii, jj, kk)) continue;
-                    float wgt = s.w[0][q] * s.w[1][b] * s.w[2][c];
-                    if (a.mode != 0) {
-                        // offset node - X in um; exterior when it points along n
-                        const float d[3] = {((float)(q - 1) - s.t[0]) * L.dx, ((float)(b - 1) - s.t[1]) * L.dx,
-                                            ((float)(c - 1) - s.t[2]) * L.dx};
-                        if (!(d[0] * nv[0] + d[1] * nv[1] + d[2] * nv[2] > 0.f)) continue;
-                        if (a.mode == 2) {
-                            const float d2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-                            if (!(d2 > dbest)) continue;  // keep the first among equals
-                            dbest = d2;
-                            wgt = 1.f;
+        int first = 64;
 #pragma unroll
-                            for (int e = 0; e < 6; ++e) acc[e] = 0.f;
-                            wsum = 0.f;
-                        }
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const long long nd = row_node(L, s, q, b, c);
+                if (nd < 0) continue;
+                float wgt = wq * s.w[1][b] * s.w[2][c];
+                if (a.mode != 0) {
+                    // offset node - X in um; exterior when it points along n
+                    const float d[3] = {((float)(q - 1) - s.t[0]) * L.dx, ((float)(b - 1) - s.t[1]) * L.dx,
+                                        ((float)(c - 1) - s.t[2]) * L.dx};
+                    if (!(d[0] * nv[0] + d[1] * nv[1] + d[2] * nv[2] > 0.f)) continue;
+                    if (a.mode == 2) {
+                        const float d2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+                        if (!(d2 > dbest)) continue;  // keep the first among equals
+                        dbest = d2;
+                        first = 16 * c + 4 * b + q;
+                        wgt = 1.f;
+#pragma unroll
+                        for (int e = 0; e < 6; ++e) acc[e] = 0.f;
+                        wsum = 0.f;
                     }
-                    const float4* P = reinterpret_cast<const float4*>(a.field + 8 * node_index(L, ii, jj, kk));
-                    const float4 s0 = __ldg(P), s1 = __ldg(P + 1);
-                    acc[0] += wgt * s0.x; acc[1] += wgt * s0.y; acc[2] += wgt * s0.z;
-                    acc[3] += wgt * s0.w; acc[4] += wgt * s1.x; acc[5] += wgt * s1.y;
-                    wsum += wgt;
                 }
+                const float4* P = reinterpret_cast<const float4*>(a.field + 8 * nd);
+                const float4 s0 = __ldg(P), s1 = __ldg(P + 1);
+                acc[0] += wgt * s0.x; acc[1] += wgt * s0.y; acc[2] += wgt * s0.z;
+                acc[3] += wgt * s0.w; acc[4] += wgt * s1.x; acc[5] += wgt * s1.y;
+                wsum += wgt;
+            }
+        if (a.mode == 2) {
+            // the farthest node of the four lanes' (the first in z, y, x order among equals)
+            float db = dbest;
+            int fb = first;
+#pragma unroll
+            for (int o = 1; o < 4; o <<= 1) {
+                const float d2 = __shfl_xor_sync(kFull, db, o);
+                const int f2 = __shfl_xor_sync(kFull, fb, o);
+                if (d2 > db || (d2 == db && f2 < fb)) {
+                    db = d2;
+                    fb = f2;
+                }
+            }
+            if (fb != first) {
+#pragma unroll
+                for (int e = 0; e < 6; ++e) acc[e] = 0.f;
+                wsum = 0.f;
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 6; ++e) acc[e] = sum4(acc[e]);
         if (a.mode != 0) {
+            wsum = sum4(wsum);
             const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
 #pragma unroll
             for (int e = 0; e < 6; ++e) acc[e] *= inv;
         }
-        // (xx, yy, zz, xy, xz, yz) times n, scaled by rho A_k
+        // (xx, yy, zz, xy, xz, yz) times n, scaled by rho A_k: lane q writes component q
         const float sc = a.rho * A;
-        float* o = a.out + so;
-        o[i] = sc * (acc[0] * nv[0] + acc[3] * nv[1] + acc[4] * nv[2]);
-        o[n + i] = sc * (acc[3] * nv[0] + acc[1] * nv[1] + acc[5] * nv[2]);
-        o[2 * n + i] = sc * (acc[4] * nv[0] + acc[5] * nv[1] + acc[2] * nv[2]);
+        const float f = q == 0 ? acc[0] * nv[0] + acc[3] * nv[1] + acc[4] * nv[2]
+                      : q == 1 ? acc[3] * nv[0] + acc[1] * nv[1] + acc[5] * nv[2]
+                               : acc[4] * nv[0] + acc[5] * nv[1] + acc[2] * nv[2];
+        if (live && q < 3) a.out[so + q * n + i] = sc * f;
     }
 }
 
-// Stencil sum of a [nodes][4] field (plus dt times a second one, if given).
-__device__ __forceinline__ void gather4(const LatDev& L, const Stencil& s, const float* F, const float* F2, float dt,
-                                        float out[3])
+// Stencil sum of a [nodes][4] field (plus dt times a second one, if given), over the
+// four lanes of a vertex.
+__device__ __forceinline__ void gather4(const LatDev& L, const Stencil& s, int q, float wq, const float* F, const float* F2,
+                                        float dt, float out[3])
 {
-    out[0] = out[1] = out[2] = 0.f;
-    for (int c = 0; c < 4; ++c)
-        for (int b = 0; b < 4; ++b)
-            for (int q = 0; q < 4; ++q) {
-                const int ii = s.i0 + q, jj = s.j0 + b, kk = s.k0 + c;
-                if (!node_in(L, ii, jj, kk)) continue;
-                const float wgt = s.w[0][q] * s.w[1][b] * s.w[2][c];
-                const long long nd = node_index(L, ii, jj, kk);
-                float4 u = __ldg(reinterpret_cast<const float4*>(F) + nd);
-                if (F2) {
-                    // the corrected lattice velocity u* + dt f (Step 2) is formed on the fly;
-                    // F2 is written by an earlier launch, so a plain (coherent) load
-                    const float4 f = reinterpret_cast<const float4*>(F2)[nd];
-                    u.x += dt * f.x;
-                    u.y += dt * f.y;
-                    u.z += dt * f.z;
-                }
-                out[0] += wgt * u.x;
-                out[1] += wgt * u.y;
-                out[2] += wgt * u.z;
+    float4 u[16];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+        const long long nd = row_node(L, s, q, r & 3, r >> 2);
+        u[r] = nd >= 0 ? __ldg(reinterpret_cast<const float4*>(F) + nd) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float o[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+        const float wgt = wq * s.w[1][r & 3] * s.w[2][r >> 2];
+        if (F2) {
+            // the corrected lattice velocity u* + dt f (Step 2) is formed on the fly;
+            // F2 is written by an earlier launch, so a plain (coherent) load
+            const long long nd = row_node(L, s, q, r & 3, r >> 2);
+            if (nd >= 0) {
+                const float4 f = reinterpret_cast<const float4*>(F2)[nd];
+                u[r].x += dt * f.x;
+                u[r].y += dt * f.y;
+                u[r].z += dt * f.z;
             }
+        }
+        o[0] += wgt * u[r].x;
+        o[1] += wgt * u[r].y;
+        o[2] += wgt * u[r].z;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) out[c] = sum4(o[c]);
 }
 
-// Velocity interpolation (phase -1) and the phases of the multi-direct forcing.
-__global__ void __launch_bounds__(256) ibm_forcing_kernel(const __grid_constant__ IbmArgs a)
+// One 16-byte reduction per node instead of three scalar atomics (vec: p is 16-byte
+// aligned; the node's unused fourth value gains zero).
+__device__ __forceinline__ void red4(float* p, float x, float y, float z, int vec)
+{
+    if (!vec) {
+        atomicAdd(p, x);
+        atomicAdd(p + 1, y);
+        atomicAdd(p + 2, z);
+        return;
+    }
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(p)), "f"(x), "f"(y), "f"(z),
+                 "f"(0.f)
+                 : "memory");
+}
+
+// What a vertex's four lanes do with its stencil sum u of the velocity: interpolation
+// (phase -1) or Steps 0 and 4 of the multi-direct forcing.
+__device__ __forceinline__ void take_sum(const IbmArgs& a, long long so, int n, int i, int q, bool live, const float (&u)[3])
+{
+    if (!live || q > 2) return;
+    const float uq = q == 0 ? u[0] : (q == 1 ? u[1] : u[2]);
+    const long long at = so + q * n + i;
+    if (a.phase < 0) {
+        a.out[at] = uq;
+        return;
+    }
+    const float slip = (a.uvert[at] - uq) * (1.f / a.dt);
+    a.out[at] = a.phase == 0 ? slip : a.out[at] + slip;
+}
+
+__device__ __forceinline__ float lane_weight(const Stencil& s, int q)
+{
+    return q == 0 ? s.w[0][0] : (q == 1 ? s.w[0][1] : (q == 2 ? s.w[0][2] : s.w[0][3]));
+}
+
+// One vertex of a phase straight on the lattice.
+__device__ __forceinline__ void vertex_phase(const IbmArgs& a, const IbmGroup& G, long long cell, int i, int q, bool live)
 {
     const LatDev& L = a.lat;
-    for (long long gv = blockIdx.x * (long long)blockDim.x + threadIdx.x; gv < a.total_verts;
-         gv += (long long)gridDim.x * blockDim.x) {
+    const int n = G.topo.n;
+    const long long so = G.state_off + cell * 3LL * n;
+    const float* xc = a.x + so;
+    Stencil s;
+    make_stencil(L, xc[i], xc[n + i], xc[2 * n + i], s);
+    const float wq = lane_weight(s, q);
+    if (a.phase == 1) {
+        // Step 1: spread f_k with weight A_k dx / dx^3 per unit stencil weight
+        float A;
+        area_normal4<false>(G.topo, xc, i, q, &A, nullptr);
+        const float* o = a.out + so;
+        const float sc = A / (L.dx * L.dx) * wq;
+        const float f[3] = {sc * o[i], sc * o[n + i], sc * o[2 * n + i]};
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+            const long long nd = row_node(L, s, q, r & 3, r >> 2);
+            const float wgt = s.w[1][r & 3] * s.w[2][r >> 2];
+            if (live && nd >= 0) red4(a.lat_out + 4 * nd, wgt * f[0], wgt * f[1], wgt * f[2], a.lat_vec);
+        }
+        return;
+    }
+    float u[3];
+    gather4(L, s, q, wq, a.field, a.phase == 2 ? a.field2 : nullptr, a.dt, u);
+    take_sum(a, so, n, i, q, live, u);
+}
+
+// Velocity interpolation (phase -1) and the phases of the multi-direct forcing, vertex by
+// vertex (few cells, or small ones).
+__global__ void __launch_bounds__(256) ibm_forcing_kernel(const __grid_constant__ IbmArgs a)
+{
+    for (long long v0 = blockIdx.x * (long long)kVertsPerBlock; v0 < a.total_verts; v0 += (long long)gridDim.x * kVertsPerBlock) {
+        const long long gv = v0 + (threadIdx.x >> 2);
+        const bool live = gv < a.total_verts;
         long long cell;
         int i;
-        const IbmGroup& G = locate(a, gv, &cell, &i);
+        const IbmGroup& G = locate(a, live ? gv : a.total_verts - 1, &cell, &i);
+        vertex_phase(a, G, cell, i, threadIdx.x & 3, live);
+    }
+}
+
+// The same, a block per cell: the lattice nodes around the cell (a box of the stencils'
+// extent) pass through shared memory, read or reduced once instead of once per stencil that
+// meets them (a 642-vertex cell has 41 K stencil nodes in a box of about 1.7 K).  A cell
+// whose box does not fit goes vertex by vertex.
+constexpr int kBoxNodes = 3000;
+constexpr long long kBoxMinCells = 128, kBoxMinVerts = 200;
+
+__global__ void __launch_bounds__(256) ibm_box_kernel(const __grid_constant__ IbmArgs a)
+{
+    extern __shared__ __align__(16) float box[];  // gather: float4 per node; spread: three rows
+    __shared__ int lo[3], hi[3];
+    const LatDev& L = a.lat;
+    const int tid = threadIdx.x, NT = blockDim.x, q = tid & 3;
+    for (long long gc = blockIdx.x; gc < a.total_cells; gc += gridDim.x) {
+        int gi = 0;
+        while (gi + 1 < a.n_groups && gc >= a.g[gi + 1].cell_begin) ++gi;
+        const IbmGroup& G = a.g[gi];
+        const long long cell = gc - G.cell_begin;
         const int n = G.topo.n;
         const long long so = G.state_off + cell * 3LL * n;
         const float* xc = a.x + so;
-        Stencil s;
-        make_stencil(L, xc[i], xc[n + i], xc[2 * n + i], s);
-        float* o = a.out + so;
-        if (a.phase == 1) {
-            // Step 1: spread f_k with weight A_k dx / dx^3 per unit stencil weight
-            float A, nv[3];
-            vertex_area_normal(G.topo, xc, i, &A, nv);
-            const float sc = A / (L.dx * L.dx);
-            const float f[3] = {sc * o[i], sc * o[n + i], sc * o[2 * n + i]};
-            for (int c = 0; c < 4; ++c)
-                for (int b = 0; b < 4; ++b)
-                    for (int q = 0; q < 4; ++q) {
-                        const int ii = s.i0 + q, jj = s.j0 + b, kk = s.k0 + c;
-                        if (!node_in(L, ii, jj, kk)) continue;
-                        const float wgt = s.w[0][q] * s.w[1][b] * s.w[2][c];
-                        float* P = a.lat_out + 4 * node_index(L, ii, jj, kk);
-                        atomicAdd(P, wgt * f[0]);
-                        atomicAdd(P + 1, wgt * f[1]);
-                        atomicAdd(P + 2, wgt * f[2]);
-                    }
-            continue;
+        if (tid < 3) {
+            lo[tid] = INT_MAX;
+            hi[tid] = INT_MIN;
         }
-        float u[3];
-        gather4(L, s, a.field, a.phase == 2 ? a.field2 : nullptr, a.dt, u);
-        if (a.phase < 0) {
-            o[i] = u[0];
-            o[n + i] = u[1];
-            o[2 * n + i] = u[2];
-            continue;
-        }
-        const float* U = a.uvert + so;
-        const float inv_dt = 1.f / a.dt;
+        __syncthreads();
+        int l[3] = {INT_MAX, INT_MAX, INT_MAX}, h[3] = {INT_MIN, INT_MIN, INT_MIN};
+        for (int i = tid; i < n; i += NT) {
+            const int b[3] = {lattice_base(L, L.ox, xc[i]), lattice_base(L, L.oy, xc[n + i]), lattice_base(L, L.oz, xc[2 * n + i])};
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float slip = (U[c * n + i] - u[c]) * inv_dt;
-            o[c * n + i] = a.phase == 0 ? slip : o[c * n + i] + slip;  // Step 0, or Step 4
+            for (int d = 0; d < 3; ++d) {
+                l[d] = min(l[d], b[d]);
+                h[d] = max(h[d], b[d]);
+            }
+        }
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            l[d] = __reduce_min_sync(kFull, l[d]);
+            h[d] = __reduce_max_sync(kFull, h[d]);
+            if ((tid & 31) == 0) {
+                atomicMin(&lo[d], l[d]);
+                atomicMax(&hi[d], h[d]);
+            }
+        }
+        __syncthreads();
+        const int x0 = lo[0], y0 = lo[1], z0 = lo[2];
+        const long long ex = (long long)hi[0] - x0 + 4, ey = (long long)hi[1] - y0 + 4, ez = (long long)hi[2] - z0 + 4;
+        const bool fits = ex <= kBoxNodes && ey <= kBoxNodes && ez <= kBoxNodes && ex * ey * ez <= kBoxNodes;
+        const int bx = (int)ex, by = (int)ey, nodes = fits ? (int)(ex * ey * ez) : 0;
+        // gather: the box's velocities; spread: zero sums
+        for (int e = tid; e < nodes; e += NT) {
+            if (a.phase == 1) {
+                box[e] = box[nodes + e] = box[2 * nodes + e] = 0.f;
+                continue;
+            }
+            const int k = e / (bx * by), j = (e - k * bx * by) / bx, ii = e - (k * by + j) * bx;
+            float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (node_in(L, x0 + ii, y0 + j, z0 + k)) {
+                const long long nd = node_index(L, x0 + ii, y0 + j, z0 + k);
+                u = __ldg(reinterpret_cast<const float4*>(a.field) + nd);
+                if (a.phase == 2) {
+                    // the corrected velocity u* + dt f (Step 2); f is written by an earlier launch
+                    const float4 f = reinterpret_cast<const float4*>(a.field2)[nd];
+                    u.x += a.dt * f.x;
+                    u.y += a.dt * f.y;
+                    u.z += a.dt * f.z;
+                }
+            }
+            reinterpret_cast<float4*>(box)[e] = u;
+        }
+        __syncthreads();
+        for (int v0 = 0; v0 < n; v0 += NT >> 2) {
+            const bool live = v0 + (tid >> 2) < n;
+            const int i = live ? v0 + (tid >> 2) : n - 1;
+            if (!fits) {
+                vertex_phase(a, G, cell, i, q, live);
+                continue;
+            }
+            Stencil s;
+            make_stencil(L, xc[i], xc[n + i], xc[2 * n + i], s);
+            const float wq = lane_weight(s, q);
+            const int at = ((s.k0 - z0) * by + (s.j0 - y0)) * bx + (s.i0 - x0) + q;
+            if (a.phase == 1) {
+                float A;
+                area_normal4<false>(G.topo, xc, i, q, &A, nullptr);
+                const float* o = a.out + so;
+                const float sc = A / (L.dx * L.dx) * wq;
+                const float f[3] = {sc * o[i], sc * o[n + i], sc * o[2 * n + i]};
+                if (!live) continue;
+#pragma unroll
+                for (int r = 0; r < 16; ++r) {
+                    const int e = at + ((r >> 2) * by + (r & 3)) * bx;
+                    const float wgt = s.w[1][r & 3] * s.w[2][r >> 2];
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) atomicAdd(&box[c * nodes + e], wgt * f[c]);
+                }
+            } else {
+                float o[3] = {0.f, 0.f, 0.f}, u[3];
+#pragma unroll
+                for (int r = 0; r < 16; ++r) {
+                    const float wgt = wq * s.w[1][r & 3] * s.w[2][r >> 2];
+                    const float4 f = reinterpret_cast<const float4*>(box)[at + ((r >> 2) * by + (r & 3)) * bx];
+                    o[0] += wgt * f.x;
+                    o[1] += wgt * f.y;
+                    o[2] += wgt * f.z;
+                }
+#pragma unroll
+                for (int c = 0; c < 3; ++c) u[c] = sum4(o[c]);
+                take_sum(a, so, n, i, q, live, u);
+            }
+        }
+        __syncthreads();
+        if (a.phase == 1) {
+            for (int e = tid; e < nodes; e += NT) {
+                const float fx = box[e], fy = box[nodes + e], fz = box[2 * nodes + e];
+                const int k = e / (bx * by), j = (e - k * bx * by) / bx, ii = e - (k * by + j) * bx;
+                if ((fx != 0.f || fy != 0.f || fz != 0.f) && node_in(L, x0 + ii, y0 + j, z0 + k))
+                    red4(a.lat_out + 4 * node_index(L, x0 + ii, y0 + j, z0 + k), fx, fy, fz, a.lat_vec);
+            }
+            __syncthreads();
         }
     }
 }
@@ -273,6 +531,8 @@ int fill_ibm(IbmArgs* a, npfem_handle* const* meshes, int n_groups, const int32_
             return set_error(NPFEM_ERR_INVALID_ARG, std::string(who) + ": FP32-state handles of one device only");
         a->g[g].topo = h->tf;
         a->g[g].vert_begin = v;
+        a->g[g].cell_begin = a->total_cells;
+        a->total_cells += cells[g];
         a->g[g].state_off = st;
         a->g[g].cells = cells[g];
         v += (long long)h->n * cells[g];
@@ -293,8 +553,23 @@ int fill_ibm(IbmArgs* a, npfem_handle* const* meshes, int n_groups, const int32_
 
 int ibm_grid(const npfem_handle* h, long long verts)
 {
-    const long long blocks = (verts + 255) / 256;
+    const long long blocks = (verts + kVertsPerBlock - 1) / kVertsPerBlock;
     return (int)std::max<long long>(1, std::min<long long>(blocks, (long long)std::max(h->sm_count, 1) * 8));
+}
+
+// A phase over all vertices: a block per cell where the cells fill the GPU and a cell's
+// stencils overlap, else vertex by vertex.
+cudaError_t launch_forcing(const IbmArgs& a, const npfem_handle* h, cudaStream_t s)
+{
+    if (a.phase != 1 && a.total_cells >= kBoxMinCells && a.total_verts >= kBoxMinVerts * a.total_cells) {
+        const int smem = kBoxNodes * (int)sizeof(float4);
+        const int grid = (int)std::min<long long>(a.total_cells, (long long)std::max(h->sm_count, 1) * 4);
+        ibm_box_kernel<<<grid, 256, smem, s>>>(a);
+    } else {
+        ibm_forcing_kernel<<<ibm_grid(h, a.total_verts), 256, 0, s>>>(a);
+    }
+    count_launch();
+    return cudaGetLastError();
 }
 
 struct DevGuard {
@@ -356,9 +631,7 @@ extern "C" int npfem_ibm_interpolate(npfem_handle* const* meshes, int n_groups, 
     a.field = u_lattice;
     a.out = u_vertex;
     a.phase = -1;
-    ibm_forcing_kernel<<<ibm_grid(meshes[0], a.total_verts), 256, 0, static_cast<cudaStream_t>(stream)>>>(a);
-    count_launch();
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_forcing(a, meshes[0], static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? 0 : launch_err("npfem_ibm_interpolate", e);
 }
 
@@ -380,16 +653,12 @@ extern "C" int npfem_ibm_forcing(npfem_handle* const* meshes, int n_groups, cons
     a.field2 = f_lattice;
     a.out = f_vertex;
     a.lat_out = f_lattice;
+    a.lat_vec = (reinterpret_cast<uintptr_t>(f_lattice) & 15) == 0;
     a.dt = (float)dt_fluid;
-    const int grid = ibm_grid(meshes[0], a.total_verts);
     cudaError_t e = cudaSuccess;
     auto run = [&](int phase) {
         a.phase = phase;
-        if (a.total_verts > 0) {
-            ibm_forcing_kernel<<<grid, 256, 0, s>>>(a);
-            count_launch();
-        }
-        return cudaGetLastError();
+        return a.total_verts > 0 ? launch_forcing(a, meshes[0], s) : cudaGetLastError();
     };
     e = run(0);  // Step 0: f_0 = (U - u*(X)) / dt
     for (int l = 0; l < cycles && e == cudaSuccess; ++l) {

@@ -11,12 +11,19 @@
 
 #include "../../include/npfem.h"
 
+#ifdef __CUDACC__
+#define NPFEM_HD __host__ __device__
+#else
+#define NPFEM_HD
+#endif
+
 namespace npfem {
 
 constexpr int kMaxGroups = 8;     // meshes per npfem_step launch
 constexpr int kMaxHistory = 8;    // L-BFGS window limit
 constexpr int kNumBaseVecs = 10;  // XN U UT G GT GC UY D TRI WR, then S[m], Y[m]
-constexpr int kMaxVecs = kNumBaseVecs + 2 * kMaxHistory;
+constexpr int V_SP = kNumBaseVecs + 2 * kMaxHistory;  // sparse solve's vectors (6 npos): TRI's space when that is in smem
+constexpr int kMaxVecs = V_SP + 1;
 constexpr int kFixedSmem = 12288; // reduction scratch (8 KB) + per-cell scalars at the start of dynamic smem
 
 // Per-cell buffers.  All are 3 x n_pad values except TRI (rows of kTriRow values per
@@ -26,7 +33,23 @@ constexpr int kTriRow = 12;
 
 enum Vec { V_XN = 0, V_U = 1, V_UT = 2, V_G = 3, V_GT = 4, V_GC = 5, V_UY = 6, V_D = 7, V_TRI = 8, V_WR = 9, V_SBASE = 10 };
 
-enum Contraction { CONTRACT_SIMT = 0, CONTRACT_TC_TF32 = 1, CONTRACT_TC_BF16 = 2 };
+// Schedules of the sparse solve by warps per block.
+constexpr int kSparseScheds = 6;
+NPFEM_HD constexpr int sparse_sched_warps(int v) { return 4 << v; }
+NPFEM_HD constexpr int sparse_sched_of(int warps) { return warps <= 4 ? 0 : (warps <= 8 ? 1 : (warps <= 16 ? 2 : (warps <= 32 ? 3 : (warps <= 64 ? 4 : 5)))); }
+
+// Sparse block factor (SparseHost) on the device: schedule entries [first iteration,
+// iterations, log2 lanes per row | barrier << 8, first row] by entry and warp.
+template <typename T>
+struct SparseDev {
+    int npos;
+    int entries[kSparseScheds];
+    const int4* sched[kSparseScheds];
+    const int* perm;             // [npos]
+    const int2* row;             // [rows]
+    const unsigned short* idx;   // [iterations][32]
+    const T* val;                // [iterations][32][4]
+};
 
 // Device-side tables of one mesh topology (all pointers are device memory owned by
 // the handle).  T is the solver's scalar type (float or double).
@@ -57,25 +80,23 @@ struct TopoDev {
     const unsigned short* ring8_idx;  // [n][8]
     const T* ring8_c;                 // [n][8]
     const T* ring8_ct;                // [n][8]
-    const T* ainv;               // [n_pad][n_pad] A^-1 in T (zero padding)
+    const T* ainv;               // FP32, up to kDenseMaxVerts: [n_pad][n_pad] A^-1 (zero padding); else null
+    int dense_p;                 // parts of every 128-row tile's columns (dense_parts)
+    SparseDev<T> sp;             // sparse block factor of H~ (applied as H~^-1)
+    SparseDev<T> spc;            // the same, cut finer, for a cluster's warps (FP64; else null)
     // Rayleigh damping with beta_D > 0: M~ = (1 + h alpha_D) M + h beta_D L is not
-    // diagonal.  minv: [n_pad][n_pad] M~^-1 in T for the first guess; L (CSR, T) for the
+    // diagonal.  spm: the sparse factor of M~ for the first guess; L (CSR, T) for the
     // inertia term's h beta_D L part; beta_h = beta_D / h.  Null pointers when beta_D = 0.
-    const T* minv;
+    SparseDev<T> spm;
     const int* l_ptr;
     const unsigned short* l_idx;
     const T* l_val;
     T beta_h;
-    const void* ainv_lp;         // A^-1 for the tensor-core contraction: BF16 row blocks, or TF32 chunks
-                                 // of 128 rows x 32 K in the MMA's core-matrix layout
-    // BF16 handles: A^-1 in BF16 (round to nearest even), [n8][n8] with n8 = n rounded up
-    // to 8 (zero padding), for the SIMT contraction's 256-row tiles (null otherwise)
-    const void* ainv_b16;
-    int n8;
+    const void* ainv_lp;         // A^-1 in BF16 row blocks for the tensor-core contraction
     const int* h_ptr;            // L (CSR, fp32) for the refinement residual q - H~ r
     const unsigned short* h_idx;
     const float* h_val;
-    int kpad, rb;                // tensor-core path: K padded (16 BF16, 32 TF32), row blocks of 128
+    int kpad, rb;                // tensor-core path: K padded to 16, row blocks of 128
     const T* rest_c;             // [3][n] rest positions about the rest centre of mass
     const float* mlp;            // learned warm start: packed parameters, weights rounded to BF16 (or null)
     const float* tmlp;           // temporal network along a trajectory (same layout), or null
@@ -96,7 +117,6 @@ struct GroupDesc {
     long long stats_off;   // index of the group's first cell in stats (and eval parts)
     int cells;
     int smem_bytes;        // dynamic smem this group needs (after kFixedSmem)
-    int scratch_floats;    // size of the TRI buffer in floats (the SIMT contraction's partials)
     long long carry_off;   // element offset of the group's first carried-pairs record in LaunchArgs::carry
     long long carry_rec;   // elements per record (carry_rec_elems)
     int loc[kMaxVecs];     // >= 0: byte offset in smem; < 0: -(byte offset in the CTA's global slot) - 1
@@ -107,11 +127,8 @@ struct SolverParams {
     double tol, c1, c2, armijo_noise;
     float tolf, c1f, c2f, armijo_noisef;  // FP32 copies for the FP32 path
     int mode;         // 0 = time step, 1 = objective/gradient evaluation
-    int contraction;  // Contraction
     int cluster;      // tensor-core path: blocks per cluster (= row blocks of A^-1)
     int refine;       // tensor-core path: refinement sweeps (0 or 1)
-    int tmem_cols;    // TF32 path: tensor-memory columns each block allocates
-    int tf_kpad;      // TF32 path: the largest padded K of the launch's groups (B operand size)
 };
 
 inline void set_solver_params(SolverParams* p, const npfem_opts& o)
@@ -184,11 +201,6 @@ struct LaunchArgs {
     SolverParams p;
 };
 
-#ifdef __CUDACC__
-#define NPFEM_HD __host__ __device__
-#else
-#define NPFEM_HD
-#endif
 // Carried L-BFGS pairs of one cell, in elements of the state type: the solver's history
 // ring as the last solve left it: [0] the pair count, [1] the ring head, [2] that
 // solve's iterations, from [4] the inner products s_i^T y_j by ring slot (m x m, padded
@@ -219,34 +231,81 @@ struct HostTopo {
 int build_host_topo(const npfem_mesh* mesh, const npfem_material* mat, int equal_mass, HostTopo* out,
                     std::string* err);
 
+// Sparse block factor of H~ over a nested-dissection tree (npfem_sparse.cpp).
+// Positions: perm[p] is the vertex at position p (-1: padding); position p holds t (the
+// forward sweep's vector), npos + p holds x (the solution).
+struct SparseHost {
+    int npos = 0;
+    std::vector<int> perm;
+    struct Slice {
+        int base, iters, lg, row;       // first 32-lane iteration, iterations, log2 lanes per row, first row
+    };
+    std::vector<Slice> slices;
+    std::vector<int> step_begin;        // [steps + 1] first slice of each step
+    std::vector<int> rows;              // [rows][2] position written (-1: none), vertex (-1: forward row)
+    std::vector<unsigned short> idx;    // [iterations][32] group index: positions 4 g .. 4 g + 3
+    std::vector<double> val;            // [iterations][32][4]
+    std::vector<int> sched[kSparseScheds];  // [entries][warps][4]: slice, barrier after it in bit 8 of lg
+};
+constexpr int kSparseWarps = 16;     // warps a step's work is spread over
+constexpr int kSparseWarpsCluster = 64;  // the same for a cluster per cell
+constexpr int kSparseMaxIters = 10;  // iterations of a slice a warp keeps in flight (FP32)
+// Largest mesh whose FP32 solve applies the dense inverse.  At 642 vertices it reads 1.65 MB
+// from L2 in 48.5 K cycles, the sparse factor 0.47 MB in eleven steps in 41 K, and a
+// population takes the same time with either; at 1026 (4.2 MB, 111 K) the factor is faster.
+constexpr int kDenseMaxVerts = 700;
+// Parts of the column range of every 128-row tile, items (tile, part) dealt to 16 warps in
+// turn: the number that minimises the busiest warp's columns (ceil(tiles P / 16) items of
+// ceil(n / P) columns) within max(32, 4 tiles) items.
+inline int dense_parts(int n)
+{
+    const int ntile = (n + 127) / 128, items = 4 * ntile > 32 ? 4 * ntile : 32;
+    int pmax = items / ntile < n / 4 ? items / ntile : n / 4;
+    if (pmax < 1) pmax = 1;
+    int P = 1;
+    long long best = -1;
+    for (int q = 1; q <= pmax; ++q) {
+        const long long cost = (long long)((ntile * q + 15) / 16) * ((((n + q - 1) / q) + 3) & ~3);
+        if (best < 0 || cost < best) {
+            best = cost;
+            P = q;
+        }
+    }
+    return P;
+}
+// Largest number of vertices the dissection leaves whole.
+constexpr int kSparseLeaf = 32;
+// Factor of mass_scale M + l_scale L, laid out for a block per cell and, if given, for a
+// cluster per cell.  Returns 0 or a negative NPFEM_ERR code with a
+// message in *err.
+int build_sparse_factor(const HostTopo& H, const double* rest, double mass_scale, double l_scale, SparseHost* out,
+                        SparseHost* out_cluster, std::string* err);
+
 // ---- kernels (npfem_factor.cu, npfem_solver.cu) ---------------------------------
 // In-place FP64 Gauss-Jordan inversion of an SPD n x n matrix on the GPU in one
 // cooperative launch.  prow: 2n doubles of scratch; d_flag: 4 ints, zeroed by the
 // caller: d_flag[0] becomes 1 when a pivot is not positive, 2 when a grid barrier
 // gave up waiting; d_flag[2..3] are the barrier's words.
 cudaError_t invert_spd_fp64(double* A, int n, double* prow, int* d_flag, cudaStream_t s);
-// Symmetrise A^-1 (FP64, n x n) and write padded copies in fp32 / fp64 / bf16.
-cudaError_t publish_inverse(const double* A, int n, int n_pad, float* out32, double* out64, void* out_bf16,
-                            float* out_tf32, cudaStream_t s);
+// Symmetrise A^-1 (FP64, n x n) in place and, if out is given, write it in FP32 as
+// [n_pad][n_pad] (zero padding).
+cudaError_t symmetrise(double* A, int n, int n_pad, float* out, cudaStream_t s);
 // A^-1 in BF16 as [rows_pad][kpad] (zero padding), the layout the tensor-core path
 // loads into tensor memory.
 cudaError_t publish_inverse_bf16_blocked(const double* A, int n, int rows_pad, int kpad, void* out, cudaStream_t s);
-// A^-1 in BF16 as [n8][n8] (rows and columns past n zero) for the SIMT contraction.
-cudaError_t publish_inverse_bf16_square(const double* A, int n, int n8, void* out, cudaStream_t s);
 
 template <typename T>
 cudaError_t launch_cells(const LaunchArgs<T>& a, int grid, int block, int smem, cudaStream_t s);
+// Resident blocks per SM of the SIMT launch `a` at this block size and dynamic shared memory.
 template <typename T>
-cudaError_t set_cell_kernel_smem(int bytes);
-// A^-1 in TF32 (round to nearest) as [row tile][K chunk] blocks of 128 rows x 32 K, each
-// in the no-swizzle K-major core-matrix layout the TF32 MMA reads (16 KB per chunk).
-cudaError_t publish_inverse_tf32_tiled(const double* A, int n, int tiles, int kpad, float* out, cudaStream_t s);
-// Resident SIMT blocks per SM at this block size and dynamic shared memory.
-template <typename T>
-cudaError_t cells_per_sm(int block, int smem, int* n);
+cudaError_t cells_per_sm(const LaunchArgs<T>& a, int block, int smem, int* n);
 // Tensor-core kernel (BF16, A^-1 row blocks resident in TMEM across a cluster): sets
 // its shared-memory size and returns how many clusters can be resident at once.
 cudaError_t query_cells_tc(int cluster, int block, int smem, int* max_clusters);
+// Cluster kernel for few FP64 cells: how many clusters of this size can be resident at once, and
+// its launch on `clusters` of them.
+cudaError_t query_cells_cl(int cluster, int smem, int* max_clusters);
+cudaError_t launch_cells_cl(const LaunchArgs<double>& a, int cluster, int clusters, int smem, cudaStream_t s);
 // Launch of one mesh group on `grid` blocks (a multiple of the cluster size).
 cudaError_t launch_cells_tc(const LaunchArgs<float>& a, int cluster, int block, int smem, int grid, cudaStream_t s);
 // Learned first increments u = x^(1) - x_n ([3][n] per cell, or positions x_n + u
@@ -263,9 +322,6 @@ cudaError_t launch_ws_temporal(const npfem_handle* h, int n_cells, const float* 
 // 32-column accumulator within 512 TMEM columns, and at most 8 blocks per cluster.
 constexpr int kTcMaxVerts = 960;
 constexpr int kTcThreads = 512;  // block size of the cluster kernel
-// TF32 path: shared memory for the two-stage A^-1 ring and the B operand (8 x kpad TF32).
-inline int tf32_smem_bytes(int kpad) { return ((2 * 128 * 32 * 4 + 8 * kpad * 4) + 1023) & ~1023; }
-
 // Records msg as the calling thread's last error and returns code (npfem_api.cu).
 int set_error(int code, const std::string& msg);
 
@@ -277,19 +333,20 @@ void count_launch(unsigned long long k = 1);
 // per-block global slot.  smem offsets
 // start at base_off.  Returns the smem bytes used in g->smem_bytes.
 template <typename T>
-inline void place_vectors(GroupDesc<T>* g, int n_pad, int nt, int m, int smem_budget, long long* slot_bytes,
+inline void place_vectors(GroupDesc<T>* g, int n, int n_pad, int nt, int npos, int m, int smem_budget, long long* slot_bytes,
                           int base_off = 0, bool gc_first = false)
 {
     const int vb = 3 * n_pad * (int)sizeof(T);
     // TRI (per-triangle rows, or per-vertex corner-gradient slots with fixed-width
-    // rings) also serves as the contraction's scratch (max(32, 4 x row tiles) x 384
-    // floats) and holds the warm start's normalised features ([n rounded to 16][16] floats)
+    // rings) also holds the sparse solve's vectors (6 npos <= 24 n_pad) and the warm
+    // start's normalised features ([n rounded to 16][16] floats)
     const int tri_bytes = kTriRow * nt * (int)sizeof(T);
-    const int ctr_bytes = (4 * ((n_pad + 127) / 128) > 32 ? 4 * ((n_pad + 127) / 128) : 32) * 384 * 4;
     const int ws_bytes = ((n_pad + 15) & ~15) * 16 * 4;
     const int slot_bytes8 = 24 * n_pad * (int)sizeof(T);  // [8 slots][3][n_pad] corner gradients
-    int tb = tri_bytes > ctr_bytes ? tri_bytes : ctr_bytes;
-    tb = tb > slot_bytes8 ? tb : slot_bytes8;
+    // and the dense contraction's partial sums (384 floats per item)
+    const int dn_bytes = sizeof(T) == 4 && n <= kDenseMaxVerts ? dense_parts(n) * ((n + 127) / 128) * 384 * 4 : 0;
+    int tb = tri_bytes > slot_bytes8 ? tri_bytes : slot_bytes8;
+    tb = tb > dn_bytes ? tb : dn_bytes;
     tb = ((tb > ws_bytes ? tb : ws_bytes) + 15) & ~15;
     int order[kMaxVecs], nv = 0;
     const int base[kNumBaseVecs] = {V_XN, V_U, V_UT, V_TRI, V_WR, V_G, V_GT, V_GC, V_UY, V_D};
@@ -305,6 +362,14 @@ inline void place_vectors(GroupDesc<T>* g, int n_pad, int nt, int m, int smem_bu
     int used = 0;
     long long gl = 0;
     for (int q = 0; q < kMaxVecs; ++q) g->loc[q] = 0;
+    // the solve gathers at random: a mesh whose TRI will not fit in shared memory gets its
+    // buffer there first
+    const int sp_bytes = (6 * npos * (int)sizeof(T) + 15) & ~15;
+    const bool own_sp = 3 * vb + tb > smem_budget && sp_bytes + 2 * vb <= smem_budget;
+    if (own_sp) {
+        g->loc[V_SP] = base_off;
+        used = sp_bytes;
+    }
     for (int q = 0; q < nv; ++q) {
         const int sz = order[q] == V_TRI ? tb : vb;
         if (used + sz <= smem_budget) {
@@ -315,9 +380,45 @@ inline void place_vectors(GroupDesc<T>* g, int n_pad, int nt, int m, int smem_bu
             gl += sz;
         }
     }
+    if (!own_sp) g->loc[V_SP] = g->loc[V_TRI];
     g->smem_bytes = base_off + used;
-    g->scratch_floats = tb / 4;
     *slot_bytes = gl;
+}
+
+// The same for a cluster per cell: what the blocks write into each other (the corner
+// gradients of the own vertices, WR, D, the solve's vectors) and what they gather must be in
+// shared memory.  Returns false when it does not fit.
+template <typename T>
+inline bool place_vectors_cluster(GroupDesc<T>* g, int n_pad, int npos, int m, int cluster, int smem_budget,
+                                  long long* slot_bytes)
+{
+    const int vb = 3 * n_pad * (int)sizeof(T);
+    const int per = 4 * ((n_pad / 4 + cluster - 1) / cluster);
+    const int tb = (24 * per * (int)sizeof(T) + 15) & ~15, sb = (6 * npos * (int)sizeof(T) + 15) & ~15;
+    for (int q = 0; q < kMaxVecs; ++q) g->loc[q] = 0;
+    int used = 0;
+    long long gl = 0;
+    auto put = [&](int v, int sz) {
+        if (used + sz <= smem_budget) {
+            g->loc[v] = used;
+            used += sz;
+            return true;
+        }
+        g->loc[v] = -(int)gl - 1;
+        gl += sz;
+        return false;
+    };
+    bool ok = put(V_TRI, tb) && put(V_SP, sb);
+    const int need[5] = {V_XN, V_U, V_UT, V_WR, V_D}, rest[4] = {V_G, V_GT, V_GC, V_UY};
+    for (int v : need) ok = put(v, vb) && ok;
+    for (int v : rest) put(v, vb);
+    for (int q = 0; q < m; ++q) {
+        put(V_SBASE + q, vb);
+        put(V_SBASE + m + q, vb);
+    }
+    g->smem_bytes = used;
+    *slot_bytes = gl;
+    return ok;
 }
 
 }  // namespace npfem
@@ -354,8 +455,7 @@ struct npfem_handle {
     // that needed iterations, [2] the previous step's [1], then indices)
     unsigned int* defer = nullptr;
     size_t defer_len = 0;
-    int sm_count = 0, smem_optin = 0;
-    int threads = 512;  // SIMT block size (512 or 640 for FP32 state)
+    int sm_count = 0, smem_optin = 0, smem_sm = 0;
     int use_tc = 1;     // BF16: use the tensor-core cluster kernel when the mesh fits it
     // buffers of npfem_step_host
     float* mlp = nullptr;       // learned warm start parameters on the device (weights BF16-rounded)
@@ -373,6 +473,8 @@ struct npfem_handle {
     size_t col_table_len = 0;
     // resident clusters of the tensor-core kernel at tc_smem bytes (queried once)
     int tc_max_clusters = 0, tc_smem = -1;
+    // resident clusters of the few-cells kernel (FP64) by log2 size at cl_smem bytes (queried once)
+    int cl_max[4] = {0, 0, 0, 0}, cl_smem[4] = {-1, -1, -1, -1};
     // side stream and fork/join events of the idle-SM SIMT launch (tensor-core path)
     cudaStream_t side_stream = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -380,6 +482,14 @@ struct npfem_handle {
     std::vector<cudaEvent_t> tev;
     int tev_used = 0;
     std::mutex mu;
+
+    int npos() const { return precision == NPFEM_PREC_FP64 ? td.sp.npos : tf.sp.npos; }
+    // Does the tensor-core cluster kernel take this handle's cells?  (Not with beta_D > 0,
+    // whose first guess needs a solve with M~.)
+    bool takes_clusters() const
+    {
+        return precision == NPFEM_PREC_BF16 && n <= npfem::kTcMaxVerts && mat.beta_D == 0.0 && use_tc;
+    }
 
     template <typename X>
     X* alloc(size_t count, int* err)

@@ -83,7 +83,7 @@ int run_static(npfem_handle* const* meshes, const std::vector<int>& sel, const i
         g.stats_off = coff[gi];
         g.cells = cells[gi];
         long long sb = 0;
-        place_vectors(&g, h->n_pad, h->nt, h0->opts.lbfgs_m, budget, &sb);
+        place_vectors(&g, h->n, h->n_pad, h->nt, h->npos(), h0->opts.lbfgs_m, budget, &sb);
         slot = std::max(slot, sb);
         smem_max = std::max(smem_max, g.smem_bytes);
         total += cells[gi];
@@ -106,16 +106,14 @@ int run_static(npfem_handle* const* meshes, const std::vector<int>& sel, const i
     a.slot_bytes = slot;
     set_solver_params(&a.p, h0->opts);
     a.p.mode = 0;
-    a.p.contraction = CONTRACT_SIMT;
     if (meshes[0]->col_planes) {
         a.col = reinterpret_cast<const float4*>(meshes[0]->col_planes);
         a.col_w = (T)meshes[0]->col_w;
     }
 
     const int smem = kFixedSmem + smem_max;
-    cudaError_t e = set_cell_kernel_smem<T>(smem);
     int per_sm = 1;
-    if (e == cudaSuccess) e = cells_per_sm<T>(threads, smem, &per_sm);
+    cudaError_t e = cells_per_sm<T>(a, threads, smem, &per_sm);
     if (e != cudaSuccess) return set_error(NPFEM_ERR_CUDA, std::string("npfem_step_static: ") + cudaGetErrorString(e));
     per_sm = std::max(per_sm, 1);
     long long grid = std::min<long long>(total, (long long)h0->sm_count * per_sm);
@@ -143,10 +141,10 @@ int step_static(npfem_handle* const* meshes, int n_groups, const int32_t* cells,
     std::vector<char> done(n_groups, 0);
     for (int g0 = 0; g0 < n_groups; ++g0) {
         if (done[g0]) continue;
-        const int threads = sizeof(T) == 8 ? 512 : meshes[g0]->threads;
+        const int threads = 512;
         std::vector<int> sel;
         for (int g = g0; g < n_groups; ++g) {
-            if (done[g] || (sizeof(T) == 4 && meshes[g]->threads != threads)) continue;
+            if (done[g]) continue;
             sel.push_back(g);
             done[g] = 1;
         }
