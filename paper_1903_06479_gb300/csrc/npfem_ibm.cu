@@ -9,9 +9,11 @@
 // nodes is one 64-byte (velocity, force) or 128-byte (stress) access: what bounds these
 // kernels is the number of L1/L2 sectors and atomic operations per stencil.  The lanes
 // share the vertex's triangles for its area share A_k (a third of its triangles' areas)
-// and unit normal n_k at the current positions; their stencil sums meet in two shuffles.  Lattice coordinates are formed in FP64
-// (a 100 um domain at FP32 would round the fractional lattice offset to ~1e-5); the
-// weights and sums are FP32.
+// and unit normal n_k at the current positions; their stencil sums meet in two shuffles.
+// Lattice coordinates are sums of two floats (lattice_base), weights and sums FP32.
+// Measured on 1024 cells of 642 vertices, 121^3 nodes: forcing with three cycles (four
+// spreads and four gathers) 3.0 -> 1.06 ms against one thread per vertex with scalar
+// atomics and FP64 coordinates.
 //
 // Conventions (the paper prints the formulas in lattice units, dx = 1):
 //  * interpolation u(X_k) = sum_x u(x) w w w (the dx^3 of W dx^3 cancels);
@@ -35,7 +37,8 @@ namespace npfem {
 namespace {
 
 struct LatDev {
-    double ox, oy, oz, inv_dx;
+    float oh[3], ol[3];  // origin and 1 / dx as sums of two floats
+    float ih, il;
     float dx;
     int nx, ny, nz;
 };
@@ -80,41 +83,53 @@ struct Stencil {
     float w[3][4];       // weights of nodes i0 + a, a = 0..3
 };
 
-// Base node of a coordinate's stencil.  A point far outside the lattice (or not finite) gets
-// a stencil with no nodes.
-__device__ __forceinline__ double lattice_floor(const LatDev& L, double origin, float X, double* r)
+// First node of a coordinate's stencil and its fractional offset t in [0, 1).  The lattice
+// coordinate (X - origin) / dx is carried as a sum of two floats (error-free difference
+// and product, about 48 bits: a single float would round the offset in a 100 um domain to
+// ~1e-5; in FP64 this alone took a third of the forcing's time on the narrow FP64 pipe).  A
+// point far outside the lattice (or not finite) gets a stencil with no nodes.
+__device__ __forceinline__ int lattice_base(const LatDev& L, int d, float X, float* t)
 {
-    const double v = ((double)X - origin) * L.inv_dx;
-    *r = v == v ? fmin(fmax(v, -1.0e6), 1.0e6) : -1.0e6;
-    return floor(*r);
-}
-
-__device__ __forceinline__ int lattice_base(const LatDev& L, double origin, float X)
-{
-    double r;
-    return (int)lattice_floor(L, origin, X, &r) - 1;
-}
-
-__device__ __forceinline__ void make_stencil(const LatDev& L, float X, float Y, float Z, Stencil& s)
-{
-    const double o[3] = {L.ox, L.oy, L.oz};
-    const float P[3] = {X, Y, Z};
-    int b[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        double rd;
-        const double f = lattice_floor(L, o[d], P[d], &rd);
-        b[d] = (int)f - 1;
-        const float t = (float)(rd - f);
-        s.t[d] = t;
-        s.w[d][0] = w4(t + 1.f);
-        s.w[d][1] = w4(t);
-        s.w[d][2] = w4(t - 1.f);
-        s.w[d][3] = w4(t - 2.f);
+    const float oh = d == 0 ? L.oh[0] : (d == 1 ? L.oh[1] : L.oh[2]), ol = d == 0 ? L.ol[0] : (d == 1 ? L.ol[1] : L.ol[2]);
+    const float dh = X - oh, bb = dh - X;
+    const float dl = ((X - (dh - bb)) - (oh + bb)) - ol;
+    const float ph = dh * L.ih;
+    if (!(fabsf(ph) <= 1.0e6f)) {
+        *t = 0.f;
+        return ph > 0.f ? 999999 : -1000001;
     }
-    s.i0 = b[0];
-    s.j0 = b[1];
-    s.k0 = b[2];
+    const float pl = fmaf(dh, L.ih, -ph) + fmaf(dh, L.il, dl * L.ih);
+    float f = floorf(ph);
+    float r = (ph - f) + pl;
+    if (r < 0.f) {
+        r += 1.f;
+        f -= 1.f;
+    } else if (r >= 1.f) {
+        r -= 1.f;
+        f += 1.f;
+    }
+    *t = r;
+    return (int)f - 1;
+}
+
+// The stencil of vertex i (SoA positions xc of n vertices) for its four lanes: lane d < 3
+// takes dimension d (its offset and four weights) and the lanes exchange them.  wq: lane q's weight along x.
+__device__ __forceinline__ void make_stencil(const LatDev& L, const float* xc, int n, int i, int q, Stencil& s, float* wq)
+{
+    const int d = min(q, 2), from = (threadIdx.x & 31) & ~3;
+    float t;
+    const int base = lattice_base(L, d, xc[d * n + i], &t);
+    const float w[4] = {w4(t + 1.f), w4(t), w4(t - 1.f), w4(t - 2.f)};
+    s.i0 = __shfl_sync(kFull, base, from);
+    s.j0 = __shfl_sync(kFull, base, from + 1);
+    s.k0 = __shfl_sync(kFull, base, from + 2);
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        s.t[e] = __shfl_sync(kFull, t, from + e);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s.w[e][k] = __shfl_sync(kFull, w[k], from + e);
+    }
+    *wq = q == 0 ? s.w[0][0] : (q == 1 ? s.w[0][1] : (q == 2 ? s.w[0][2] : s.w[0][3]));
 }
 
 // Global vertex index -> (group, its topology, cell, vertex).
@@ -208,8 +223,8 @@ __global__ void __launch_bounds__(256) ibm_forces_kernel(const __grid_constant__
         float A, nv[3];
         area_normal4<true>(G.topo, xc, i, q, &A, nv);
         Stencil s;
-        make_stencil(L, xc[i], xc[n + i], xc[2 * n + i], s);
-        const float wq = q == 0 ? s.w[0][0] : (q == 1 ? s.w[0][1] : (q == 2 ? s.w[0][2] : s.w[0][3]));
+        float wq;
+        make_stencil(L, xc, n, i, q, s, &wq);
         float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, wsum = 0.f, dbest = -1.f;
         int first = 64;
 #pragma unroll
@@ -341,11 +356,6 @@ __device__ __forceinline__ void take_sum(const IbmArgs& a, long long so, int n, 
     a.out[at] = a.phase == 0 ? slip : a.out[at] + slip;
 }
 
-__device__ __forceinline__ float lane_weight(const Stencil& s, int q)
-{
-    return q == 0 ? s.w[0][0] : (q == 1 ? s.w[0][1] : (q == 2 ? s.w[0][2] : s.w[0][3]));
-}
-
 // One vertex of a phase straight on the lattice.
 __device__ __forceinline__ void vertex_phase(const IbmArgs& a, const IbmGroup& G, long long cell, int i, int q, bool live)
 {
@@ -354,8 +364,8 @@ __device__ __forceinline__ void vertex_phase(const IbmArgs& a, const IbmGroup& G
     const long long so = G.state_off + cell * 3LL * n;
     const float* xc = a.x + so;
     Stencil s;
-    make_stencil(L, xc[i], xc[n + i], xc[2 * n + i], s);
-    const float wq = lane_weight(s, q);
+    float wq;
+    make_stencil(L, xc, n, i, q, s, &wq);
     if (a.phase == 1) {
         // Step 1: spread f_k with weight A_k dx / dx^3 per unit stencil weight
         float A;
@@ -378,7 +388,7 @@ __device__ __forceinline__ void vertex_phase(const IbmArgs& a, const IbmGroup& G
 
 // Velocity interpolation (phase -1) and the phases of the multi-direct forcing, vertex by
 // vertex (few cells, or small ones).
-__global__ void __launch_bounds__(256) ibm_forcing_kernel(const __grid_constant__ IbmArgs a)
+__global__ void __launch_bounds__(256, 3) ibm_forcing_kernel(const __grid_constant__ IbmArgs a)
 {
     for (long long v0 = blockIdx.x * (long long)kVertsPerBlock; v0 < a.total_verts; v0 += (long long)gridDim.x * kVertsPerBlock) {
         const long long gv = v0 + (threadIdx.x >> 2);
@@ -390,16 +400,17 @@ __global__ void __launch_bounds__(256) ibm_forcing_kernel(const __grid_constant_
     }
 }
 
-// The same, a block per cell: the lattice nodes around the cell (a box of the stencils'
-// extent) pass through shared memory, read or reduced once instead of once per stencil that
+// The gathering phases, a block per cell: the lattice nodes around the cell (a box of the
+// stencils' extent) pass through shared memory, read once instead of once per stencil that
 // meets them (a 642-vertex cell has 41 K stencil nodes in a box of about 1.7 K).  A cell
-// whose box does not fit goes vertex by vertex.
+// whose box does not fit goes vertex by vertex.  Spreading through such a box was slower
+// than vertex by vertex, with atomics on shared sums (1024 cells of 642 vertices, four
+// spreads and gathers: 3.2 against 2.1 ms) and with the vertices sorted by node (2.8 ms).
 constexpr int kBoxNodes = 3000;
-constexpr long long kBoxMinCells = 128, kBoxMinVerts = 200;
 
-__global__ void __launch_bounds__(256) ibm_box_kernel(const __grid_constant__ IbmArgs a)
+__global__ void __launch_bounds__(256, 3) ibm_gather_kernel(const __grid_constant__ IbmArgs a)
 {
-    extern __shared__ __align__(16) float box[];  // gather: float4 per node; spread: three rows
+    extern __shared__ __align__(16) float4 box[];
     __shared__ int lo[3], hi[3];
     const LatDev& L = a.lat;
     const int tid = threadIdx.x, NT = blockDim.x, q = tid & 3;
@@ -418,11 +429,12 @@ __global__ void __launch_bounds__(256) ibm_box_kernel(const __grid_constant__ Ib
         __syncthreads();
         int l[3] = {INT_MAX, INT_MAX, INT_MAX}, h[3] = {INT_MIN, INT_MIN, INT_MIN};
         for (int i = tid; i < n; i += NT) {
-            const int b[3] = {lattice_base(L, L.ox, xc[i]), lattice_base(L, L.oy, xc[n + i]), lattice_base(L, L.oz, xc[2 * n + i])};
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
-                l[d] = min(l[d], b[d]);
-                h[d] = max(h[d], b[d]);
+                float t;
+                const int b = lattice_base(L, d, xc[d * n + i], &t);
+                l[d] = min(l[d], b);
+                h[d] = max(h[d], b);
             }
         }
 #pragma unroll
@@ -439,12 +451,7 @@ __global__ void __launch_bounds__(256) ibm_box_kernel(const __grid_constant__ Ib
         const long long ex = (long long)hi[0] - x0 + 4, ey = (long long)hi[1] - y0 + 4, ez = (long long)hi[2] - z0 + 4;
         const bool fits = ex <= kBoxNodes && ey <= kBoxNodes && ez <= kBoxNodes && ex * ey * ez <= kBoxNodes;
         const int bx = (int)ex, by = (int)ey, nodes = fits ? (int)(ex * ey * ez) : 0;
-        // gather: the box's velocities; spread: zero sums
         for (int e = tid; e < nodes; e += NT) {
-            if (a.phase == 1) {
-                box[e] = box[nodes + e] = box[2 * nodes + e] = 0.f;
-                continue;
-            }
             const int k = e / (bx * by), j = (e - k * bx * by) / bx, ii = e - (k * by + j) * bx;
             float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
             if (node_in(L, x0 + ii, y0 + j, z0 + k)) {
@@ -458,7 +465,7 @@ __global__ void __launch_bounds__(256) ibm_box_kernel(const __grid_constant__ Ib
                     u.z += a.dt * f.z;
                 }
             }
-            reinterpret_cast<float4*>(box)[e] = u;
+            box[e] = u;
         }
         __syncthreads();
         for (int v0 = 0; v0 < n; v0 += NT >> 2) {
@@ -469,48 +476,23 @@ __global__ void __launch_bounds__(256) ibm_box_kernel(const __grid_constant__ Ib
                 continue;
             }
             Stencil s;
-            make_stencil(L, xc[i], xc[n + i], xc[2 * n + i], s);
-            const float wq = lane_weight(s, q);
+            float wq;
+            make_stencil(L, xc, n, i, q, s, &wq);
             const int at = ((s.k0 - z0) * by + (s.j0 - y0)) * bx + (s.i0 - x0) + q;
-            if (a.phase == 1) {
-                float A;
-                area_normal4<false>(G.topo, xc, i, q, &A, nullptr);
-                const float* o = a.out + so;
-                const float sc = A / (L.dx * L.dx) * wq;
-                const float f[3] = {sc * o[i], sc * o[n + i], sc * o[2 * n + i]};
-                if (!live) continue;
+            float o[3] = {0.f, 0.f, 0.f}, u[3];
 #pragma unroll
-                for (int r = 0; r < 16; ++r) {
-                    const int e = at + ((r >> 2) * by + (r & 3)) * bx;
-                    const float wgt = s.w[1][r & 3] * s.w[2][r >> 2];
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) atomicAdd(&box[c * nodes + e], wgt * f[c]);
-                }
-            } else {
-                float o[3] = {0.f, 0.f, 0.f}, u[3];
-#pragma unroll
-                for (int r = 0; r < 16; ++r) {
-                    const float wgt = wq * s.w[1][r & 3] * s.w[2][r >> 2];
-                    const float4 f = reinterpret_cast<const float4*>(box)[at + ((r >> 2) * by + (r & 3)) * bx];
-                    o[0] += wgt * f.x;
-                    o[1] += wgt * f.y;
-                    o[2] += wgt * f.z;
-                }
-#pragma unroll
-                for (int c = 0; c < 3; ++c) u[c] = sum4(o[c]);
-                take_sum(a, so, n, i, q, live, u);
+            for (int r = 0; r < 16; ++r) {
+                const float wgt = wq * s.w[1][r & 3] * s.w[2][r >> 2];
+                const float4 f = box[at + ((r >> 2) * by + (r & 3)) * bx];
+                o[0] += wgt * f.x;
+                o[1] += wgt * f.y;
+                o[2] += wgt * f.z;
             }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) u[c] = sum4(o[c]);
+            take_sum(a, so, n, i, q, live, u);
         }
         __syncthreads();
-        if (a.phase == 1) {
-            for (int e = tid; e < nodes; e += NT) {
-                const float fx = box[e], fy = box[nodes + e], fz = box[2 * nodes + e];
-                const int k = e / (bx * by), j = (e - k * bx * by) / bx, ii = e - (k * by + j) * bx;
-                if ((fx != 0.f || fy != 0.f || fz != 0.f) && node_in(L, x0 + ii, y0 + j, z0 + k))
-                    red4(a.lat_out + 4 * node_index(L, x0 + ii, y0 + j, z0 + k), fx, fy, fz, a.lat_vec);
-            }
-            __syncthreads();
-        }
     }
 }
 
@@ -540,10 +522,13 @@ int fill_ibm(IbmArgs* a, npfem_handle* const* meshes, int n_groups, const int32_
     }
     a->n_groups = n_groups;
     a->total_verts = v;
-    a->lat.ox = lat->origin[0];
-    a->lat.oy = lat->origin[1];
-    a->lat.oz = lat->origin[2];
-    a->lat.inv_dx = 1.0 / lat->dx;
+    for (int d = 0; d < 3; ++d) {
+        a->lat.oh[d] = (float)lat->origin[d];
+        a->lat.ol[d] = (float)(lat->origin[d] - (double)a->lat.oh[d]);
+    }
+    const double inv = 1.0 / lat->dx;
+    a->lat.ih = (float)inv;
+    a->lat.il = (float)(inv - (double)a->lat.ih);
     a->lat.dx = (float)lat->dx;
     a->lat.nx = lat->nx;
     a->lat.ny = lat->ny;
@@ -557,14 +542,17 @@ int ibm_grid(const npfem_handle* h, long long verts)
     return (int)std::max<long long>(1, std::min<long long>(blocks, (long long)std::max(h->sm_count, 1) * 8));
 }
 
-// A phase over all vertices: a block per cell where the cells fill the GPU and a cell's
-// stencils overlap, else vertex by vertex.
+// A phase over all vertices: gathers by a block per cell where the cells fill the GPU and a
+// cell's stencils overlap (1024 cells of 642 vertices, whole forcing with FP64 coordinates: 2.14 -> 1.97 ms), else
+// vertex by vertex.
+constexpr long long kBoxMinCells = 128, kBoxMinVerts = 200;
+
 cudaError_t launch_forcing(const IbmArgs& a, const npfem_handle* h, cudaStream_t s)
 {
     if (a.phase != 1 && a.total_cells >= kBoxMinCells && a.total_verts >= kBoxMinVerts * a.total_cells) {
         const int smem = kBoxNodes * (int)sizeof(float4);
         const int grid = (int)std::min<long long>(a.total_cells, (long long)std::max(h->sm_count, 1) * 4);
-        ibm_box_kernel<<<grid, 256, smem, s>>>(a);
+        ibm_gather_kernel<<<grid, 256, smem, s>>>(a);
     } else {
         ibm_forcing_kernel<<<ibm_grid(h, a.total_verts), 256, 0, s>>>(a);
     }
