@@ -272,7 +272,7 @@ int check_opts(const npfem_opts* o)
 int simt_threads(const npfem_handle* h, int n, long long cells)
 {
     const long long sms = h->sm_count;
-    if (h->precision == NPFEM_PREC_FP64) return cells > sms ? 128 : 512;
+    if (h->precision == NPFEM_PREC_FP64) return cells > sms || n <= 320 ? 128 : 512;
     if (n <= 384 && cells > 2 * sms) return 128;
     if (n <= 1200 && cells > sms) return 256;
     return 512;
@@ -284,28 +284,28 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
               const T* u0 = nullptr, const long long* state_offs = nullptr, const long long* stats_offs = nullptr,
               int threads = 0, const T* hist_in = nullptr, T* hist_out = nullptr, long long pos_stride = 0,
               unsigned int* defer = nullptr, int hist_ext = 0, T* carry = nullptr,
-              const long long* carry_offs = nullptr)
+              const long long* carry_offs = nullptr, npfem_handle* lead = nullptr)
 {
-    npfem_handle* h0 = meshes[0];
+    // options, collision planes, counters and scratch are the call's first handle's
+    npfem_handle* h0 = lead ? lead : meshes[0];
     LaunchArgs<T> a;
     memset(&a, 0, sizeof(a));
     long long total = 0, state = 0, slot = 0;
     int smem_max = 0;
-    if (threads <= 0) {
-        int n_max = 0;
-        long long all = 0;
-        for (int gi = 0; gi < n_groups; ++gi) {
-            n_max = std::max(n_max, meshes[gi]->n);
-            all += cells[gi];
-        }
-        threads = simt_threads(h0, n_max, all);
+    int n_max = 0;
+    long long all = 0;
+    for (int gi = 0; gi < n_groups; ++gi) {
+        n_max = std::max(n_max, meshes[gi]->n);
+        all += cells[gi];
     }
+    if (threads <= 0) threads = simt_threads(h0, n_max, all);
     // 512 / threads blocks share an SM's shared memory (1 KB of it per block is the system's)
     const int budget = (threads < 512 ? h0->smem_sm / (512 / threads) : h0->smem_optin) - kFixedSmem - 1024;
     for (int gi = 0; gi < n_groups; ++gi) {
         npfem_handle* h = meshes[gi];
         GroupDesc<T>& g = a.g[gi];
         g.topo = *reinterpret_cast<const TopoDev<T>*>(sizeof(T) == 4 ? (const void*)&h->tf : (const void*)&h->td);
+        if (h->n > kDenseVerts && all > kDenseCells) g.topo.ainv = nullptr;  // the sparse factor
         g.cell_begin = total;
         g.state_off = state_offs ? state_offs[gi] : state;
         g.stats_off = stats_offs ? stats_offs[gi] : total;
@@ -373,10 +373,10 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
 // with beta_D > 0, one-rings past the fixed width or meshes too large).
 int run_cells_cluster(npfem_handle* const* meshes, int n_groups, const int32_t* cells, double* x, double* v, const double* f,
                       npfem_cell_stats* stats, cudaStream_t stream, const long long* state_offs, const long long* stats_offs,
-                      const double* hist_in, double* hist_out, double* carry, const long long* carry_offs, bool* done)
+                      const double* hist_in, double* hist_out, double* carry, const long long* carry_offs,
+                      npfem_handle* h0, bool* done)
 {
     *done = false;
-    npfem_handle* h0 = meshes[0];
     long long total = 0;
     for (int gi = 0; gi < n_groups; ++gi) {
         const npfem_handle* h = meshes[gi];
@@ -390,7 +390,7 @@ int run_cells_cluster(npfem_handle* const* meshes, int n_groups, const int32_t* 
         LaunchArgs<double> a;
         memset(&a, 0, sizeof(a));
         long long at = 0, slot = 0;
-        int smem_max = 0;
+        int smem_max = 0, nt_max = 0;
         bool fits = true;
         for (int gi = 0; gi < n_groups; ++gi) {
             npfem_handle* h = meshes[gi];
@@ -407,13 +407,19 @@ int run_cells_cluster(npfem_handle* const* meshes, int n_groups, const int32_t* 
                                          h0->smem_optin - kFixedSmem - 1024, &sb) && fits;
             slot = std::max(slot, sb);
             smem_max = std::max(smem_max, g.smem_bytes);
+            nt_max = std::max(nt_max, h->nt);
             at += cells[gi];
         }
         if (!fits) continue;
+        // a thread per two to four triangles of a block's share: every further warp runs the
+        // reductions' FP64 shuffles and merges without data
+        int block = 128;
+        while (block < 512 && 4 * block < nt_max / C) block *= 2;
         const int smem = kFixedSmem + smem_max;
-        if (h0->cl_smem[lg] != smem) {
-            NPFEM_CUDA(query_cells_cl(C, smem, &h0->cl_max[lg]));
-            h0->cl_smem[lg] = smem;
+        const int key = smem + (block << 20);
+        if (h0->cl_smem[lg] != key) {
+            NPFEM_CUDA(query_cells_cl(C, block, smem, &h0->cl_max[lg]));
+            h0->cl_smem[lg] = key;
         }
         if (h0->cl_max[lg] < total) continue;
         a.n_groups = n_groups;
@@ -447,7 +453,7 @@ int run_cells_cluster(npfem_handle* const* meshes, int n_groups, const int32_t* 
             }
             a.scratch = h0->scratch;
         }
-        NPFEM_CUDA(launch_cells_cl(a, C, (int)total, smem, stream));
+        NPFEM_CUDA(launch_cells_cl(a, C, (int)total, block, smem, stream));
         *done = true;
         return 0;
     }
@@ -519,6 +525,7 @@ int run_cells_tc(npfem_handle* h, int cells, float* x, float* v, const float* f,
     if (cells <= grid || h->opts.fill_idle_sms == 0) helper = 0;
     if (helper > 0) {
         b = a;
+        if (h->n > kDenseVerts) b.g[0].topo.ainv = nullptr;  // the sparse factor
         place_vectors(&b.g[0], h->n, h->n_pad, h->nt, h->npos(), h->opts.lbfgs_m, h->smem_optin - kFixedSmem - 1024, &slot_b);
         b.p.cluster = 0;
         b.p.refine = 0;
@@ -640,15 +647,30 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
         }
     }
     // the other groups: with at most a cell per SM in all one launch, else each at its own
-    // block size, groups of one size together
+    // block size, groups of one size together.  A group with at most a cell per SM beside a
+    // larger population of meshes at least as fine joins that launch (alone it would take
+    // the time of a cell on an empty GPU).
+    const long long sms = meshes[0]->sm_count;
     long long left = 0;
-    for (int g = 0; g < n_groups; ++g)
-        if (!done[g]) left += cells_per_group[g];
+    npfem_handle* lead = nullptr;
+    for (int g = n_groups - 1; g >= 0; --g)
+        if (!done[g]) {
+            left += cells_per_group[g];
+            lead = meshes[g];
+        }
     std::vector<int> shape(n_groups, 512);
-    if (left > meshes[0]->sm_count)
-        for (int g = 0; g < n_groups; ++g) shape[g] = simt_threads(meshes[g], meshes[g]->n, cells_per_group[g]);
-    else if (n_groups == 1)
+    std::vector<char> dense(n_groups, 0);
+    if (left > sms) {
+        for (int g = 0; g < n_groups; ++g) {
+            int as = g;
+            for (int m = 0; m < n_groups && cells_per_group[g] <= sms; ++m)
+                if (!done[m] && cells_per_group[m] > sms && meshes[m]->n >= meshes[g]->n) as = m;
+            shape[g] = simt_threads(meshes[as], meshes[as]->n, cells_per_group[as]);
+            dense[g] = prec != NPFEM_PREC_FP64 && meshes[as]->n <= kDenseVerts;
+        }
+    } else if (n_groups == 1) {
         shape[0] = simt_threads(meshes[0], meshes[0]->n, left);
+    }
     for (int g0 = 0; g0 < n_groups; ++g0) {
         if (done[g0]) continue;
         const int threads = shape[g0];
@@ -656,8 +678,7 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
         std::vector<int32_t> cs;
         std::vector<long long> so, co, ko;
         for (int g = g0; g < n_groups; ++g) {
-            if (done[g] || shape[g] != threads || (left > meshes[0]->sm_count && !meshes[g]->tf.ainv != !meshes[g0]->tf.ainv))
-                continue;
+            if (done[g] || shape[g] != threads || dense[g] != dense[g0]) continue;
             hs.push_back(meshes[g]);
             cs.push_back(cells_per_group[g]);
             so.push_back(soff[g]);
@@ -670,7 +691,7 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
         if (prec == NPFEM_PREC_FP64) {
             rc = run_cells_cluster(hs.data(), (int)hs.size(), cs.data(), (double*)x, (double*)v, (const double*)f_ext,
                                    stats, s, so.data(), co.data(), (const double*)hist_in, (double*)hist_out,
-                                   (double*)carry, ko.data(), &clustered);
+                                   (double*)carry, ko.data(), lead, &clustered);
             if (rc) return rc;
         }
         if (clustered) continue;
@@ -678,12 +699,12 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
             rc = run_cells<double>(hs.data(), (int)hs.size(), cs.data(), (double*)x, (double*)v, (const double*)f_ext,
                                    nullptr, nullptr, nullptr, stats, 0, s, nullptr, so.data(), co.data(), threads,
                                    (const double*)hist_in, (double*)hist_out, 0, nullptr, 0, (double*)carry,
-                                   ko.data());
+                                   ko.data(), lead);
         else
             rc = run_cells<float>(hs.data(), (int)hs.size(), cs.data(), (float*)x, (float*)v, (const float*)f_ext,
                                   nullptr, nullptr, nullptr, stats, 0, s, u0, so.data(), co.data(), threads,
                                   (const float*)hist_in, (float*)hist_out, pos_stride, nullptr, hist_ext,
-                                  (float*)carry, ko.data());
+                                  (float*)carry, ko.data(), lead);
         if (rc) return rc;
     }
     return 0;

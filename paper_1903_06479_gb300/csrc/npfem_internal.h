@@ -250,10 +250,13 @@ struct SparseHost {
 constexpr int kSparseWarps = 16;     // warps a step's work is spread over
 constexpr int kSparseWarpsCluster = 64;  // the same for a cluster per cell
 constexpr int kSparseMaxIters = 10;  // iterations of a slice a warp keeps in flight (FP32)
-// Largest mesh whose FP32 solve applies the dense inverse.  At 642 vertices it reads 1.65 MB
-// from L2 in 48.5 K cycles, the sparse factor 0.47 MB in eleven steps in 41 K, and a
-// population takes the same time with either; at 1026 (4.2 MB, 111 K) the factor is faster.
-constexpr int kDenseMaxVerts = 700;
+// Meshes whose FP32 solve applies the dense inverse: all up to kDenseVerts (at 642 vertices
+// it reads 1.65 MB from L2 in 48.5 K cycles, the sparse factor 0.47 MB in eleven steps in
+// 41 K, and a population takes the same time with either: 1520 cells 1869 / 1726 us, 3001
+// cells of 258 2.38 / 2.99 ms), and up to kDenseMaxVerts in launches of at most kDenseCells
+// cells, which have the L2 to themselves (one cell of 786 vertices is 3 to 9 % faster with
+// the factor; 37 cells of 1026, 4.2 MB, 111 K cycles dense: 2.65 / 2.24 ms).
+constexpr int kDenseVerts = 700, kDenseMaxVerts = 1100, kDenseCells = 8;
 // Parts of the column range of every 128-row tile, items (tile, part) dealt to 16 warps in
 // turn: the number that minimises the busiest warp's columns (ceil(tiles P / 16) items of
 // ceil(n / P) columns) within max(32, 4 tiles) items.
@@ -304,8 +307,8 @@ cudaError_t cells_per_sm(const LaunchArgs<T>& a, int block, int smem, int* n);
 cudaError_t query_cells_tc(int cluster, int block, int smem, int* max_clusters);
 // Cluster kernel for few FP64 cells: how many clusters of this size can be resident at once, and
 // its launch on `clusters` of them.
-cudaError_t query_cells_cl(int cluster, int smem, int* max_clusters);
-cudaError_t launch_cells_cl(const LaunchArgs<double>& a, int cluster, int clusters, int smem, cudaStream_t s);
+cudaError_t query_cells_cl(int cluster, int block, int smem, int* max_clusters);
+cudaError_t launch_cells_cl(const LaunchArgs<double>& a, int cluster, int clusters, int block, int smem, cudaStream_t s);
 // Launch of one mesh group on `grid` blocks (a multiple of the cluster size).
 cudaError_t launch_cells_tc(const LaunchArgs<float>& a, int cluster, int block, int smem, int grid, cudaStream_t s);
 // Learned first increments u = x^(1) - x_n ([3][n] per cell, or positions x_n + u

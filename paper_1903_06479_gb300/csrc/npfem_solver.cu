@@ -82,23 +82,23 @@ cudaError_t launch_cells(const LaunchArgs<T>& a, int grid, int block, int smem, 
     return e;
 }
 
-cudaError_t query_cells_cl(int cluster, int smem, int* max_clusters)
+cudaError_t query_cells_cl(int cluster, int block, int smem, int* max_clusters)
 {
     const void* k = cell_kernel_cl_f64();
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = tc_config(cluster, 512, smem, cluster, nullptr, attr);
+    cudaLaunchConfig_t cfg = tc_config(cluster, block, smem, cluster, nullptr, attr);
     return cudaOccupancyMaxActiveClusters(max_clusters, k, &cfg);
 }
 
-cudaError_t launch_cells_cl(const LaunchArgs<double>& a, int cluster, int clusters, int smem, cudaStream_t s)
+cudaError_t launch_cells_cl(const LaunchArgs<double>& a, int cluster, int clusters, int block, int smem, cudaStream_t s)
 {
     const void* k = cell_kernel_cl_f64();
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = tc_config(cluster, 512, smem, cluster * clusters, s, attr);
+    cudaLaunchConfig_t cfg = tc_config(cluster, block, smem, cluster * clusters, s, attr);
     void* args[1] = {const_cast<LaunchArgs<double>*>(&a)};
     e = cudaLaunchKernelExC(&cfg, k, args);
     if (e == cudaSuccess) count_launch();

@@ -165,3 +165,37 @@ def test_forcing_cell_by_cell(N, dx):
     N.ibm_forcing([h], [cells], x, v, lat, u, DT, 1, fv, fl)
     torch.cuda.synchronize()
     assert bool(torch.isfinite(fv).all()) and bool(torch.isfinite(fl).all())
+
+
+def test_groups_of_several_block_sizes_share_options_and_planes(N):
+    """A call whose groups run in separate launches (by block size): every group takes the
+    options and the collision planes of the call's first handle, as in one launch."""
+    import torch
+    sizes, cells = (258, 1026), (310, 160)
+    hs, pops = [], []
+    for k, (n, c) in enumerate(zip(sizes, cells)):
+        rest, tris = W.discocyte(n)
+        # the second handle's own tolerance would stop it at the first iterate
+        hs.append(N.Handle(rest, tris, N.material(), N.default_opts(precision="fp32", tol=1e-6 if k == 0 else 1e3,
+                                                                    lbfgs_m=5 if k == 0 else 2), dt=DT))
+        pops.append(population32(n, c, seed=800 + n, forces="shear", noise_pN=0.5, box=40.0))
+    cat = lambda k: torch.tensor(np.concatenate([W.to_soa(p[k]).ravel() for p in pops]), dtype=torch.float32, device="cuda")
+    x, v, f = cat("x"), cat("v"), cat("f")
+    verts = sum(n * c for n, c in zip(sizes, cells))
+    planes = torch.zeros((verts, 4), device="cuda")
+    first = sizes[0] * cells[0]
+    # the second group's last cell: every vertex 0.01 um behind a plane normal to x
+    xl = W.to_soa(pops[1]["x"])[-1]
+    planes[verts - sizes[1]:, 0] = 1.0
+    planes[verts - sizes[1]:, 3] = torch.tensor(xl[0] - xl[0, 0] + 0.01, dtype=torch.float32, device="cuda")
+    hs[0].set_collisions(planes, 2000.0)
+    st = torch.zeros((sum(cells), 32), dtype=torch.uint8, device="cuda")
+    for _ in range(2):
+        N.step(hs, cells, x, v, f, DT, stats=st)
+    torch.cuda.synchronize()
+    st = st.cpu().numpy().view(N.CELL_STATS_DTYPE).reshape(-1)
+    assert (st["status"] == 0).all() and (st["residual"] <= 1e-6).all()
+    vx = v[3 * first:].view(cells[1], 3, sizes[1])[:, 0].mean(1).cpu().numpy()
+    # the push is w_col d h / m per step on every vertex, far above the noise's mean velocity
+    push = 2000.0 * 0.01 * DT / (94e3 / sizes[1])
+    assert vx[-1] > 0.5 * push and np.abs(vx[:-1]).max() < 0.2 * push
