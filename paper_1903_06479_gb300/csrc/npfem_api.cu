@@ -630,10 +630,12 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
                 // along a trajectory many cells are accepted at the first iterate: a SIMT
                 // launch on every SM (the clusters' idle SMs included) evaluates each cell
                 // there and finishes those, and the cluster kernel takes only the rest
+                // (one block of 512 threads per SM: its vectors fit in shared memory, so a
+                // trajectory's first pass does not grow the handle's scratch)
                 NPFEM_CUDA(cudaMemcpyAsync(hg->defer + 2, hg->defer + 1, sizeof(unsigned int), cudaMemcpyDeviceToDevice, s));
                 NPFEM_CUDA(cudaMemsetAsync(hg->defer, 0, 2 * sizeof(unsigned int), s));
                 int rc = run_cells<float>(&hg, 1, &cg, xg, vg, fg, nullptr, nullptr, nullptr, sg, 0, s,
-                                          u0 ? u0 + soff[g] : nullptr, nullptr, nullptr, 0, hin, hout, pos_stride,
+                                          u0 ? u0 + soff[g] : nullptr, nullptr, nullptr, 512, hin, hout, pos_stride,
                                           hg->defer, hist_ext, kg);
                 if (rc) return rc;
                 only = hg->defer;

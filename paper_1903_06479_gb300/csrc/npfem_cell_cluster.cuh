@@ -2,7 +2,9 @@
 // (Team in npfem_cell.cuh), for launches with fewer cells than SMs, where a block per cell
 // would leave the other SMs idle.  One block is bound by its SM's FP64 pipe (about 1650 FP64
 // instructions per triangle and evaluation); eight share them, and what is left is the
-// latency of one triangle's chain (one 258-vertex cell, four steps: 10.9 -> 6.15 ms).  In
+// latency of one triangle's chain (one 258-vertex cell, four steps: 10.9 ms by one block of
+// 512 threads, 6.18 by eight of 512, 4.64 by eight of 128, which do not run the reductions
+// on warps without data).  In
 // FP32 a block's evaluation is too short to pay for the cluster barriers (one 642-vertex
 // cell, eight steps: 1.31 ms by one block, 1.35 ms by eight), so FP32 stays at a block per
 // cell.  Clusters take the cells in turn.
