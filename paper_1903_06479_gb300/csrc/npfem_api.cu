@@ -305,7 +305,9 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
         npfem_handle* h = meshes[gi];
         GroupDesc<T>& g = a.g[gi];
         g.topo = *reinterpret_cast<const TopoDev<T>*>(sizeof(T) == 4 ? (const void*)&h->tf : (const void*)&h->td);
-        if (h->n > kDenseVerts && all > kDenseCells) g.topo.ainv = nullptr;  // the sparse factor
+        // the sparse factor; few cells of an FP32 handle keep the dense inverse (kDenseCells), which
+        // 1026 x 1 pays for with 1284 us against 1110: BF16 and TF32 handles need not
+        if (h->n > kDenseVerts && (all > kDenseCells || h->precision != NPFEM_PREC_FP32)) g.topo.ainv = nullptr;
         g.cell_begin = total;
         g.state_off = state_offs ? state_offs[gi] : state;
         g.stats_off = stats_offs ? stats_offs[gi] : total;
@@ -661,7 +663,7 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
             lead = meshes[g];
         }
     std::vector<int> shape(n_groups, 512);
-    std::vector<char> dense(n_groups, 0);
+    std::vector<char> dense(n_groups, 0), joined(n_groups, 0);
     if (left > sms) {
         for (int g = 0; g < n_groups; ++g) {
             int as = g;
@@ -669,6 +671,27 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
                 if (!done[m] && cells_per_group[m] > sms && meshes[m]->n >= meshes[g]->n) as = m;
             shape[g] = simt_threads(meshes[as], meshes[as]->n, cells_per_group[as]);
             dense[g] = prec != NPFEM_PREC_FP64 && meshes[as]->n <= kDenseVerts;
+            if (as != g) joined[g] = 1;
+        }
+        // Launches follow one another, so a group that leaves SMs idle costs its own latency
+        // (about n) where one launch of 512-thread blocks would fill those SMs with the other
+        // cells; that launch takes longest-cell or total work, the separate ones gain 1.9 from
+        // four blocks per SM and 1.2 from two.  642 x 100 + 258 x 200, two steps: 467 us in one
+        // launch, 589 in two.
+        if (prec != NPFEM_PREC_FP64) {
+            double apart = 0, sum = 0, longest = 0;
+            for (int g = 0; g < n_groups; ++g) {
+                if (done[g]) continue;
+                const double n = meshes[g]->n, w = n * cells_per_group[g] / sms;
+                sum += w;
+                longest = std::max(longest, n);
+                const double per_sm = shape[g] == 128 ? 1.9 : (shape[g] == 256 ? 1.2 : 1.0);
+                apart += joined[g] ? w / per_sm : std::max(n, w / per_sm);
+            }
+            if (n_groups > 1 && std::max(longest, sum) < apart) {
+                std::fill(shape.begin(), shape.end(), 512);
+                std::fill(dense.begin(), dense.end(), 0);
+            }
         }
     } else if (n_groups == 1) {
         shape[0] = simt_threads(meshes[0], meshes[0]->n, left);
