@@ -685,8 +685,11 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
                 const double n = meshes[g]->n, w = n * cells_per_group[g] / sms;
                 sum += w;
                 longest = std::max(longest, n);
-                const double per_sm = shape[g] == 128 ? 1.9 : (shape[g] == 256 ? 1.2 : 1.0);
-                apart += joined[g] ? w / per_sm : std::max(n, w / per_sm);
+                // two sparse solves on an SM take 1.8 of one (1026 x 200 + 642 x 200: 2828 us apart,
+                // 2565 in one launch; 642 x 300 + 1026 x 300: 2893 and 3518)
+                const bool two = shape[g] == 256 && !dense[g];
+                const double per_sm = shape[g] == 128 ? 1.9 : (two ? 1.1 : (shape[g] == 256 ? 1.2 : 1.0));
+                apart += joined[g] ? w / per_sm : std::max(two ? 1.8 * n : n, w / per_sm);
             }
             if (n_groups > 1 && std::max(longest, sum) < apart) {
                 std::fill(shape.begin(), shape.end(), 512);
