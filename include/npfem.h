@@ -190,6 +190,9 @@ int npfem_destroy(npfem_handle* h);
    in its previous step, that launch only lists the cells (no evaluation).
    meshes[g] and cells_per_group[g] (host arrays) name each group; all handles must
    share device, precision and dt.
+   Groups of the SIMT kernel take the options of the first such group with cells, groups
+   of the cluster kernel their own handle's; collision planes and trajectory state are
+   meshes[0]'s.
    x, v: device SoA state (float, or double for NPFEM_PREC_FP64), updated in place
    to x_{n+1}, v_{n+1}. f_ext: device SoA external forces (pN), read only.
    dt must equal the handle's dt (a new dt needs a new handle).

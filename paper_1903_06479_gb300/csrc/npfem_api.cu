@@ -278,15 +278,24 @@ int simt_threads(const npfem_handle* h, int n, long long cells)
     return 512;
 }
 
+// Collision planes of a call (those installed on its first handle), from the first vertex of
+// the launch's x on.
+struct Planes {
+    const float* at = nullptr;
+    double w = 0.0;
+};
+
+// One SIMT launch.  Options, counters and scratch are those of `lead` (the first handle of the
+// call's SIMT groups; the launch's own first one if null).
 template <typename T>
 int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T* x, T* v, const T* f, const T* y,
               T* grad_out, double* parts, npfem_cell_stats* stats, int mode, cudaStream_t stream,
               const T* u0 = nullptr, const long long* state_offs = nullptr, const long long* stats_offs = nullptr,
               int threads = 0, const T* hist_in = nullptr, T* hist_out = nullptr, long long pos_stride = 0,
               unsigned int* defer = nullptr, int hist_ext = 0, T* carry = nullptr,
-              const long long* carry_offs = nullptr, npfem_handle* lead = nullptr)
+              const long long* carry_offs = nullptr, const long long* carry_recs = nullptr, Planes col = Planes(),
+              npfem_handle* lead = nullptr)
 {
-    // options, collision planes, counters and scratch are the call's first handle's
     npfem_handle* h0 = lead ? lead : meshes[0];
     LaunchArgs<T> a;
     memset(&a, 0, sizeof(a));
@@ -312,7 +321,7 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
         g.state_off = state_offs ? state_offs[gi] : state;
         g.stats_off = stats_offs ? stats_offs[gi] : total;
         g.cells = cells[gi];
-        g.carry_rec = carry_rec_elems(h->n_pad, h0->opts.lbfgs_m);
+        g.carry_rec = carry_recs ? carry_recs[gi] : 0;
         g.carry_off = carry_offs ? carry_offs[gi] : 0;
         long long sb = 0;
         place_vectors(&g, h->n, h->n_pad, h->nt, h->npos(), h0->opts.lbfgs_m, budget, &sb);
@@ -341,10 +350,8 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
     a.hist_ext = sizeof(T) == 4 && hist_out ? hist_ext : 0;
     a.carry = mode == 0 && hist_out ? carry : nullptr;
     a.defer = defer;
-    if (mode == 0 && h0->col_planes) {
-        a.col = reinterpret_cast<const float4*>(h0->col_planes);
-        a.col_w = (T)h0->col_w;
-    }
+    a.col = reinterpret_cast<const float4*>(col.at);
+    a.col_w = (T)col.w;
 
     const int smem = kFixedSmem + smem_max;
     int per_sm = 1;
@@ -376,7 +383,7 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
 int run_cells_cluster(npfem_handle* const* meshes, int n_groups, const int32_t* cells, double* x, double* v, const double* f,
                       npfem_cell_stats* stats, cudaStream_t stream, const long long* state_offs, const long long* stats_offs,
                       const double* hist_in, double* hist_out, double* carry, const long long* carry_offs,
-                      npfem_handle* h0, bool* done)
+                      const long long* carry_recs, Planes col, npfem_handle* h0, bool* done)
 {
     *done = false;
     long long total = 0;
@@ -402,7 +409,7 @@ int run_cells_cluster(npfem_handle* const* meshes, int n_groups, const int32_t* 
             g.state_off = state_offs[gi];
             g.stats_off = stats_offs[gi];
             g.cells = cells[gi];
-            g.carry_rec = carry_rec_elems(h->n_pad, h0->opts.lbfgs_m);
+            g.carry_rec = carry_recs[gi];
             g.carry_off = carry_offs[gi];
             long long sb = 0;
             fits = place_vectors_cluster(&g, h->n_pad, h->npos(), h0->opts.lbfgs_m, C,
@@ -436,10 +443,8 @@ int run_cells_cluster(npfem_handle* const* meshes, int n_groups, const int32_t* 
         a.hist_in = hist_in;
         a.hist_out = hist_out;
         a.carry = hist_out ? carry : nullptr;
-        if (h0->col_planes) {
-            a.col = reinterpret_cast<const float4*>(h0->col_planes);
-            a.col_w = h0->col_w;
-        }
+        a.col = reinterpret_cast<const float4*>(col.at);
+        a.col_w = col.w;
         a.slot_bytes = slot;
         if (slot > 0) {
             const size_t need = (size_t)slot * (size_t)(C * total);
@@ -465,16 +470,15 @@ int run_cells_cluster(npfem_handle* const* meshes, int n_groups, const int32_t* 
 // One tensor-core launch for one mesh group (BF16, n <= kTcMaxVerts).
 int run_cells_tc(npfem_handle* h, int cells, float* x, float* v, const float* f, npfem_cell_stats* stats,
                  cudaStream_t stream, const float* u0, const float* hist_in, float* hist_out, long long pos_stride,
-                 unsigned int* only, const float* col = nullptr, double col_w = 0.0, int hist_ext = 0,
-                 float* carry = nullptr)
+                 unsigned int* only, Planes col, int hist_ext, float* carry, long long carry_rec)
 {
     if (cells == 0) return 0;
     LaunchArgs<float> a;
     memset(&a, 0, sizeof(a));
     a.hist_ext = hist_out ? hist_ext : 0;
     a.carry = hist_out ? carry : nullptr;
-    a.col = reinterpret_cast<const float4*>(col);
-    a.col_w = (float)col_w;
+    a.col = reinterpret_cast<const float4*>(col.at);
+    a.col_w = (float)col.w;
     a.u0 = u0;
     a.hist_in = hist_in;
     a.hist_out = hist_out;
@@ -486,7 +490,7 @@ int run_cells_tc(npfem_handle* h, int cells, float* x, float* v, const float* f,
     g.cell_begin = 0;
     g.state_off = 0;
     g.cells = cells;
-    g.carry_rec = carry_rec_elems(h->n_pad, h->opts.lbfgs_m);
+    g.carry_rec = carry_rec;
     g.carry_off = 0;
     const int cluster = h->tf.rb;
     const int ncol = cluster * 3 > 16 ? 32 : 16;
@@ -585,18 +589,18 @@ int run_cells_tc(npfem_handle* h, int cells, float* x, float* v, const float* f,
 // one persistent SIMT launch per block size over the other groups.
 int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_per_group, void* x, void* v,
                 const void* f_ext, cudaStream_t s, npfem_cell_stats* stats, const float* u0, const void* hist_in,
-                void* hist_out, long long pos_stride, int hist_ext = 0, void* carry = nullptr)
+                void* hist_out, long long pos_stride, int hist_ext, void* carry, const CarryPlan& kept)
 {
     const int prec = meshes[0]->precision;
-    std::vector<long long> soff(n_groups), coff(n_groups), koff(n_groups);
-    long long st = 0, ct = 0, kt = 0;
+    const npfem_handle* first = meshes[0];  // its collision planes hold for the whole call
+    std::vector<long long> soff(n_groups), coff(n_groups);
+    const std::vector<long long>&koff = kept.off, &krec = kept.rec;
+    long long st = 0, ct = 0;
     for (int g = 0; g < n_groups; ++g) {
         soff[g] = st;
         coff[g] = ct;
-        koff[g] = kt;
         st += 3LL * meshes[g]->n * cells_per_group[g];
         ct += cells_per_group[g];
-        kt += carry_rec_elems(meshes[g]->n_pad, meshes[0]->opts.lbfgs_m) * cells_per_group[g];
     }
     std::vector<char> done(n_groups, 0);
     for (int g = 0; g < n_groups; ++g) {
@@ -614,6 +618,8 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
             const float* hin = hist_in ? (const float*)hist_in + soff[g] : nullptr;
             float* hout = hist_out ? (float*)hist_out + soff[g] : nullptr;
             float* kg = carry ? (float*)carry + koff[g] : nullptr;
+            Planes colg;
+            if (first->col_planes) colg = {first->col_planes + 4 * (soff[g] / 3), first->col_w};
             unsigned int* only = nullptr;
             if (hout && (size_t)cg + 3 > hg->defer_len) {
                 // allocated with the history (first call of a trajectory), so that the
@@ -638,14 +644,12 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
                 NPFEM_CUDA(cudaMemsetAsync(hg->defer, 0, 2 * sizeof(unsigned int), s));
                 int rc = run_cells<float>(&hg, 1, &cg, xg, vg, fg, nullptr, nullptr, nullptr, sg, 0, s,
                                           u0 ? u0 + soff[g] : nullptr, nullptr, nullptr, 512, hin, hout, pos_stride,
-                                          hg->defer, hist_ext, kg);
+                                          hg->defer, hist_ext, kg, nullptr, &krec[g], colg);
                 if (rc) return rc;
                 only = hg->defer;
             }
-            const npfem_handle* hc = meshes[0];
-            const float* colg = hc->col_planes ? hc->col_planes + 4 * (soff[g] / 3) : nullptr;
             int rc = run_cells_tc(hg, cg, xg, vg, fg, sg, s, u0 ? u0 + soff[g] : nullptr, hin, hout, pos_stride, only,
-                                  colg, hc->col_w, hist_ext, kg);
+                                  colg, hist_ext, kg, krec[g]);
             if (rc) return rc;
             done[g] = 1;
         }
@@ -660,7 +664,7 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
     for (int g = n_groups - 1; g >= 0; --g)
         if (!done[g]) {
             left += cells_per_group[g];
-            lead = meshes[g];
+            lead = meshes[g];  // in the end that of simt_lead()
         }
     std::vector<int> shape(n_groups, 512);
     std::vector<char> dense(n_groups, 0), joined(n_groups, 0);
@@ -704,7 +708,7 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
         const int threads = shape[g0];
         std::vector<npfem_handle*> hs;
         std::vector<int32_t> cs;
-        std::vector<long long> so, co, ko;
+        std::vector<long long> so, co, ko, kr;
         for (int g = g0; g < n_groups; ++g) {
             if (done[g] || shape[g] != threads || dense[g] != dense[g0]) continue;
             hs.push_back(meshes[g]);
@@ -712,14 +716,17 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
             so.push_back(soff[g]);
             co.push_back(coff[g]);
             ko.push_back(koff[g]);
+            kr.push_back(krec[g]);
             done[g] = 1;
         }
         int rc;
+        Planes col;
+        if (first->col_planes) col = {first->col_planes, first->col_w};
         bool clustered = false;
         if (prec == NPFEM_PREC_FP64) {
             rc = run_cells_cluster(hs.data(), (int)hs.size(), cs.data(), (double*)x, (double*)v, (const double*)f_ext,
                                    stats, s, so.data(), co.data(), (const double*)hist_in, (double*)hist_out,
-                                   (double*)carry, ko.data(), lead, &clustered);
+                                   (double*)carry, ko.data(), kr.data(), col, lead, &clustered);
             if (rc) return rc;
         }
         if (clustered) continue;
@@ -727,12 +734,12 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
             rc = run_cells<double>(hs.data(), (int)hs.size(), cs.data(), (double*)x, (double*)v, (const double*)f_ext,
                                    nullptr, nullptr, nullptr, stats, 0, s, nullptr, so.data(), co.data(), threads,
                                    (const double*)hist_in, (double*)hist_out, 0, nullptr, 0, (double*)carry,
-                                   ko.data(), lead);
+                                   ko.data(), kr.data(), col, lead);
         else
             rc = run_cells<float>(hs.data(), (int)hs.size(), cs.data(), (float*)x, (float*)v, (const float*)f_ext,
                                   nullptr, nullptr, nullptr, stats, 0, s, u0, so.data(), co.data(), threads,
                                   (const float*)hist_in, (float*)hist_out, pos_stride, nullptr, hist_ext,
-                                  (float*)carry, ko.data(), lead);
+                                  (float*)carry, ko.data(), kr.data(), col, lead);
         if (rc) return rc;
     }
     return 0;
@@ -1126,12 +1133,18 @@ int npfem_step(npfem_handle* const* meshes, int n_groups, const int32_t* cells_p
     long long pos_stride = 0;
     int hist_ext = 0;
     void* carry = nullptr;
+    std::vector<PlanGroup> groups;
+    for (int g = 0; g < n_groups; ++g)
+        groups.push_back({meshes[g]->n, meshes[g]->n_pad, meshes[g]->opts.lbfgs_m, cells_per_group[g],
+                          meshes[g]->takes_clusters()});
+    const CarryPlan kept = plan_carry(groups);
     if (h0->opts.warm_history) {
         std::vector<long long> sig;
         size_t elems = 0;
         for (int g = 0; g < n_groups; ++g) {
             sig.push_back(reinterpret_cast<long long>(meshes[g]));
             sig.push_back(cells_per_group[g]);
+            sig.push_back(kept.window[g]);
             elems += (size_t)3 * meshes[g]->n * cells_per_group[g];
             if (meshes[g]->precision != NPFEM_PREC_FP64 && meshes[g]->tf.tmlp) hist_ext = 1;
         }
@@ -1155,10 +1168,7 @@ int npfem_step(npfem_handle* const* meshes, int n_groups, const int32_t* cells_p
         }
         if (h0->opts.warm_history == 2 && bytes > 0) {
             // carried L-BFGS pairs: one record per cell, valid together with the corrections
-            size_t kb = 0;
-            for (int g = 0; g < n_groups; ++g)
-                kb += (size_t)carry_rec_elems(meshes[g]->n_pad, h0->opts.lbfgs_m) * cells_per_group[g];
-            kb *= f32 ? 4 : 8;
+            const size_t kb = (size_t)kept.total * (f32 ? 4 : 8);
             if (kb > h0->carry_bytes) {
                 if (h0->carry) {
                     NPFEM_CUDA(cudaStreamSynchronize(s));
@@ -1200,7 +1210,7 @@ int npfem_step(npfem_handle* const* meshes, int n_groups, const int32_t* cells_p
         NPFEM_CUDA(cudaEventRecordWithFlags(h0->tev[h0->tev_used], s, rec_flags));
     }
     int rc = step_groups(meshes, n_groups, cells_per_group, x, v, f_ext, s, stats, u0, hist_in, hist_out, pos_stride,
-                         hist_ext, carry);
+                         hist_ext, carry, kept);
     if (rc) h0->hist_sig.clear();
     if (!rc && timed) {
         NPFEM_CUDA(cudaEventRecordWithFlags(h0->tev[h0->tev_used + 1], s, rec_flags));

@@ -11,15 +11,10 @@
 
 #include "../../include/npfem.h"
 
-#ifdef __CUDACC__
-#define NPFEM_HD __host__ __device__
-#else
-#define NPFEM_HD
-#endif
+#include "npfem_plan.h"
 
 namespace npfem {
 
-constexpr int kMaxGroups = 8;     // meshes per npfem_step launch
 constexpr int kMaxHistory = 8;    // L-BFGS window limit
 constexpr int kNumBaseVecs = 10;  // XN U UT G GT GC UY D TRI WR, then S[m], Y[m]
 constexpr int V_SP = kNumBaseVecs + 2 * kMaxHistory;  // sparse solve's vectors (6 npos): TRI's space when that is in smem
@@ -200,16 +195,6 @@ struct LaunchArgs {
     long long reserve;
     SolverParams p;
 };
-
-// Carried L-BFGS pairs of one cell, in elements of the state type: the solver's history
-// ring as the last solve left it: [0] the pair count, [1] the ring head, [2] that
-// solve's iterations, from [4] the inner products s_i^T y_j by ring slot (m x m, padded
-// to a multiple of 4), then the s vectors of ring slots 0..m-1 and the y vectors
-// ([3][n_pad] each).  The pairs are used while that solve took at most kCarryMaxIters
-// iterations.
-constexpr int kCarryMaxIters = 3;
-NPFEM_HD inline long long carry_head_elems(int m) { return 4 + (((long long)m * m + 3) & ~3LL); }
-NPFEM_HD inline long long carry_rec_elems(int n_pad, int m) { return carry_head_elems(m) + 2LL * m * 3 * n_pad; }
 
 // ---- host-side rest precompute (npfem_setup.cpp) ------------------------------
 struct HostTopo {

@@ -1,0 +1,65 @@
+// Host-side decisions of a step that need no CUDA call: what the groups of a call take from
+// which handle and where their carried pairs lie.
+#pragma once
+
+#include <vector>
+
+#ifdef __CUDACC__
+#define NPFEM_HD __host__ __device__
+#else
+#define NPFEM_HD
+#endif
+
+namespace npfem {
+
+constexpr int kMaxGroups = 8;  // meshes per npfem_step launch
+
+// Carried L-BFGS pairs of one cell, in elements of the state type: the solver's history
+// ring as the last solve left it: [0] the pair count, [1] the ring head, [2] that
+// solve's iterations, from [4] the inner products s_i^T y_j by ring slot (m x m, padded
+// to a multiple of 4), then the s vectors of ring slots 0..m-1 and the y vectors
+// ([3][n_pad] each).  The pairs are used while that solve took at most kCarryMaxIters
+// iterations.
+constexpr int kCarryMaxIters = 3;
+NPFEM_HD inline long long carry_head_elems(int m) { return 4 + (((long long)m * m + 3) & ~3LL); }
+NPFEM_HD inline long long carry_rec_elems(int n_pad, int m) { return carry_head_elems(m) + 2LL * m * 3 * n_pad; }
+
+// One group of a call: its mesh, its own handle's L-BFGS window, and whether its cells go to
+// the tensor-core cluster kernel (with its own handle's options).
+struct PlanGroup {
+    int n, n_pad, window;
+    long long cells;
+    bool clusters;
+};
+
+// The first group with cells for the SIMT launches, whose handle's options they take (-1: none).
+inline int simt_lead(const std::vector<PlanGroup>& groups)
+{
+    for (size_t g = 0; g < groups.size(); ++g)
+        if (groups[g].cells > 0 && !groups[g].clusters) return (int)g;
+    return -1;
+}
+
+// Where every group's carried pairs lie in the call's buffer, in elements: its first record and
+// the size of one, by the window of the options its launch takes.  The buffer is sized and
+// the launches are set up by this alone (handles of one call may differ in their window).
+struct CarryPlan {
+    std::vector<int> window;
+    std::vector<long long> off, rec;
+    long long total = 0;
+};
+
+inline CarryPlan plan_carry(const std::vector<PlanGroup>& groups)
+{
+    CarryPlan c;
+    const int lead = simt_lead(groups);
+    for (const PlanGroup& g : groups) {
+        c.window.push_back(g.clusters || lead < 0 ? g.window : groups[lead].window);
+        c.rec.push_back(carry_rec_elems(g.n_pad, c.window.back()));
+        c.off.push_back(c.total);
+        c.total += c.rec.back() * g.cells;
+    }
+    return c;
+}
+
+}  // namespace npfem

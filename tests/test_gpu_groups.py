@@ -1,0 +1,97 @@
+"""What the groups of one call share: the collision planes of the first handle, whichever
+kernel solves a group, and the carried pairs of handles that differ in their L-BFGS window."""
+import numpy as np
+import pytest
+
+from helpers import DT, max_rel_disp, population32
+from paper_1903_06479_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+WCOL = 2000.0
+
+
+@pytest.fixture(scope="module")
+def N():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1903_06479_gb300 import npfem
+    npfem.lib()
+    return npfem
+
+
+def _call(N, sizes, cells, precision, seed=900, **opts):
+    """Handles and the concatenated state of a call's groups."""
+    import torch
+    hs, pops = [], []
+    for k, (n, c) in enumerate(zip(sizes, cells)):
+        rest, tris = W.discocyte(n)
+        kw = {q: v[k] if isinstance(v, (list, tuple)) else v for q, v in opts.items()}
+        hs.append(N.Handle(rest, tris, N.material(), N.default_opts(precision=precision, tol=1e-6, **kw), dt=DT))
+        pops.append(population32(n, max(c, 1), seed=seed + n, forces="shear", noise_pN=0.5, box=40.0))
+    cat = lambda k: torch.tensor(np.concatenate([W.to_soa(p[k])[:c].ravel() for p, c in zip(pops, cells)]),
+                                 dtype=torch.float32, device="cuda")
+    return hs, pops, [cat(k) for k in "xvf"]
+
+
+# the pressed group: SIMT beside clusters; SIMT and clusters behind a first group without cells; a
+# second cluster group
+@pytest.mark.parametrize("precision,sizes,cells", [("bf16", (642, 2562), (3, 4)), ("fp32", (258, 642), (0, 4)),
+                                                   ("bf16", (258, 642), (0, 4)), ("bf16", (642, 258), (3, 5)),
+                                                   ("fp64", (258, 642), (0, 4))])
+def test_planes_of_the_first_handle_press_every_group(N, precision, sizes, cells):
+    """Planes installed on the first handle press the last group's last cell after three steps
+    without them (so that BF16 cells pass through the first-iterate pass): its mean velocity
+    gains about w d h / m, the other cells' none."""
+    import torch
+    hs, pops, (x, v, f) = _call(N, sizes, cells, precision)
+    if precision == "fp64":
+        x, v, f = x.double(), v.double(), f.double()
+    f.zero_()
+    for _ in range(3):
+        N.step(hs, cells, x, v, f, DT)
+    n, verts = sizes[-1], sum(a * b for a, b in zip(sizes, cells))
+    mean = lambda: v.view(-1)[-3 * n * cells[-1]:].view(cells[-1], 3, n)[:, 0].mean(1).double().cpu().numpy()
+    before = mean()
+    planes = torch.zeros((verts, 4), device="cuda")
+    xl = x[-3 * n:].view(3, n)[0]
+    planes[-n:, 0] = 1.0
+    planes[-n:, 3] = (xl - xl[0] + 0.01).float()
+    hs[0].set_collisions(planes, WCOL)
+    N.step(hs, cells, x, v, f, DT)
+    torch.cuda.synchronize()
+    gain = mean() - before
+    push = WCOL * 0.01 * DT / (94e3 / n)
+    assert gain[-1] > 0.5 * push and np.abs(gain[:-1]).max() < 0.2 * push
+
+
+@pytest.mark.parametrize("precision,sizes,windows", [("bf16", (162, 258), (2, 8)), ("bf16", (258, 1026), (1, 8)),
+                                                     ("fp32", (162, 258), (8, 2)), ("fp64", (66, 162), (2, 8))])
+def test_groups_with_different_windows(N, precision, sizes, windows):
+    """Each group of a call, stepped with carried pairs, agrees with the group stepped alone (every
+    cell converges to 1e-6 in both)."""
+    import torch
+    cells = (5, 6)
+    hs, pops, (x, v, f) = _call(N, sizes, cells, precision, lbfgs_m=windows)
+    td = torch.float64 if precision == "fp64" else torch.float32
+    x, v, f = x.to(td), v.to(td), f.to(td)
+    x0, v0 = x.clone(), v.clone()
+    st = torch.zeros((sum(cells), 32), dtype=torch.uint8, device="cuda")
+    for _ in range(4):
+        N.step(hs, cells, x, v, f, DT, stats=st)
+    torch.cuda.synchronize()
+    st = st.cpu().numpy().view(N.CELL_STATS_DTYPE).reshape(-1)
+    assert (st["status"] == 0).all() and (st["residual"] <= 1e-6).all()
+    at = 0
+    for h, n, c in zip(hs, sizes, cells):
+        part = slice(at, at + 3 * n * c)
+        xa, va = x0[part].clone(), v0[part].clone()
+        rest, tris = W.discocyte(n)
+        alone = N.Handle(rest, tris, N.material(), h.opts, dt=DT)
+        for _ in range(4):
+            N.step([alone], [c], xa, va, f[part], DT)
+        torch.cuda.synchronize()
+        lb = alone.rest_info()[1]["lbar"]
+        X = lambda t: W.from_soa(t.double().cpu().numpy().reshape(c, 3, n))
+        assert max_rel_disp(X(x[part]), X(xa), lb) <= 4e-5
+        at += 3 * n * c
