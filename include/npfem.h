@@ -454,8 +454,10 @@ int npfem_get_tuning(const npfem_handle* h, int* use_tc, int* threads, int* fill
    included, replays as one graph launch).  Creation runs two steps on temporary copies
    of x and v (sizing the handles' buffers; x, v are not modified, stats is written)
    and captures the steps on an internal stream.  The graph holds the pointers it was
-   created with; it must be destroyed before the handles.  Errors: INVALID_ARG, CUDA,
-   OOM. */
+   created with; it must be destroyed before the handles.  Library buffers that it uses
+   stay until then, also when later calls on the handles need larger ones (after a
+   capture that is not the library's own, until the handle is destroyed).  Errors:
+   INVALID_ARG, CUDA, OOM. */
 typedef struct npfem_graph npfem_graph;
 int npfem_graph_create(npfem_handle* const* meshes, int n_groups, const int32_t* cells_per_group, void* x, void* v,
                        const void* f_ext, double dt, int steps, npfem_cell_stats* stats, npfem_graph** out);

@@ -360,18 +360,8 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
     long long grid = std::min<long long>(total, (long long)h0->sm_count * per_sm);
     a.slot_bytes = slot;
     if (slot > 0) {
-        size_t need = (size_t)slot * (size_t)grid;
-        if (need > h0->scratch_bytes) {
-            if (h0->scratch) {
-                NPFEM_CUDA(cudaStreamSynchronize(stream));
-                cudaFree(h0->scratch);
-                h0->scratch = nullptr;
-                h0->scratch_bytes = 0;
-            }
-            NPFEM_CUDA(cudaMalloc(&h0->scratch, need));
-            h0->scratch_bytes = need;
-        }
-        a.scratch = h0->scratch;
+        NPFEM_CUDA(h0->reserve(&h0->scratch, (size_t)slot * (size_t)grid, stream));
+        a.scratch = static_cast<char*>(h0->scratch.p);
     }
     NPFEM_CUDA(launch_cells<T>(a, (int)grid, threads, smem, stream));
     return 0;
@@ -447,18 +437,8 @@ int run_cells_cluster(npfem_handle* const* meshes, int n_groups, const int32_t* 
         a.col_w = col.w;
         a.slot_bytes = slot;
         if (slot > 0) {
-            const size_t need = (size_t)slot * (size_t)(C * total);
-            if (need > h0->scratch_bytes) {
-                if (h0->scratch) {
-                    NPFEM_CUDA(cudaStreamSynchronize(stream));
-                    cudaFree(h0->scratch);
-                    h0->scratch = nullptr;
-                    h0->scratch_bytes = 0;
-                }
-                NPFEM_CUDA(cudaMalloc(&h0->scratch, need));
-                h0->scratch_bytes = need;
-            }
-            a.scratch = h0->scratch;
+            NPFEM_CUDA(h0->reserve(&h0->scratch, (size_t)slot * (size_t)(C * total), stream));
+            a.scratch = static_cast<char*>(h0->scratch.p);
         }
         NPFEM_CUDA(launch_cells_cl(a, C, (int)total, block, smem, stream));
         *done = true;
@@ -542,24 +522,15 @@ int run_cells_tc(npfem_handle* h, int cells, float* x, float* v, const float* f,
     a.slot_bytes = slot;
     const size_t need = (size_t)slot * (size_t)grid + (size_t)slot_b * (size_t)helper;
     if (need > 0) {
-        if (need > h->scratch_bytes) {
-            if (h->scratch) {
-                NPFEM_CUDA(cudaStreamSynchronize(stream));
-                cudaFree(h->scratch);
-                h->scratch = nullptr;
-                h->scratch_bytes = 0;
-            }
-            NPFEM_CUDA(cudaMalloc(&h->scratch, need));
-            h->scratch_bytes = need;
-        }
-        a.scratch = slot > 0 ? h->scratch : nullptr;
+        NPFEM_CUDA(h->reserve(&h->scratch, need, stream));
+        a.scratch = slot > 0 ? static_cast<char*>(h->scratch.p) : nullptr;
     }
     if (helper > 0) {
         b.total_blocks = a.total_blocks;
         b.claim_top = 1;
         b.reserve = grid;  // about one cell per cluster block: the helper's cells take longer
         b.slot_bytes = slot_b;
-        b.scratch = slot_b > 0 ? h->scratch + (size_t)slot * (size_t)grid : nullptr;
+        b.scratch = slot_b > 0 ? static_cast<char*>(h->scratch.p) + (size_t)slot * (size_t)grid : nullptr;
         if (!h->side_stream) {
             NPFEM_CUDA(cudaStreamCreateWithFlags(&h->side_stream, cudaStreamNonBlocking));
             NPFEM_CUDA(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
@@ -621,32 +592,28 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
             Planes colg;
             if (first->col_planes) colg = {first->col_planes + 4 * (soff[g] / 3), first->col_w};
             unsigned int* only = nullptr;
-            if (hout && (size_t)cg + 3 > hg->defer_len) {
+            const size_t listed = sizeof(unsigned int) * ((size_t)cg + 3);
+            if (hout) {
                 // allocated with the history (first call of a trajectory), so that the
                 // steps that use it allocate nothing (they may be captured in a graph)
-                if (hg->defer) {
-                    NPFEM_CUDA(cudaStreamSynchronize(s));
-                    cudaFree(hg->defer);
-                    hg->defer = nullptr;
-                    hg->defer_len = 0;
-                }
-                NPFEM_CUDA(cudaMalloc(&hg->defer, sizeof(unsigned int) * ((size_t)cg + 3)));
-                hg->defer_len = (size_t)cg + 3;
-                NPFEM_CUDA(cudaMemsetAsync(hg->defer, 0, 3 * sizeof(unsigned int), s));
+                const bool fresh = listed > hg->defer.bytes;
+                NPFEM_CUDA(hg->reserve(&hg->defer, listed, s));
+                if (fresh) NPFEM_CUDA(cudaMemsetAsync(hg->defer.p, 0, 3 * sizeof(unsigned int), s));
             }
-            if (hin && (size_t)cg + 3 <= hg->defer_len) {
+            if (hin && listed <= hg->defer.bytes) {
+                unsigned int* defer = static_cast<unsigned int*>(hg->defer.p);
                 // along a trajectory many cells are accepted at the first iterate: a SIMT
                 // launch on every SM (the clusters' idle SMs included) evaluates each cell
                 // there and finishes those, and the cluster kernel takes only the rest
                 // (one block of 512 threads per SM: its vectors fit in shared memory, so a
                 // trajectory's first pass does not grow the handle's scratch)
-                NPFEM_CUDA(cudaMemcpyAsync(hg->defer + 2, hg->defer + 1, sizeof(unsigned int), cudaMemcpyDeviceToDevice, s));
-                NPFEM_CUDA(cudaMemsetAsync(hg->defer, 0, 2 * sizeof(unsigned int), s));
+                NPFEM_CUDA(cudaMemcpyAsync(defer + 2, defer + 1, sizeof(unsigned int), cudaMemcpyDeviceToDevice, s));
+                NPFEM_CUDA(cudaMemsetAsync(defer, 0, 2 * sizeof(unsigned int), s));
                 int rc = run_cells<float>(&hg, 1, &cg, xg, vg, fg, nullptr, nullptr, nullptr, sg, 0, s,
                                           u0 ? u0 + soff[g] : nullptr, nullptr, nullptr, 512, hin, hout, pos_stride,
-                                          hg->defer, hist_ext, kg, nullptr, &krec[g], colg);
+                                          defer, hist_ext, kg, nullptr, &krec[g], colg);
                 if (rc) return rc;
-                only = hg->defer;
+                only = defer;
             }
             int rc = run_cells_tc(hg, cg, xg, vg, fg, sg, s, u0 ? u0 + soff[g] : nullptr, hin, hout, pos_stride, only,
                                   colg, hist_ext, kg, krec[g]);
@@ -760,23 +727,15 @@ int precompute_warm_start(npfem_handle* const* meshes, int n_groups, const int32
     }
     if (!any) return 0;
     npfem_handle* h0 = meshes[0];
-    if (total > h0->ws_u_len) {
-        if (h0->ws_u) {
-            NPFEM_CUDA(cudaStreamSynchronize(s));
-            cudaFree(h0->ws_u);
-            h0->ws_u = nullptr;
-            h0->ws_u_len = 0;
-        }
-        NPFEM_CUDA(cudaMalloc(&h0->ws_u, total * sizeof(float)));
-        h0->ws_u_len = total;
-    }
+    NPFEM_CUDA(h0->reserve(&h0->ws_u, total * sizeof(float), s));
+    float* u = static_cast<float*>(h0->ws_u.p);
     size_t off = 0;
     for (int g = 0; g < n_groups; ++g) {
         if (meshes[g]->tf.ws_mode && meshes[g]->tf.mlp && cells[g] > 0)
-            NPFEM_CUDA(launch_ws_increments(meshes[g], cells[g], x + off, v + off, f + off, h0->ws_u + off, false, s));
+            NPFEM_CUDA(launch_ws_increments(meshes[g], cells[g], x + off, v + off, f + off, u + off, false, s));
         off += (size_t)3 * meshes[g]->n * cells[g];
     }
-    *u0 = h0->ws_u;
+    *u0 = u;
     return 0;
 }
 
@@ -789,16 +748,8 @@ int precompute_temporal(npfem_handle* const* meshes, int n_groups, const int32_t
     npfem_handle* h0 = meshes[0];
     size_t total = 0;
     for (int g = 0; g < n_groups; ++g) total += (size_t)3 * meshes[g]->n * cells[g];
-    if (total > h0->ws_u_len) {
-        if (h0->ws_u) {
-            NPFEM_CUDA(cudaStreamSynchronize(s));
-            cudaFree(h0->ws_u);
-            h0->ws_u = nullptr;
-            h0->ws_u_len = 0;
-        }
-        NPFEM_CUDA(cudaMalloc(&h0->ws_u, total * sizeof(float)));
-        h0->ws_u_len = total;
-    }
+    NPFEM_CUDA(h0->reserve(&h0->ws_u, total * sizeof(float), s));
+    float* u = static_cast<float*>(h0->ws_u.p);
     size_t off = 0;
     const float* c1 = hist;                  // c_{n-1}
     const float* c2 = hist + 3 * pos_stride;  // c_{n-2}
@@ -806,10 +757,10 @@ int precompute_temporal(npfem_handle* const* meshes, int n_groups, const int32_t
     for (int g = 0; g < n_groups; ++g) {
         if (cells[g] > 0)
             NPFEM_CUDA(launch_ws_temporal(meshes[g], cells[g], x + off, v + off, f + off, fp + off, c1 + off, c2 + off,
-                                          nullptr, nullptr, nullptr, nullptr, h0->ws_u + off, 3LL * meshes[g]->n, s));
+                                          nullptr, nullptr, nullptr, nullptr, u + off, 3LL * meshes[g]->n, s));
         off += (size_t)3 * meshes[g]->n * cells[g];
     }
-    *u0 = h0->ws_u;
+    *u0 = u;
     return 0;
 }
 
@@ -1155,36 +1106,18 @@ int npfem_step(npfem_handle* const* meshes, int n_groups, const int32_t* cells_p
         const bool f32 = h0->precision != NPFEM_PREC_FP64;
         pos_stride = f32 ? (long long)elems : 0;
         const size_t bytes = elems * (f32 ? (hist_ext ? 5 : 3) * 4 : 8);
-        if (bytes > h0->hist_bytes) {
-            if (h0->hist) {
-                NPFEM_CUDA(cudaStreamSynchronize(s));
-                cudaFree(h0->hist);
-                h0->hist = nullptr;
-                h0->hist_bytes = 0;
-                h0->hist_sig.clear();
-            }
-            NPFEM_CUDA(cudaMalloc(&h0->hist, bytes));
-            h0->hist_bytes = bytes;
-        }
+        if (bytes > h0->hist.bytes) h0->hist_sig.clear();
+        NPFEM_CUDA(h0->reserve(&h0->hist, bytes, s));
         if (h0->opts.warm_history == 2 && bytes > 0) {
             // carried L-BFGS pairs: one record per cell, valid together with the corrections
             const size_t kb = (size_t)kept.total * (f32 ? 4 : 8);
-            if (kb > h0->carry_bytes) {
-                if (h0->carry) {
-                    NPFEM_CUDA(cudaStreamSynchronize(s));
-                    cudaFree(h0->carry);
-                    h0->carry = nullptr;
-                    h0->carry_bytes = 0;
-                }
-                h0->hist_sig.clear();
-                NPFEM_CUDA(cudaMalloc(&h0->carry, kb));
-                h0->carry_bytes = kb;
-            }
-            carry = h0->carry;
+            if (kb > h0->carry.bytes) h0->hist_sig.clear();
+            NPFEM_CUDA(h0->reserve(&h0->carry, kb, s));
+            carry = h0->carry.p;
         }
         if (bytes > 0) {
-            if (sig == h0->hist_sig) hist_in = h0->hist;
-            hist_out = h0->hist;
+            if (sig == h0->hist_sig) hist_in = h0->hist.p;
+            hist_out = h0->hist.p;
             h0->hist_sig = sig;
         }
     }

@@ -197,19 +197,10 @@ extern "C" int npfem_collision_detect(npfem_handle* const* meshes, int n_groups,
     cudaError_t e = cudaSuccess;
     {
         std::lock_guard<std::mutex> lk(h0->mu);
-        if (need > h0->col_table_len) {
-            if (h0->col_table) {
-                e = cudaStreamSynchronize(s);
-                cudaFree(h0->col_table);
-                h0->col_table = nullptr;
-                h0->col_table_len = 0;
-            }
-            if (e == cudaSuccess) e = cudaMalloc(&h0->col_table, need * sizeof(unsigned));
-            if (e == cudaSuccess) h0->col_table_len = need;
-        }
+        e = h0->reserve(&h0->col_table, need * sizeof(unsigned), s);
         a.mask = (unsigned)(buckets - 1);
-        a.counts = h0->col_table;
-        a.slots = h0->col_table + buckets;
+        a.counts = static_cast<unsigned*>(h0->col_table.p);
+        a.slots = a.counts + buckets;
         if (e == cudaSuccess) e = cudaMemsetAsync(a.counts, 0, buckets * sizeof(unsigned), s);
         if (e == cudaSuccess) e = cudaMemsetAsync(stats, 0, 2 * sizeof(unsigned), s);
         if (e == cudaSuccess && v > 0) {

@@ -12,6 +12,7 @@ struct npfem_graph {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     int device = 0;
+    std::vector<std::shared_ptr<npfem::Captures>> holds;  // of the handles whose buffers the graph uses
     unsigned long long kernels = 0;  // kernel launches one replay performs
 };
 
@@ -78,8 +79,19 @@ int npfem_graph_create(npfem_handle* const* meshes, int n_groups, const int32_t*
     }
     if (!rc) {
         const unsigned long long k0 = npfem_launch_count();
+        for (int g = 0; g < n_groups; ++g) {
+            // counted before the capture, so that nothing it sees is freed from here on
+            std::lock_guard<std::mutex> lk(meshes[g]->captures->mu);
+            ++meshes[g]->captures->graphs;
+            meshes[g]->captures->own = true;
+            G->holds.push_back(meshes[g]->captures);
+        }
         for (int k = 0; k < steps && !rc; ++k)
             rc = npfem_step(meshes, n_groups, cells_per_group, x, v, f_ext, dt, s, stats);
+        for (auto& c : G->holds) {
+            std::lock_guard<std::mutex> lk(c->mu);
+            c->own = false;
+        }
         cudaGraph_t graph = nullptr;
         e = cudaStreamEndCapture(s, &graph);
         if (!rc && e != cudaSuccess) cuda_fail(e, "end capture");
@@ -123,6 +135,11 @@ int npfem_graph_destroy(npfem_graph* g)
     cudaSetDevice(g->device);
     if (g->exec) cudaGraphExecDestroy(g->exec);
     if (g->graph) cudaGraphDestroy(g->graph);
+    for (auto& c : g->holds) {
+        const std::vector<void*> spare = c->end_graph();
+        if (!spare.empty()) cudaDeviceSynchronize();  // a last replay may still run
+        for (void* p : spare) cudaFree(p);
+    }
     cudaSetDevice(dev_prev);
     delete g;
     return 0;

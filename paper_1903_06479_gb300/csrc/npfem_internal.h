@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -426,23 +427,20 @@ struct npfem_handle {
     double* ainv64 = nullptr;   // n x n FP64 inverse (unpadded)
     // launch resources (used when this handle is the first of a step call)
     unsigned int* work = nullptr;
-    char* scratch = nullptr;
-    size_t scratch_bytes = 0;
-    float* ws_u = nullptr;  // learned first increments of the cluster kernel's cells
-    size_t ws_u_len = 0;
+    npfem::GrowBuf scratch;
+    npfem::GrowBuf ws_u;  // learned first increments of the cluster kernel's cells
     // temporal warm start: corrections of the last step (element type of the state) and,
     // for FP32, the positions' rounding residues with their FP32 values; valid for the
     // groups and cell counts recorded in hist_sig
-    void* hist = nullptr;
-    size_t hist_bytes = 0;
+    npfem::GrowBuf hist;
     std::vector<long long> hist_sig;
     // carried L-BFGS pairs (opts.warm_history = 2), one record per cell, valid with hist
-    void* carry = nullptr;
-    size_t carry_bytes = 0;
+    npfem::GrowBuf carry;
     // cells the first-iterate pass leaves to the cluster kernel ([0] count, [1] cells
     // that needed iterations, [2] the previous step's [1], then indices)
-    unsigned int* defer = nullptr;
-    size_t defer_len = 0;
+    npfem::GrowBuf defer;
+    // what captured graphs hold of the buffers above and of col_table
+    std::shared_ptr<npfem::Captures> captures = std::make_shared<npfem::Captures>();
     int sm_count = 0, smem_optin = 0, smem_sm = 0;
     int use_tc = 1;     // BF16: use the tensor-core cluster kernel when the mesh fits it
     // buffers of npfem_step_host
@@ -457,8 +455,7 @@ struct npfem_handle {
     // handle, and the hash table of npfem_collision_detect
     const float* col_planes = nullptr;
     double col_w = 0.0;
-    unsigned* col_table = nullptr;
-    size_t col_table_len = 0;
+    npfem::GrowBuf col_table;
     // resident clusters of the tensor-core kernel at tc_smem bytes (queried once)
     int tc_max_clusters = 0, tc_smem = -1;
     // resident clusters of the few-cells kernel (FP64) by log2 size at cl_smem bytes (queried once)
@@ -479,6 +476,25 @@ struct npfem_handle {
         return precision == NPFEM_PREC_BF16 && n <= npfem::kTcMaxVerts && mat.beta_D == 0.0 && use_tc;
     }
 
+    // Room for `need` bytes in one of the handle's buffers for work on stream s, which may be
+    // capturing.
+    cudaError_t reserve(npfem::GrowBuf* b, size_t need, cudaStream_t s)
+    {
+        struct Mem {
+            cudaStream_t s;
+            int settle() { return (int)cudaStreamSynchronize(s); }
+            void release(void* p) { cudaFree(p); }
+            int acquire(void** p, size_t bytes) { return (int)cudaMalloc(p, bytes); }
+        };
+        const cudaError_t e = (cudaError_t)npfem::grow(b, need, captures.get(), Mem{s});
+        if (e != cudaSuccess) return e;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess)
+            cudaGetLastError();  // the legacy stream beside another stream's capture
+        else if (cap == cudaStreamCaptureStatusActive)
+            captures->see(b);
+        return cudaSuccess;
+    }
     template <typename X>
     X* alloc(size_t count, int* err)
     {
@@ -496,25 +512,16 @@ struct npfem_handle {
     {
         for (void* p : allocs) cudaFree(p);
         allocs.clear();
-        if (scratch) cudaFree(scratch);
-        scratch = nullptr;
-        scratch_bytes = 0;
-        if (ws_u) cudaFree(ws_u);
-        ws_u = nullptr;
-        ws_u_len = 0;
-        if (hist) cudaFree(hist);
-        hist = nullptr;
-        hist_bytes = 0;
+        for (npfem::GrowBuf* b : {&scratch, &ws_u, &hist, &carry, &defer, &col_table}) {
+            if (b->p) cudaFree(b->p);
+            *b = npfem::GrowBuf();
+        }
+        {
+            std::lock_guard<std::mutex> lk(captures->mu);
+            for (void* p : captures->kept) cudaFree(p);
+            captures->kept.clear();
+        }
         hist_sig.clear();
-        if (carry) cudaFree(carry);
-        carry = nullptr;
-        carry_bytes = 0;
-        if (defer) cudaFree(defer);
-        defer = nullptr;
-        defer_len = 0;
-        if (col_table) cudaFree(col_table);
-        col_table = nullptr;
-        col_table_len = 0;
         if (hx) cudaFree(hx);
         if (hv) cudaFree(hv);
         if (hf) cudaFree(hf);

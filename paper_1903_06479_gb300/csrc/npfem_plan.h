@@ -1,7 +1,9 @@
 // Host-side decisions of a step that need no CUDA call: what the groups of a call take from
-// which handle and where their carried pairs lie.
+// which handle, where their carried pairs lie, and when a buffer may be freed.
 #pragma once
 
+#include <cstddef>
+#include <mutex>
 #include <vector>
 
 #ifdef __CUDACC__
@@ -60,6 +62,72 @@ inline CarryPlan plan_carry(const std::vector<PlanGroup>& groups)
         c.total += c.rec.back() * g.cells;
     }
     return c;
+}
+
+// A device buffer that grows on demand.  A captured graph's kernels keep its address, so what a
+// capture has seen is not freed when a larger buffer takes its place (its old address stays
+// good for the graph's replays): it is set aside until the last graph on the handle is gone,
+// or, when a capture that is not the library's own saw it, until the handle is.
+struct GrowBuf {
+    void* p = nullptr;
+    size_t bytes = 0;
+    unsigned seen = 0;  // Captures::epoch of the last capture that saw it (0: none)
+};
+
+// Shared by a handle and its graphs (either may go first).
+struct Captures {
+    std::mutex mu;
+    std::vector<void*> kept;  // superseded buffers that a graph may still use
+    unsigned epoch = 1;
+    int graphs = 0;           // live graphs of the library over the handle
+    bool own = false;         // a graph of the library is being captured
+    bool foreign = false;     // some other capture saw a buffer: its graph's end is not known
+
+    void see(GrowBuf* b)
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        b->seen = epoch;
+        if (!own) foreign = true;
+    }
+
+    // The graph is gone: what the caller may free now.
+    std::vector<void*> end_graph()
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        std::vector<void*> out;
+        if (graphs > 0) --graphs;
+        if (graphs == 0 && !foreign) {
+            out.swap(kept);
+            ++epoch;
+        }
+        return out;
+    }
+};
+
+// Makes room for `need` bytes (contents are lost when it grows).  mem: settle() waits until
+// nothing queued uses the buffer any more, release(p), acquire(&p, bytes); both that can
+// fail return nonzero.
+template <typename Mem>
+int grow(GrowBuf* b, size_t need, Captures* c, Mem&& mem)
+{
+    if (need <= b->bytes) return 0;
+    if (b->p) {
+        std::unique_lock<std::mutex> lk(c->mu);
+        if (b->seen == c->epoch) {
+            c->kept.push_back(b->p);
+        } else {
+            lk.unlock();
+            if (int e = mem.settle()) return e;
+            mem.release(b->p);
+        }
+        *b = GrowBuf();
+    }
+    if (int e = mem.acquire(&b->p, need)) {
+        b->p = nullptr;
+        return e;
+    }
+    b->bytes = need;
+    return 0;
 }
 
 }  // namespace npfem

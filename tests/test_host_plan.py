@@ -10,6 +10,7 @@ CSRC = os.path.join(ROOT, "paper_1903_06479_gb300", "csrc")
 
 PROGRAM = r"""
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include "npfem_plan.h"
 using namespace npfem;
@@ -35,6 +36,37 @@ int main()
             printf("%lld", c.total);
             for (size_t q = 0; q < c.rec.size(); ++q) printf(" %d %lld %lld", c.window[q], c.off[q], c.rec[q]);
             printf("\n");
+        } else if (!strcmp(what, "buffers")) {
+            // one handle's buffer: "n<bytes>" needs room, "c<bytes>" the same inside a capture of the
+            // library, "u<bytes>" inside another one, "g" a graph was made, "d" one is destroyed;
+            // prints the buffers in use, freed and set aside in order
+            struct Mem {
+                int next = 1, settled = 0;
+                std::vector<long> freed;
+                int settle() { ++settled; return 0; }
+                void release(void* p) { freed.push_back((long)p); }
+                int acquire(void** p, size_t) { *p = (void*)(long)next++; return 0; }
+            } mem;
+            Captures c;
+            GrowBuf b;
+            char op[64];
+            while (scanf("%63s", op) == 1 && strcmp(op, "end")) {
+                const size_t need = strtoull(op + 1, nullptr, 10);
+                if (op[0] == 'g') ++c.graphs;
+                if (op[0] == 'd')
+                    for (void* p : c.end_graph()) mem.release(p);
+                if (op[0] == 'n' || op[0] == 'c' || op[0] == 'u') {
+                    c.own = op[0] == 'c';
+                    if (grow(&b, need, &c, mem)) return 1;
+                    if (op[0] != 'n') c.see(&b);
+                    c.own = false;
+                }
+            }
+            printf("%ld |", (long)b.p);
+            for (long p : mem.freed) printf(" %ld", p);
+            printf(" |");
+            for (void* p : c.kept) printf(" %ld", (long)p);
+            printf(" | %d\n", mem.settled);
         }
     }
 }
@@ -85,3 +117,20 @@ def test_launches_take_the_planned_records():
     """No launch sizes a record by itself: the buffer and every launch share one plan."""
     src = open(os.path.join(CSRC, "npfem_api.cu")).read()
     assert "carry_rec_elems" not in src and src.count("plan_carry(") == 1
+
+
+# buffers are numbered as they are made: the one in use | freed | set aside | waits before a free
+@pytest.mark.parametrize("ops,want", [
+    ("n8 n4 n8", "1 | | | 0"),
+    ("n8 n16", "2 | 1 | | 1"),                          # no capture: freed once nothing uses it
+    ("n8 g c8 n16", "2 | | 1 | 0"),                     # a live graph holds the first
+    ("n8 g c8 n16 n32", "3 | 2 | 1 | 1"),               # the second was never captured
+    ("n8 g c8 n16 g c16 n32", "3 | | 1 2 | 0"),
+    ("n8 g c8 n16 d", "2 | 1 | | 0"),                   # its graph is gone
+    ("n8 g c8 n16 g c16 n32 d", "3 | | 1 2 | 0"),       # one of two graphs is left
+    ("n8 g c8 n16 g c16 n32 d d", "3 | 1 2 | | 0"),
+    ("n8 g c8 d n16", "2 | 1 | | 1"),                   # captured by a graph that no longer lives
+    ("n8 u8 n16 g d", "2 | | 1 | 0"),                   # somebody else's capture: until the handle goes
+])
+def test_buffers_of_live_graphs_are_not_freed(plan, ops, want):
+    assert " ".join(plan("buffers " + ops + " end")) == want
