@@ -120,13 +120,17 @@ cudaError_t query_cells_tc(int cluster, int block, int smem, int* max_clusters)
     return cudaSuccess;
 }
 
-// Cluster launch of the tensor-core kernel for one mesh group.
+// Cluster launch of the tensor-core kernel for one mesh group.  Its shared memory is set
+// here as for the other kernels: handles of several meshes share the kernel.
 cudaError_t launch_cells_tc(const LaunchArgs<float>& a, int cluster, int block, int smem, int grid, cudaStream_t s)
 {
+    const void* k = tc_kernel(cluster);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = tc_config(cluster, block, smem, grid, s, attr);
     void* args[1] = {const_cast<LaunchArgs<float>*>(&a)};
-    cudaError_t e = cudaLaunchKernelExC(&cfg, tc_kernel(cluster), args);
+    e = cudaLaunchKernelExC(&cfg, k, args);
     if (e == cudaSuccess) count_launch();
     return e;
 }

@@ -95,3 +95,19 @@ def test_groups_with_different_windows(N, precision, sizes, windows):
         X = lambda t: W.from_soa(t.double().cpu().numpy().reshape(c, 3, n))
         assert max_rel_disp(X(x[part]), X(xa), lb) <= 4e-5
         at += 3 * n * c
+
+
+@pytest.mark.parametrize("windows", [(5, 2), (2, 5)])
+def test_cluster_groups_of_different_shared_memory(N, windows):
+    """Two groups of one cluster kernel whose launches need different amounts of shared memory, step
+    after step."""
+    import torch
+    cells = (4, 5)
+    hs, pops, (x, v, f) = _call(N, (642, 642), cells, "bf16", lbfgs_m=windows)
+    st = torch.zeros((sum(cells), 32), dtype=torch.uint8, device="cuda")
+    for _ in range(3):
+        N.step(hs, cells, x, v, f, DT, stats=st)
+    torch.cuda.synchronize()
+    assert all(h.tuning()["tensor_core"] for h in hs)
+    st = st.cpu().numpy().view(N.CELL_STATS_DTYPE).reshape(-1)
+    assert (st["status"] == 0).all() and (st["residual"] <= 1e-6).all()
