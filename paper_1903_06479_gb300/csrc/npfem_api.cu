@@ -98,9 +98,13 @@ int upload_sparse(npfem_handle* h, const SparseHost& F, SparseDev<T>* sp)
     return 0;
 }
 
+// The factors of H~ and, with damping, M~; empty where the cells apply dense inverses.
+struct Factors {
+    SparseHost system, cluster, mass;
+};
+
 template <typename T>
-int fill_topo(npfem_handle* h, TopoDev<T>* tp, const SparseHost& factor, const SparseHost& cluster_factor,
-              const SparseHost* mass_factor)
+int fill_topo(npfem_handle* h, TopoDev<T>* tp, const Factors& F)
 {
     const HostTopo& H = h->host;
     int rc;
@@ -211,7 +215,7 @@ int fill_topo(npfem_handle* h, TopoDev<T>* tp, const SparseHost& factor, const S
     tp->l_idx = nullptr;
     tp->l_val = nullptr;
     tp->beta_h = (T)(h->mat.beta_D / h->dt);
-    if (mass_factor) {
+    if (h->mat.beta_D > 0.0) {
         if ((rc = upload(h, H.L_ptr, &tp->l_ptr))) return rc;
         std::vector<unsigned short> lidx(H.L_idx.begin(), H.L_idx.end());
         if ((rc = upload(h, lidx, &tp->l_idx))) return rc;
@@ -221,9 +225,9 @@ int fill_topo(npfem_handle* h, TopoDev<T>* tp, const SparseHost& factor, const S
     tp->h_ptr = nullptr;
     tp->h_idx = nullptr;
     tp->h_val = nullptr;
-    if ((rc = upload_sparse(h, factor, &tp->sp))) return rc;
-    if (cluster_factor.npos && (rc = upload_sparse(h, cluster_factor, &tp->spc))) return rc;
-    if (mass_factor && (rc = upload_sparse(h, *mass_factor, &tp->spm))) return rc;
+    if (F.system.npos && (rc = upload_sparse(h, F.system, &tp->sp))) return rc;
+    if (F.cluster.npos && (rc = upload_sparse(h, F.cluster, &tp->spc))) return rc;
+    if (F.mass.npos && (rc = upload_sparse(h, F.mass, &tp->spm))) return rc;
     tp->C = (T)h->mat.C;
     tp->B = (T)h->mat.B;
     tp->Dsk = (T)h->mat.D;
@@ -314,9 +318,6 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
         npfem_handle* h = meshes[gi];
         GroupDesc<T>& g = a.g[gi];
         g.topo = *reinterpret_cast<const TopoDev<T>*>(sizeof(T) == 4 ? (const void*)&h->tf : (const void*)&h->td);
-        // the sparse factor; few cells of an FP32 handle keep the dense inverse (kDenseCells), which
-        // 1026 x 1 pays for with 1284 us against 1110: BF16 and TF32 handles need not
-        if (h->n > kDenseVerts && (all > kDenseCells || h->precision != NPFEM_PREC_FP32)) g.topo.ainv = nullptr;
         g.cell_begin = total;
         g.state_off = state_offs ? state_offs[gi] : state;
         g.stats_off = stats_offs ? stats_offs[gi] : total;
@@ -511,7 +512,6 @@ int run_cells_tc(npfem_handle* h, int cells, float* x, float* v, const float* f,
     if (cells <= grid || h->opts.fill_idle_sms == 0) helper = 0;
     if (helper > 0) {
         b = a;
-        if (h->n > kDenseVerts) b.g[0].topo.ainv = nullptr;  // the sparse factor
         place_vectors(&b.g[0], h->n, h->n_pad, h->nt, h->npos(), h->opts.lbfgs_m, h->smem_optin - kFixedSmem - 1024, &slot_b);
         b.p.cluster = 0;
         b.p.refine = 0;
@@ -641,7 +641,7 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
             for (int m = 0; m < n_groups && cells_per_group[g] <= sms; ++m)
                 if (!done[m] && cells_per_group[m] > sms && meshes[m]->n >= meshes[g]->n) as = m;
             shape[g] = simt_threads(meshes[as], meshes[as]->n, cells_per_group[as]);
-            dense[g] = prec != NPFEM_PREC_FP64 && meshes[as]->n <= kDenseVerts;
+            dense[g] = meshes[as]->tf.ainv != nullptr;
             if (as != g) joined[g] = 1;
         }
         // Launches follow one another, so a group that leaves SMs idle costs its own latency
@@ -998,38 +998,65 @@ int npfem_create(const npfem_mesh* mesh, const npfem_material* mat, const npfem_
     h->work = h->alloc<unsigned int>(4, &e);
     if (e) return bail(e);
     if (cudaMemset(h->work, 0, 4 * sizeof(unsigned)) != cudaSuccess) return bail(fail(NPFEM_ERR_CUDA, "memset failed"));
-    // the dense inverse on the GPU (in place), while the host forms the sparse factor the
-    // solver applies H~^-1 with; beta_D > 0: M~ is not diagonal, the first guess solves
-    // with its factor (Eq. preOptimizationNewton)
-    if (cudaMemcpy(h->ainv64, H.data(), H.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemset(flag, 0, 4 * sizeof(int)) != cudaSuccess)
-        return bail(fail(NPFEM_ERR_CUDA, "upload of H~ failed"));
-    cudaError_t ce = invert_spd_fp64(h->ainv64, n, prow, flag, 0);
-    if (ce != cudaSuccess) return bail(fail(NPFEM_ERR_CUDA, std::string("inversion of H~: ") + cudaGetErrorString(ce)));
-    const bool damped = mat->beta_D > 0.0;
-    SparseHost factor, cluster_factor, mass_factor;
-    int frc = build_sparse_factor(h->host, mesh->rest_xyz, ms, lscale, &factor,
-                                  opts->precision == NPFEM_PREC_FP64 ? &cluster_factor : nullptr, &err);
-    if (!frc && damped)
-        frc = build_sparse_factor(h->host, mesh->rest_xyz, 1.0 + dt * mat->alpha_D, dt * mat->beta_D, &mass_factor,
-                                  nullptr, &err);
-    int hflag = 0;
-    if (cudaMemcpy(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
-        return bail(fail(NPFEM_ERR_CUDA, "inversion of H~ failed"));
-    if (hflag == 2) return bail(fail(NPFEM_ERR_TIMEOUT, "inversion of H~: a grid barrier gave up"));
-    if (hflag) return bail(fail(NPFEM_ERR_NOT_SPD, "H~ is not positive definite"));
+    // one inversion on the GPU, in place; done() waits for it
+    auto invert = [&](double* dA, const std::vector<double>& A, const char* what) -> int {
+        if (cudaMemcpy(dA, A.data(), A.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
+            cudaMemset(flag, 0, 4 * sizeof(int)) != cudaSuccess)
+            return fail(NPFEM_ERR_CUDA, std::string("upload of ") + what + " failed");
+        const cudaError_t ce = invert_spd_fp64(dA, n, prow, flag, 0);
+        if (ce != cudaSuccess) return fail(NPFEM_ERR_CUDA, std::string("inversion of ") + what + ": " + cudaGetErrorString(ce));
+        return 0;
+    };
+    auto done = [&](const char* what) -> int {
+        int hflag = 0;
+        if (cudaMemcpy(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+            return fail(NPFEM_ERR_CUDA, std::string("inversion of ") + what + " failed");
+        if (hflag == 2) return fail(NPFEM_ERR_TIMEOUT, std::string("inversion of ") + what + ": a grid barrier gave up");
+        if (hflag) return fail(NPFEM_ERR_NOT_SPD, std::string(what) + " is not positive definite");
+        return 0;
+    };
+    // the dense inverse (also for npfem_get_inverse), while the host forms the sparse factors
+    // of a mesh whose cells apply those; beta_D > 0: M~ is not diagonal, the first guess
+    // applies M~^-1 the same way (Eq. preOptimizationNewton)
+    const bool damped = mat->beta_D > 0.0, dense = h->precision != NPFEM_PREC_FP64 && n <= kDenseVerts;
+    if ((rc = invert(h->ainv64, H, "H~"))) return bail(rc);
+    Factors factors;
+    int frc = 0;
+    if (!dense) {
+        frc = build_sparse_factor(h->host, mesh->rest_xyz, ms, lscale, &factors.system,
+                                  opts->precision == NPFEM_PREC_FP64 ? &factors.cluster : nullptr, &err);
+        if (!frc && damped)
+            frc = build_sparse_factor(h->host, mesh->rest_xyz, 1.0 + dt * mat->alpha_D, dt * mat->beta_D, &factors.mass,
+                                      nullptr, &err);
+        if (frc == NPFEM_ERR_NOT_SPD && factors.mass.npos) err = "M~ is not positive definite";
+    }
+    if ((rc = done("H~"))) return bail(rc);
     if (frc) return bail(fail(frc, err));
-    float* a32 = nullptr;
-    if (h->precision != NPFEM_PREC_FP64 && n <= kDenseMaxVerts) {
+    float *a32 = nullptr, *m32 = nullptr;
+    if (dense) {
         a32 = h->alloc<float>((size_t)np * np, &e);
         if (e) return bail(e);
     }
     if (symmetrise(h->ainv64, n, np, a32, 0) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
         return bail(fail(NPFEM_ERR_CUDA, "symmetrising A^-1 failed"));
-    rc = h->precision == NPFEM_PREC_FP64 ? fill_topo<double>(h, &h->td, factor, cluster_factor, damped ? &mass_factor : nullptr)
-                                         : fill_topo<float>(h, &h->tf, factor, cluster_factor, damped ? &mass_factor : nullptr);
+    if (dense && damped) {
+        std::vector<double> Mt((size_t)n * n, 0.0);
+        for (int i = 0; i < n; ++i) {
+            Mt[(size_t)i * n + i] += (1.0 + dt * mat->alpha_D) * h->host.mass[i];
+            for (int q = h->host.L_ptr[i]; q < h->host.L_ptr[i + 1]; ++q)
+                Mt[(size_t)i * n + h->host.L_idx[q]] += dt * mat->beta_D * h->host.L_val[q];
+        }
+        m32 = h->alloc<float>((size_t)np * np, &e);
+        double* m64 = h->alloc<double>((size_t)n * n, &e);
+        if (e) return bail(e);
+        if ((rc = invert(m64, Mt, "M~")) || (rc = done("M~"))) return bail(rc);
+        if (symmetrise(m64, n, np, m32, 0) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
+            return bail(fail(NPFEM_ERR_CUDA, "symmetrising M~^-1 failed"));
+    }
+    rc = h->precision == NPFEM_PREC_FP64 ? fill_topo<double>(h, &h->td, factors) : fill_topo<float>(h, &h->tf, factors);
     if (rc) return bail(rc);
     h->tf.ainv = a32;
+    h->tf.minv = m32;
     h->tf.dense_p = dense_parts(n);
     if (h->precision == NPFEM_PREC_BF16 && n <= kTcMaxVerts) {
         // tensor-core path: BF16 A^-1 in 128-row blocks with K padded to 16, and L for

@@ -520,18 +520,17 @@ __device__ void evaluate(const TopoDev<T>& tp, const Team<CL>& tm, const T* XN, 
     });
 }
 
-// R = A^-1 Q for the three coordinate rows with the dense FP32 inverse (meshes of at most
-// kDenseMaxVerts vertices, where its bytes cost no more than the sparse factor's steps): a
+// R = A Q for the three coordinate rows with a dense FP32 inverse (meshes of at most
+// kDenseVerts vertices, where its bytes cost no more than the sparse factor's steps): a
 // warp owns a tile of 128 rows (4 consecutive rows per lane, float4 loads of the symmetric
-// A^-1 by columns, coalesced) and a share of the columns; Q is broadcast from shared
+// A by columns, coalesced) and a share of the columns; Q is broadcast from shared
 // memory.  The parts' partial sums go to `scratch` (the triangle buffer, idle outside the
 // evaluation) and are added in a fixed order that does not depend on the block's size
 // (dense_parts), so the result does not either.
-__device__ void contract_dense(const TopoDev<float>& tp, const float* Q, float* R, float* scratch)
+__device__ void contract_dense(const TopoDev<float>& tp, const float* __restrict__ A, const float* Q, float* R, float* scratch)
 {
     const int n = tp.n, np = tp.n_pad, N3 = 3 * np;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const float* __restrict__ A = tp.ainv;
     const int ntile = (n + 127) >> 7, P = tp.dense_p;
     const int chunk = (((n + P - 1) / P) + 3) & ~3;
     const int nitems = ntile * P;
@@ -898,9 +897,38 @@ __device__ void refine_residual(const TopoDev<T>& tp, const T* src, const T* R, 
 // One cell's quasi-Newton solve, split into the phases that both kernels drive.
 // All threads of the block call every method (control flow is block-uniform).
 // ---------------------------------------------------------------------------------
-// MS: the topology may need the first guess's solve with M~ (beta_D > 0).  CL: the block is
-// one of a cluster that solves the cell together (Team).
-template <typename T, bool MS, bool CL = false>
+// What a kernel may have to apply H~^-1 and (beta_D > 0) M~^-1 with: dense inverses and no
+// damping, dense inverses, or what each cell's mesh has.  The narrower variants hold no call
+// of the sparse solve, whose register saves cost the rest of the kernel 10 % (one 642-vertex
+// cell 1.31 against 1.47 ms per eight steps).
+enum Kind { kDense = 0, kDenseDamped = 1, kAny = 2 };
+
+__device__ __noinline__ void contract_dense_call(const TopoDev<float>& tp, const float* A, const float* Q, float* R,
+                                                 float* scratch)
+{
+    contract_dense(tp, A, Q, R, scratch);
+}
+
+// R = H~^-1 Q (or M~^-1 Q) with the dense inverse A of the cell's mesh or, if it has none, its
+// sparse factor; buf and scratch as solve_sparse and contract_dense want them.
+template <typename T, int K>
+__device__ __forceinline__ void apply_inverse(const TopoDev<T>& tp, const T* A, const SparseDev<T>& sp, const T* Q, T* R,
+                                              T* scratch, T* buf)
+{
+    if constexpr (sizeof(T) == 4 && K != kAny) {
+        contract_dense(tp, A, Q, R, scratch);
+        return;
+    } else if constexpr (sizeof(T) == 4) {
+        if (A) {
+            contract_dense_call(tp, A, Q, R, scratch);
+            return;
+        }
+    }
+    solve_sparse<T, false>(sp, Team<false>{}, tp.n, Q, R, buf);
+}
+
+// K: a Kind.  CL: the block is one of a cluster that solves the cell together (Team).
+template <typename T, int K, bool CL = false>
 struct CellSolver {
     Team<CL> tm;
     const LaunchArgs<T>* a;
@@ -1049,7 +1077,7 @@ struct CellSolver {
         }
         // temporal warm start: u = u_y + (x_n - y_{n-1}), the cell's previous correction,
         // folded into this pass (except with a temporal network or beta_D > 0)
-        const T* Hc = (hist && !(a->hist_ext && a->u0) && !T_.spm.val) ? a->hist_in + so : nullptr;
+        const T* Hc = (hist && !(a->hist_ext && a->u0) && !T_.l_ptr) ? a->hist_in + so : nullptr;
         // U elements per thread at a time, every global load issued before the stores
         // (the stores to shared memory would otherwise hold up the next element's loads)
         constexpr int U = 4;
@@ -1062,7 +1090,7 @@ struct CellSolver {
                 if (e < N3 && i < n) {
                     const int gi = c * n + i;
                     xv[q] = x[gi];
-                    mv[q] = T_.spm.val ? __ldg(&T_.mass[i]) : __ldg(&T_.inv_mass[i]);
+                    mv[q] = T_.l_ptr ? __ldg(&T_.mass[i]) : __ldg(&T_.inv_mass[i]);
                     if (XLO) {
                         hv[q] = XHI[gi];
                         lv[q] = XLO[gi];
@@ -1086,13 +1114,13 @@ struct CellSolver {
                     if (XLO) xn += (hv[q] == xv[q] ? lv[q] : T(0)) - (c == 0 ? l0 : (c == 1 ? l1 : l2));
                     if (eval_mode) {
                         uy = vv[q] - xv[q];
-                    } else if (T_.spm.val) {
+                    } else if (T_.l_ptr) {
                         // right-hand side h M v_n + h^2 F_ext of M~ (y - x_n), solved below
                         ut[e] = h * mv[q] * vv[q] + h * h * fv[q];
                     } else {
                         uy = (h * vv[q] + h * h * fv[q] * mv[q]) * inv_ms;
                     }
-                } else if (T_.spm.val && !eval_mode) {
+                } else if (T_.l_ptr && !eval_mode) {
                     ut[e] = T(0);
                 }
                 XN[e] = xn;
@@ -1101,9 +1129,9 @@ struct CellSolver {
             }
         }
         __syncthreads();
-        if constexpr (MS) if (T_.spm.val && !eval_mode) {
+        if constexpr (K != kDense) if (T_.l_ptr && !eval_mode) {
             // beta_D > 0: y - x_n = M~^-1 (h M v_n + h^2 F_ext) (Eq. preOptimizationNewton)
-            solve_sparse<T, false>(T_.spm, Team<false>{}, n, ut, UYv, SPv);
+            apply_inverse<T, K>(T_, T_.minv, T_.spm, ut, UYv, TRIv, SPv);
             for (int e = tid; e < N3; e += NT) u[e] = UYv[e];
             __syncthreads();
         }
@@ -1119,7 +1147,7 @@ struct CellSolver {
             }
             __syncthreads();
         } else if (hist && !Hc) {
-            // beta_D > 0: the correction on top of the dense first guess
+            // beta_D > 0: the correction on top of the first guess
             const T* Hp = a->hist_in + so;
             for (int e = tid; e < N3; e += NT) {
                 const int c = e / np, i = e - c * np;

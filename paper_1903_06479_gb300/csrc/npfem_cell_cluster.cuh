@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(512, 1) cell_kernel_cl(const __grid_constant__
     }
     __syncthreads();
     cluster_barrier();
-    CellSolver<T, false, true> S;
+    CellSolver<T, kDense, true> S;
     for (long long item = blockIdx.x / C; item < a.total_cells; item += gridDim.x / C) {
         int gi = 0;
         while (gi + 1 < a.n_groups && item >= a.g[gi + 1].cell_begin) ++gi;

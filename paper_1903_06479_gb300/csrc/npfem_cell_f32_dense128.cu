@@ -4,6 +4,6 @@
 
 namespace npfem {
 
-const void* cell_kernel_f32_dense128() { return reinterpret_cast<const void*>(&cell_kernel<float, 128, 4, true>); }
+const void* cell_kernel_f32_dense128() { return reinterpret_cast<const void*>(&cell_kernel<float, 128, 4, kDense>); }
 
 }  // namespace npfem

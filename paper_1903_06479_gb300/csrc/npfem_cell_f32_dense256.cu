@@ -4,6 +4,6 @@
 
 namespace npfem {
 
-const void* cell_kernel_f32_dense256() { return reinterpret_cast<const void*>(&cell_kernel<float, 256, 2, true>); }
+const void* cell_kernel_f32_dense256() { return reinterpret_cast<const void*>(&cell_kernel<float, 256, 2, kDense>); }
 
 }  // namespace npfem

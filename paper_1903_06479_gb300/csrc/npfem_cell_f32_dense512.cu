@@ -4,6 +4,6 @@
 
 namespace npfem {
 
-const void* cell_kernel_f32_dense512() { return reinterpret_cast<const void*>(&cell_kernel<float, 512, 1, true>); }
+const void* cell_kernel_f32_dense512() { return reinterpret_cast<const void*>(&cell_kernel<float, 512, 1, kDense>); }
 
 }  // namespace npfem

@@ -4,6 +4,6 @@
 
 namespace npfem {
 
-const void* cell_kernel_f64_128() { return reinterpret_cast<const void*>(&cell_kernel<double, 128, 4, false>); }
+const void* cell_kernel_f64_128() { return reinterpret_cast<const void*>(&cell_kernel<double, 128, 4, kAny>); }
 
 }  // namespace npfem

@@ -4,6 +4,6 @@
 
 namespace npfem {
 
-const void* cell_kernel_f64_512() { return reinterpret_cast<const void*>(&cell_kernel<double, 512, 1, false>); }
+const void* cell_kernel_f64_512() { return reinterpret_cast<const void*>(&cell_kernel<double, 512, 1, kAny>); }
 
 }  // namespace npfem

@@ -1,7 +1,4 @@
 // The persistent SIMT kernel: blocks pull cells from a work counter and solve them alone.
-// DN: every topology of the launch has the dense FP32 inverse (and no beta_D), so the kernel
-// holds no call of the sparse solve, whose register saves cost the rest of it 10 % (one
-// 642-vertex cell 1.31 against 1.47 ms per eight steps).
 #pragma once
 
 #include "npfem_cell.cuh"
@@ -9,11 +6,11 @@
 namespace npfem {
 namespace {
 
-template <typename T, int MAXT, int MINB, bool DN>
+template <typename T, int MAXT, int MINB, int K>
 __global__ void __launch_bounds__(MAXT, MINB) cell_kernel(const __grid_constant__ LaunchArgs<T> a)
 {
     unsigned char* smem = smem_dyn;
-    CellSolver<T, !DN> S;
+    CellSolver<T, K> S;
     // first-iterate pass: evaluate only while most cells of the last step were accepted
     const bool eval_first = a.defer && 2ll * (long long)a.defer[2] <= a.total_cells;
     for (;;) {
@@ -38,15 +35,12 @@ __global__ void __launch_bounds__(MAXT, MINB) cell_kernel(const __grid_constant_
         const TopoDev<T>& tp = a.g[gi].topo;
         while (S.wants_direction()) {
             S.first_loop();
-            // r = H0 q
-            if constexpr (DN) contract_dense(tp, S.Dv, S.GCv, S.TRIv);
-            else solve_sparse<T, false>(tp.sp, S.tm, tp.n, S.Dv, S.GCv, S.SPv);
+            apply_inverse<T, K>(tp, tp.ainv, tp.sp, S.Dv, S.GCv, S.TRIv, S.SPv);  // r = H0 q
             S.second_loop();
             if (!S.descent()) {
                 // not a descent direction: drop the history, d = -H~^-1 g
                 S.count = 0;
-                if constexpr (DN) contract_dense(tp, S.g, S.GCv, S.TRIv);
-                else solve_sparse<T, false>(tp.sp, S.tm, tp.n, S.g, S.GCv, S.SPv);
+                apply_inverse<T, K>(tp, tp.ainv, tp.sp, S.g, S.GCv, S.TRIv, S.SPv);
                 S.negate_direction();
             }
             if (!S.line_search_update()) break;

@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(512, 1) cell_kernel_tc(const __grid_constant__
     tc::cluster_sync();  // every block's barriers and flags are initialised
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
-    CellSolver<T, false> S;
+    CellSolver<T, kDense> S;
     S.bind(a, gd, smem);
     TcRounds<T, NCOL> R;
     R.sh = sh;

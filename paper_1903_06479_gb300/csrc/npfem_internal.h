@@ -76,13 +76,14 @@ struct TopoDev {
     const unsigned short* ring8_idx;  // [n][8]
     const T* ring8_c;                 // [n][8]
     const T* ring8_ct;                // [n][8]
-    const T* ainv;               // FP32, up to kDenseMaxVerts: [n_pad][n_pad] A^-1 (zero padding); else null
+    const T* ainv;               // FP32, up to kDenseVerts: [n_pad][n_pad] A^-1 (zero padding); else null
     int dense_p;                 // parts of every 128-row tile's columns (dense_parts)
-    SparseDev<T> sp;             // sparse block factor of H~ (applied as H~^-1)
+    SparseDev<T> sp;             // without ainv: sparse block factor of H~ (applied as H~^-1)
     SparseDev<T> spc;            // the same, cut finer, for a cluster's warps (FP64; else null)
     // Rayleigh damping with beta_D > 0: M~ = (1 + h alpha_D) M + h beta_D L is not
-    // diagonal.  spm: the sparse factor of M~ for the first guess; L (CSR, T) for the
-    // inertia term's h beta_D L part; beta_h = beta_D / h.  Null pointers when beta_D = 0.
+    // diagonal.  For the first guess M~^-1 like ainv, or the sparse factor of M~; L (CSR, T)
+    // for the inertia term's h beta_D L part (null when beta_D = 0); beta_h = beta_D / h.
+    const T* minv;
     SparseDev<T> spm;
     const int* l_ptr;
     const unsigned short* l_idx;
@@ -236,13 +237,6 @@ struct SparseHost {
 constexpr int kSparseWarps = 16;     // warps a step's work is spread over
 constexpr int kSparseWarpsCluster = 64;  // the same for a cluster per cell
 constexpr int kSparseMaxIters = 10;  // iterations of a slice a warp keeps in flight (FP32)
-// Meshes whose FP32 solve applies the dense inverse: all up to kDenseVerts (at 642 vertices
-// it reads 1.65 MB from L2 in 48.5 K cycles, the sparse factor 0.47 MB in eleven steps in
-// 41 K, and a population takes the same time with either: 1520 cells 1869 / 1726 us, 3001
-// cells of 258 2.38 / 2.99 ms), and up to kDenseMaxVerts in launches of at most kDenseCells
-// cells, which have the L2 to themselves (one cell of 786 vertices is 3 to 9 % faster with
-// the factor; 37 cells of 1026, 4.2 MB, 111 K cycles dense: 2.65 / 2.24 ms).
-constexpr int kDenseVerts = 700, kDenseMaxVerts = 1100, kDenseCells = 8;
 // Parts of the column range of every 128-row tile, items (tile, part) dealt to 16 warps in
 // turn: the number that minimises the busiest warp's columns (ceil(tiles P / 16) items of
 // ceil(n / P) columns) within max(32, 4 tiles) items.
@@ -333,7 +327,7 @@ inline void place_vectors(GroupDesc<T>* g, int n, int n_pad, int nt, int npos, i
     const int ws_bytes = ((n_pad + 15) & ~15) * 16 * 4;
     const int slot_bytes8 = 24 * n_pad * (int)sizeof(T);  // [8 slots][3][n_pad] corner gradients
     // and the dense contraction's partial sums (384 floats per item)
-    const int dn_bytes = sizeof(T) == 4 && n <= kDenseMaxVerts ? dense_parts(n) * ((n + 127) / 128) * 384 * 4 : 0;
+    const int dn_bytes = sizeof(T) == 4 && n <= kDenseVerts ? dense_parts(n) * ((n + 127) / 128) * 384 * 4 : 0;
     int tb = tri_bytes > slot_bytes8 ? tri_bytes : slot_bytes8;
     tb = tb > dn_bytes ? tb : dn_bytes;
     tb = ((tb > ws_bytes ? tb : ws_bytes) + 15) & ~15;
@@ -354,7 +348,7 @@ inline void place_vectors(GroupDesc<T>* g, int n, int n_pad, int nt, int npos, i
     // the solve gathers at random: a mesh whose TRI will not fit in shared memory gets its
     // buffer there first
     const int sp_bytes = (6 * npos * (int)sizeof(T) + 15) & ~15;
-    const bool own_sp = 3 * vb + tb > smem_budget && sp_bytes + 2 * vb <= smem_budget;
+    const bool own_sp = npos > 0 && 3 * vb + tb > smem_budget && sp_bytes + 2 * vb <= smem_budget;
     if (own_sp) {
         g->loc[V_SP] = base_off;
         used = sp_bytes;
@@ -468,6 +462,7 @@ struct npfem_handle {
     int tev_used = 0;
     std::mutex mu;
 
+    // Positions of the sparse factor (0: the cells apply the dense inverse).
     int npos() const { return precision == NPFEM_PREC_FP64 ? td.sp.npos : tf.sp.npos; }
     // Does the tensor-core cluster kernel take this handle's cells?  (Not with beta_D > 0,
     // whose first guess needs a solve with M~.)

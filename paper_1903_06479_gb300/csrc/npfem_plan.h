@@ -26,6 +26,14 @@ constexpr int kCarryMaxIters = 3;
 NPFEM_HD inline long long carry_head_elems(int m) { return 4 + (((long long)m * m + 3) & ~3LL); }
 NPFEM_HD inline long long carry_rec_elems(int n_pad, int m) { return carry_head_elems(m) + 2LL * m * 3 * n_pad; }
 
+// Meshes whose FP32 cells apply the dense inverse; finer ones (and FP64) apply the sparse
+// factor.  A matter of the mesh alone, so that a cell's arithmetic does not depend on the
+// other cells of its call: the two differ in the order of their sums.  At 642 vertices the
+// inverse is 1.65 MB from L2 in 48.5 K cycles, the factor 0.47 MB in eleven steps in 41 K, and
+// a population takes the same time with either (1520 cells 1869 / 1726 us, 3001 cells of 258
+// 2.38 / 2.99 ms); above, the factor wins at every count (FP32, dense / sparse: DENSEFIGS).
+constexpr int kDenseVerts = 700;
+
 // One group of a call: its mesh, its own handle's L-BFGS window, and whether its cells go to
 // the tensor-core cluster kernel (with its own handle's options).
 struct PlanGroup {

@@ -10,9 +10,12 @@ namespace npfem {
 const void* cell_kernel_f32_dense512();
 const void* cell_kernel_f32_dense256();
 const void* cell_kernel_f32_dense128();
-const void* cell_kernel_f32_sparse512();
-const void* cell_kernel_f32_sparse256();
-const void* cell_kernel_f32_sparse128();
+const void* cell_kernel_f32_damped512();
+const void* cell_kernel_f32_damped256();
+const void* cell_kernel_f32_damped128();
+const void* cell_kernel_f32_any512();
+const void* cell_kernel_f32_any256();
+const void* cell_kernel_f32_any128();
 const void* cell_kernel_f64_512();
 const void* cell_kernel_f64_128();
 const void* cell_kernel_cl_f64();
@@ -21,23 +24,32 @@ const void* cell_kernel_tc32();
 
 namespace {
 
-// Do all topologies of the launch apply the dense inverse (evaluation mode applies none)?
-template <typename T>
-bool all_dense(const LaunchArgs<T>& a)
+// The narrowest variant that has what every topology of the launch applies (an evaluation
+// applies nothing).
+enum { kOfDense, kOfDamped, kOfAny };
+int variant(const LaunchArgs<float>& a)
 {
-    for (int g = 0; g < a.n_groups; ++g)
-        if (sizeof(T) == 8 || !a.g[g].topo.ainv || a.g[g].topo.spm.val) return false;
-    return true;
+    int v = kOfDense;
+    for (int g = 0; g < a.n_groups && a.p.mode == 0; ++g) {
+        if (!a.g[g].topo.ainv) return kOfAny;
+        if (a.g[g].topo.l_ptr) v = kOfDamped;
+    }
+    return v;
 }
 
-template <typename T>
-const void* simt_kernel(const LaunchArgs<T>& a, int block)
+const void* simt_kernel(const LaunchArgs<double>&, int block)
 {
-    if (sizeof(T) == 8) return block == 512 ? cell_kernel_f64_512() : (block == 128 ? cell_kernel_f64_128() : nullptr);
-    const bool dense = all_dense(a);
-    if (block == 512) return dense ? cell_kernel_f32_dense512() : cell_kernel_f32_sparse512();
-    if (block == 256) return dense ? cell_kernel_f32_dense256() : cell_kernel_f32_sparse256();
-    return block == 128 ? (dense ? cell_kernel_f32_dense128() : cell_kernel_f32_sparse128()) : nullptr;
+    return block == 512 ? cell_kernel_f64_512() : (block == 128 ? cell_kernel_f64_128() : nullptr);
+}
+
+const void* simt_kernel(const LaunchArgs<float>& a, int block)
+{
+    using Get = const void* (*)();
+    static const Get by[3][3] = {{cell_kernel_f32_dense512, cell_kernel_f32_dense256, cell_kernel_f32_dense128},
+                                 {cell_kernel_f32_damped512, cell_kernel_f32_damped256, cell_kernel_f32_damped128},
+                                 {cell_kernel_f32_any512, cell_kernel_f32_any256, cell_kernel_f32_any128}};
+    const int b = block == 512 ? 0 : (block == 256 ? 1 : (block == 128 ? 2 : -1));
+    return b < 0 ? nullptr : by[variant(a)][b]();
 }
 
 const void* tc_kernel(int cluster) { return cluster * 3 > 16 ? cell_kernel_tc32() : cell_kernel_tc16(); }

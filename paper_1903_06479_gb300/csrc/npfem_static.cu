@@ -70,8 +70,7 @@ int run_static(npfem_handle* const* meshes, const std::vector<int>& sel, const i
     npfem_handle* h0 = meshes[sel[0]];
     LaunchArgs<T> a;
     memset(&a, 0, sizeof(a));
-    long long total = 0, slot = 0, all = 0;
-    for (int gi : sel) all += cells[gi];
+    long long total = 0, slot = 0;
     int smem_max = 0;
     const int budget = h0->smem_optin - kFixedSmem - 1024;
     int ng = 0;
@@ -79,7 +78,6 @@ int run_static(npfem_handle* const* meshes, const std::vector<int>& sel, const i
         npfem_handle* h = meshes[gi];
         GroupDesc<T>& g = a.g[ng++];
         g.topo = *reinterpret_cast<const TopoDev<T>*>(sizeof(T) == 4 ? (const void*)&h->tf : (const void*)&h->td);
-        if (h->n > kDenseVerts && all > kDenseCells) g.topo.ainv = nullptr;  // the sparse factor
         g.cell_begin = total;
         g.state_off = soff[gi];
         g.stats_off = coff[gi];

@@ -111,3 +111,49 @@ def test_cluster_groups_of_different_shared_memory(N, windows):
     assert all(h.tuning()["tensor_core"] for h in hs)
     st = st.cpu().numpy().view(N.CELL_STATS_DTYPE).reshape(-1)
     assert (st["status"] == 0).all() and (st["residual"] <= 1e-6).all()
+
+
+# alone and beside finer or damped meshes; few cells (one launch for all) and more than one per SM
+@pytest.mark.parametrize("sizes,cells,damped", [((642, 1026), (20, 10), None), ((258, 1026), (20, 3), None),
+                                                ((642, 1026), (160, 160), None), ((642, 258), (20, 10), 1),
+                                                ((162, 1026), (5, 3), 0), ((1026, 642), (1, 30), None)])
+def test_first_group_does_not_depend_on_its_companions(N, sizes, cells, damped):
+    """What a cell's mesh applies (dense inverse or sparse factor) is a matter of the mesh: the first
+    group's cells come out bit for bit as in a call of their own where both calls run them in
+    blocks of one size, and to the rounding of the reductions otherwise."""
+    import torch
+    mats = [N.material(beta_D=0.3) if damped == k else N.material() for k in range(2)]
+    hs, pops, (x, v, f) = _call(N, sizes, cells, "fp32")
+    make = lambda k: N.Handle(*W.discocyte(sizes[k]), mats[k], N.default_opts(precision="fp32", tol=1e-6), dt=DT)
+    x0, v0, f0 = (t[:3 * sizes[0] * cells[0]].clone() for t in (x, v, f))
+    hs = [make(0), make(1)]
+    alone = make(0)
+    st = torch.zeros((sum(cells), 32), dtype=torch.uint8, device="cuda")
+    for _ in range(3):
+        N.step(hs, cells, x, v, f, DT, stats=st)
+        N.step([alone], cells[:1], x0, v0, f0, DT)
+    torch.cuda.synchronize()
+    st = st.cpu().numpy().view(N.CELL_STATS_DTYPE).reshape(-1)
+    assert (st["status"] == 0).all() and (st["residual"] <= 1e-6).all()
+    xa, va = x[:x0.numel()], v[:x0.numel()]
+    if sum(cells) <= 152:
+        assert torch.equal(xa, x0) and torch.equal(va, v0)
+    else:
+        lb = alone.rest_info()[1]["lbar"]
+        X = lambda t: W.from_soa(t.double().cpu().numpy().reshape(cells[0], 3, sizes[0]))
+        assert max_rel_disp(X(xa), X(x0), lb) <= 3e-5
+
+
+@pytest.mark.parametrize("n,cells", [(642, 3), (1026, 2), (1026, 9), (258, 320)])
+def test_tf32_handles_are_fp32_handles(N, n, cells):
+    """TF32 handles run the FP32 path: the same bits."""
+    import torch
+    out = []
+    for precision in ("fp32", "tf32"):
+        hs, _, (x, v, f) = _call(N, (n,), (cells,), precision, refine=int(precision == "tf32"))
+        for _ in range(2):
+            N.step(hs, (cells,), x, v, f, DT)
+        N.step_static(hs, (cells,), x, v, f, DT)
+        torch.cuda.synchronize()
+        out.append((x, v))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
