@@ -62,8 +62,8 @@ extern "C" {
 #define NPFEM_PREC_BF16 3 /* as FP32, but the A^-1 contraction runs on tcgen05 tensor    */
                           /* cores: BF16 A^-1 resident in tensor memory across a cluster */
                           /* of ceil(n/128) SMs, BF16 q, FP32 accumulation, `refine`     */
-                          /* refinement sweeps; meshes above 960 vertices and handles with */
-                          /* beta_D > 0 take the FP32 path                               */
+                          /* refinement sweeps; meshes above 960 vertices, and with        */
+                          /* beta_D > 0 meshes of at most 700, take the FP32 path         */
 
 typedef struct npfem_handle npfem_handle;
 

@@ -496,7 +496,7 @@ int run_cells_tc(npfem_handle* h, int cells, float* x, float* v, const float* f,
     int smem = kFixedSmem + g.smem_bytes;
     smem = std::max(smem, h->smem_optin / 2 + 4096);
     if (h->tc_smem != smem) {
-        NPFEM_CUDA(query_cells_tc(cluster, kTcThreads, smem, &h->tc_max_clusters));
+        NPFEM_CUDA(query_cells_tc(cluster, h->mat.beta_D > 0.0, kTcThreads, smem, &h->tc_max_clusters));
         h->tc_smem = smem;
     }
     const int max_clusters = h->tc_max_clusters;
@@ -858,7 +858,7 @@ int npfem_autotune(npfem_handle* const* meshes, int n_groups, const int32_t* cel
         if (cells == 0) continue;
         std::vector<Shape> cand;
         cand.push_back({0, h->opts.fill_idle_sms, 0});
-        if (prec == NPFEM_PREC_BF16 && h->n <= kTcMaxVerts && h->mat.beta_D == 0.0) {
+        if (h->fits_clusters()) {
             cand.push_back({1, 1, 2});
             cand.push_back({1, 0, 3});
         }
@@ -1025,7 +1025,7 @@ int npfem_create(const npfem_mesh* mesh, const npfem_material* mat, const npfem_
     if (!dense) {
         frc = build_sparse_factor(h->host, mesh->rest_xyz, ms, lscale, &factors.system,
                                   opts->precision == NPFEM_PREC_FP64 ? &factors.cluster : nullptr, &err);
-        if (!frc && damped)
+        if (!frc && damped && !h->fits_clusters())
             frc = build_sparse_factor(h->host, mesh->rest_xyz, 1.0 + dt * mat->alpha_D, dt * mat->beta_D, &factors.mass,
                                       nullptr, &err);
         if (frc == NPFEM_ERR_NOT_SPD && factors.mass.npos) err = "M~ is not positive definite";
@@ -1039,7 +1039,8 @@ int npfem_create(const npfem_mesh* mesh, const npfem_material* mat, const npfem_
     }
     if (symmetrise(h->ainv64, n, np, a32, 0) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
         return bail(fail(NPFEM_ERR_CUDA, "symmetrising A^-1 failed"));
-    if (dense && damped) {
+    const bool dense_mass = damped && (dense || h->fits_clusters());
+    if (dense_mass) {
         std::vector<double> Mt((size_t)n * n, 0.0);
         for (int i = 0; i < n; ++i) {
             Mt[(size_t)i * n + i] += (1.0 + dt * mat->alpha_D) * h->host.mass[i];

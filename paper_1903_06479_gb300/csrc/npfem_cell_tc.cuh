@@ -222,7 +222,7 @@ struct TcRounds {
     }
 };
 
-template <typename T, int NCOL>
+template <typename T, int NCOL, int K>
 __global__ void __launch_bounds__(512, 1) cell_kernel_tc(const __grid_constant__ LaunchArgs<T> a)
 {
     unsigned char* smem = smem_dyn;
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(512, 1) cell_kernel_tc(const __grid_constant__
     tc::cluster_sync();  // every block's barriers and flags are initialised
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
-    CellSolver<T, kDense> S;
+    CellSolver<T, K> S;
     S.bind(a, gd, smem);
     TcRounds<T, NCOL> R;
     R.sh = sh;

@@ -3,6 +3,6 @@
 
 namespace npfem {
 
-const void* cell_kernel_tc16() { return reinterpret_cast<const void*>(&cell_kernel_tc<float, 16>); }
+const void* cell_kernel_tc16() { return reinterpret_cast<const void*>(&cell_kernel_tc<float, 16, kDense>); }
 
 }  // namespace npfem

@@ -3,6 +3,6 @@
 
 namespace npfem {
 
-const void* cell_kernel_tc32() { return reinterpret_cast<const void*>(&cell_kernel_tc<float, 32>); }
+const void* cell_kernel_tc32() { return reinterpret_cast<const void*>(&cell_kernel_tc<float, 32, kDense>); }
 
 }  // namespace npfem

@@ -83,6 +83,7 @@ struct TopoDev {
     // Rayleigh damping with beta_D > 0: M~ = (1 + h alpha_D) M + h beta_D L is not
     // diagonal.  For the first guess M~^-1 like ainv, or the sparse factor of M~; L (CSR, T)
     // for the inertia term's h beta_D L part (null when beta_D = 0); beta_h = beta_D / h.
+    // Meshes of the cluster kernel have the dense M~^-1 too.
     const T* minv;
     SparseDev<T> spm;
     const int* l_ptr;
@@ -237,6 +238,9 @@ struct SparseHost {
 constexpr int kSparseWarps = 16;     // warps a step's work is spread over
 constexpr int kSparseWarpsCluster = 64;  // the same for a cluster per cell
 constexpr int kSparseMaxIters = 10;  // iterations of a slice a warp keeps in flight (FP32)
+// Largest mesh the tensor-core path takes: A block (kpad / 2 columns) plus a
+// 32-column accumulator within 512 TMEM columns, and at most 8 blocks per cluster.
+constexpr int kTcMaxVerts = 960;
 // Parts of the column range of every 128-row tile, items (tile, part) dealt to 16 warps in
 // turn: the number that minimises the busiest warp's columns (ceil(tiles P / 16) items of
 // ceil(n / P) columns) within max(32, 4 tiles) items.
@@ -284,7 +288,7 @@ template <typename T>
 cudaError_t cells_per_sm(const LaunchArgs<T>& a, int block, int smem, int* n);
 // Tensor-core kernel (BF16, A^-1 row blocks resident in TMEM across a cluster): sets
 // its shared-memory size and returns how many clusters can be resident at once.
-cudaError_t query_cells_tc(int cluster, int block, int smem, int* max_clusters);
+cudaError_t query_cells_tc(int cluster, bool damped, int block, int smem, int* max_clusters);
 // Cluster kernel for few FP64 cells: how many clusters of this size can be resident at once, and
 // its launch on `clusters` of them.
 cudaError_t query_cells_cl(int cluster, int block, int smem, int* max_clusters);
@@ -301,9 +305,6 @@ cudaError_t launch_ws_increments(const npfem_handle* h, int n_cells, const float
 cudaError_t launch_ws_temporal(const npfem_handle* h, int n_cells, const float* x, const float* v, const float* f,
                                const float* f_prev, const float* c1, const float* c2, const float* x_next, float* feat,
                                float* target, float* c_out, float* out, long long stride, cudaStream_t s);
-// Largest mesh the tensor-core path takes: A block (kpad / 2 columns) plus a
-// 32-column accumulator within 512 TMEM columns, and at most 8 blocks per cluster.
-constexpr int kTcMaxVerts = 960;
 constexpr int kTcThreads = 512;  // block size of the cluster kernel
 // Records msg as the calling thread's last error and returns code (npfem_api.cu).
 int set_error(int code, const std::string& msg);
@@ -327,7 +328,7 @@ inline void place_vectors(GroupDesc<T>* g, int n, int n_pad, int nt, int npos, i
     const int ws_bytes = ((n_pad + 15) & ~15) * 16 * 4;
     const int slot_bytes8 = 24 * n_pad * (int)sizeof(T);  // [8 slots][3][n_pad] corner gradients
     // and the dense contraction's partial sums (384 floats per item)
-    const int dn_bytes = sizeof(T) == 4 && n <= kDenseVerts ? dense_parts(n) * ((n + 127) / 128) * 384 * 4 : 0;
+    const int dn_bytes = sizeof(T) == 4 && n <= kTcMaxVerts ? dense_parts(n) * ((n + 127) / 128) * 384 * 4 : 0;
     int tb = tri_bytes > slot_bytes8 ? tri_bytes : slot_bytes8;
     tb = tb > dn_bytes ? tb : dn_bytes;
     tb = ((tb > ws_bytes ? tb : ws_bytes) + 15) & ~15;
@@ -464,12 +465,16 @@ struct npfem_handle {
 
     // Positions of the sparse factor (0: the cells apply the dense inverse).
     int npos() const { return precision == NPFEM_PREC_FP64 ? td.sp.npos : tf.sp.npos; }
-    // Does the tensor-core cluster kernel take this handle's cells?  (Not with beta_D > 0,
-    // whose first guess needs a solve with M~.)
-    bool takes_clusters() const
+    // Can the tensor-core cluster kernel take this handle's cells?  With beta_D > 0 only those of
+    // meshes above kDenseVerts: below, FP32 blocks are as fast or faster (damped, two steps,
+    // clusters / FP32: 258 x 2000 1932 / 1172 us, 642 x 40 309 / 282, 642 x 160 529 / 456; but
+    // four steps of 786 x 1 937 / 1042, 786 x 160 1876 / 2022).
+    bool fits_clusters() const
     {
-        return precision == NPFEM_PREC_BF16 && n <= npfem::kTcMaxVerts && mat.beta_D == 0.0 && use_tc;
+        return precision == NPFEM_PREC_BF16 && n <= npfem::kTcMaxVerts && (mat.beta_D == 0.0 || n > npfem::kDenseVerts);
     }
+    // Does it (npfem_autotune may have found the SIMT kernel faster)?
+    bool takes_clusters() const { return use_tc && fits_clusters(); }
 
     // Room for `need` bytes in one of the handle's buffers for work on stream s, which may be
     // capturing.

@@ -21,18 +21,20 @@ const void* cell_kernel_f64_128();
 const void* cell_kernel_cl_f64();
 const void* cell_kernel_tc16();
 const void* cell_kernel_tc32();
+const void* cell_kernel_tc32_damped();
 
 namespace {
 
-// The narrowest variant that has what every topology of the launch applies (an evaluation
-// applies nothing).
+// The narrowest variant that has what every topology of the launch applies.  An evaluation
+// applies nothing, a first-iterate pass (defer) M~^-1 at most.
 enum { kOfDense, kOfDamped, kOfAny };
 int variant(const LaunchArgs<float>& a)
 {
     int v = kOfDense;
     for (int g = 0; g < a.n_groups && a.p.mode == 0; ++g) {
-        if (!a.g[g].topo.ainv) return kOfAny;
-        if (a.g[g].topo.l_ptr) v = kOfDamped;
+        const TopoDev<float>& tp = a.g[g].topo;
+        if ((!tp.ainv && !a.defer) || (tp.l_ptr && !tp.minv)) return kOfAny;
+        if (tp.l_ptr) v = kOfDamped;
     }
     return v;
 }
@@ -52,7 +54,11 @@ const void* simt_kernel(const LaunchArgs<float>& a, int block)
     return b < 0 ? nullptr : by[variant(a)][b]();
 }
 
-const void* tc_kernel(int cluster) { return cluster * 3 > 16 ? cell_kernel_tc32() : cell_kernel_tc16(); }
+const void* tc_kernel(int cluster, bool damped)
+{
+    if (cluster * 3 <= 16) return damped ? nullptr : cell_kernel_tc16();
+    return damped ? cell_kernel_tc32_damped() : cell_kernel_tc32();
+}
 
 cudaLaunchConfig_t tc_config(int cluster, int block, int smem, int grid, cudaStream_t s, cudaLaunchAttribute* attr)
 {
@@ -117,9 +123,10 @@ cudaError_t launch_cells_cl(const LaunchArgs<double>& a, int cluster, int cluste
     return e;
 }
 
-cudaError_t query_cells_tc(int cluster, int block, int smem, int* max_clusters)
+cudaError_t query_cells_tc(int cluster, bool damped, int block, int smem, int* max_clusters)
 {
-    const void* k = tc_kernel(cluster);
+    const void* k = tc_kernel(cluster, damped);
+    if (!k) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
@@ -136,7 +143,8 @@ cudaError_t query_cells_tc(int cluster, int block, int smem, int* max_clusters)
 // here as for the other kernels: handles of several meshes share the kernel.
 cudaError_t launch_cells_tc(const LaunchArgs<float>& a, int cluster, int block, int smem, int grid, cudaStream_t s)
 {
-    const void* k = tc_kernel(cluster);
+    const void* k = tc_kernel(cluster, a.g[0].topo.l_ptr != nullptr);
+    if (!k) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];

@@ -3,7 +3,7 @@ kernel solves a group, and the carried pairs of handles that differ in their L-B
 import numpy as np
 import pytest
 
-from helpers import DT, max_rel_disp, population32
+from helpers import DT, fp32_store_allowance, gpu_step_device, max_rel_disp, oracle_steps, population32
 from paper_1903_06479_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -18,6 +18,34 @@ def N():
     from paper_1903_06479_gb300 import npfem
     npfem.lib()
     return npfem
+
+
+def octahedral_discocyte(f):
+    """The discocyte on an octahedron's faces cut into f x f triangles: 4 f^2 + 2 vertices."""
+    index, points, tris = {}, [], []
+
+    def at(i, j, s):
+        key = (i * s[0], j * s[1], (f - i - j) * s[2])
+        if key not in index:
+            index[key] = len(points)
+            points.append(key)
+        return index[key]
+
+    for s in np.array(np.meshgrid([1, -1], [1, -1], [1, -1])).reshape(3, -1).T:
+        for i in range(f):
+            for j in range(f - i):
+                tris.append((at(i, j, s), at(i + 1, j, s), at(i, j + 1, s)))
+                if i + j < f - 1:
+                    tris.append((at(i + 1, j, s), at(i + 1, j + 1, s), at(i, j + 1, s)))
+    p, t = np.asarray(points, dtype=np.float64), np.asarray(tris, dtype=np.int32)
+    p /= np.linalg.norm(p, axis=1, keepdims=True)
+    flip = (np.cross(p[t[:, 1]] - p[t[:, 0]], p[t[:, 2]] - p[t[:, 0]]) * p[t].sum(1)).sum(1) < 0
+    t[flip] = t[flip][:, [0, 2, 1]]
+    d = W.DISCOCYTE_D
+    xy = 0.5 * d * p[:, :2]
+    r2 = (xy ** 2).sum(1) / d ** 2
+    z = d * np.sqrt(np.clip(1.0 - 4.0 * r2, 0.0, None)) * (W.ES_A0 + W.ES_A1 * r2 + W.ES_A2 * r2 ** 2)
+    return np.column_stack([xy, np.sign(p[:, 2]) * z]), t
 
 
 def _call(N, sizes, cells, precision, seed=900, **opts):
@@ -157,3 +185,26 @@ def test_tf32_handles_are_fp32_handles(N, n, cells):
         torch.cuda.synchronize()
         out.append((x, v))
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
+# 786 vertices: the finest cluster kernel; with damping its first guess solves with M~'s factor
+@pytest.mark.parametrize("precision,refine,cells", [("bf16", 0, 1), ("bf16", 1, 9), ("bf16", 0, 160), ("fp32", 0, 3)])
+def test_damped_cells_between_the_dense_and_the_cluster_limit(N, precision, refine, cells):
+    """Damped cells (beta_D > 0) of 786 vertices against the FP64 oracle after two steps."""
+    import torch
+    from oracle import oracle as O
+    rest, tris = octahedral_discocyte(14)
+    assert len(rest) == 786
+    m = O.Model(rest, tris, W.material_vector(beta_D=0.01), DT)
+    rng = np.random.default_rng(960)
+    x = (rest[None] + 20.0 * rng.random((cells, 1, 3))).astype(np.float32).astype(np.float64)
+    v = (0.01 * rng.standard_normal(x.shape)).astype(np.float32).astype(np.float64)
+    f = (0.5 * rng.standard_normal(x.shape)).astype(np.float32).astype(np.float64)
+    h = N.Handle(rest, tris, N.material(beta_D=0.01), N.default_opts(precision=precision, tol=1e-6, refine=refine), dt=DT)
+    assert h.tuning()["tensor_core"] == (precision == "bf16")
+    xg, vg, st = gpu_step_device(h, x, v, f, steps=2)
+    h.check_device()
+    assert (st["status"] == 0).all() and (st["residual"] <= 1e-6).all()
+    pick = sorted({0, cells - 1})
+    xo, vo, _ = oracle_steps(m, x[pick], v[pick], f[pick], steps=2, tol=1e-10, max_iter=200)
+    assert max_rel_disp(xg[pick], xo, m.lbar) <= 2e-5 + fp32_store_allowance(x, m.lbar)
