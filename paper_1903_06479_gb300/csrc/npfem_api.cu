@@ -515,8 +515,8 @@ int run_cells_tc(npfem_handle* h, int cells, float* x, float* v, const float* f,
         place_vectors(&b.g[0], h->n, h->n_pad, h->nt, h->npos(), h->opts.lbfgs_m, h->smem_optin - kFixedSmem - 1024, &slot_b);
         b.p.cluster = 0;
         b.p.refine = 0;
-        smem_b = kFixedSmem + b.g[0].smem_bytes;
-        if (smem_b <= h->smem_optin / 2) helper = 0;  // would share SMs with the clusters
+        // more than half of an SM's shared memory, so that no block shares an SM with a cluster's
+        smem_b = std::max(kFixedSmem + b.g[0].smem_bytes, h->smem_optin / 2 + 4096);
     }
     a.total_blocks = grid + helper;
     a.slot_bytes = slot;

@@ -208,3 +208,21 @@ def test_damped_cells_between_the_dense_and_the_cluster_limit(N, precision, refi
     pick = sorted({0, cells - 1})
     xo, vo, _ = oracle_steps(m, x[pick], v[pick], f[pick], steps=2, tol=1e-10, max_iter=200)
     assert max_rel_disp(xg[pick], xo, m.lbar) <= 2e-5 + fp32_store_allowance(x, m.lbar)
+
+
+@pytest.mark.parametrize("n", [258, 642])
+def test_idle_sms_are_filled(N, n):
+    """Clusters of three or six blocks leave SMs of a 152-SM GPU idle; with fill_idle_sms a step of
+    more cells than cluster blocks launches the SIMT kernel on them, small meshes included."""
+    import torch
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("needs 152 SMs")
+    launches = []
+    for fill in (0, 1):
+        hs, _, (x, v, f) = _call(N, (n,), (300,), "bf16", warm_history=0, fill_idle_sms=fill)
+        N.step(hs, (300,), x, v, f, DT)
+        before = N.launch_count()
+        N.step(hs, (300,), x, v, f, DT)
+        launches.append(N.launch_count() - before)
+    torch.cuda.synchronize()
+    assert launches[1] == launches[0] + 1
