@@ -263,23 +263,10 @@ int check_opts(const npfem_opts* o)
     return 0;
 }
 
-// Block size of a SIMT group: a mesh's evaluation keeps about n / 32 warps busy and most of
-// its phases are latency-bound, so when every SM has several cells to solve, two blocks of
-// 256 threads or four of 128 per SM overlap each other's phases (vectors that then do not
-// fit in shared memory go to global memory, L2).  Measured, FP32, three steps of 3040
-// cells, 512 / 256 / 128 threads: 66 vertices 296 / 161 / 107 us, 258: 1087 / 688 / 557,
-// 362: 1223 / 830 / 804; 1520 cells: 642: 2048 / 1726 / 1901, 1026: 5235 / 4758 / 6816;
-// 400 cells of 2562: 7677 / 12086.  With at most a cell per SM a cell's own latency counts:
-// 40 cells of 66 vertices 33 / 30 / 31 us, 162: 64 / 66 / 79, 258: 68 / 78 / 105.  FP64 is
-// bound by the FP64 pipe; four blocks hide its latencies best at every size (160 cells of
-// 66 vertices 972 / 705 / 573 us, 258: 5321 / 4846 / 4666).
-int simt_threads(const npfem_handle* h, int n, long long cells)
+// What the block-size rule (npfem_plan.h) asks about a mesh.
+SimtMesh simt_mesh(const npfem_handle* h)
 {
-    const long long sms = h->sm_count;
-    if (h->precision == NPFEM_PREC_FP64) return cells > sms || n <= 320 ? 128 : 512;
-    if (n <= 384 && cells > 2 * sms) return 128;
-    if (n <= 1200 && cells > sms) return 256;
-    return 512;
+    return {h->n, h->precision == NPFEM_PREC_FP64, h->tf.ainv != nullptr, h->mat.beta_D > 0.0};
 }
 
 // Collision planes of a call (those installed on its first handle), from the first vertex of
@@ -305,13 +292,8 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
     memset(&a, 0, sizeof(a));
     long long total = 0, state = 0, slot = 0;
     int smem_max = 0;
-    int n_max = 0;
-    long long all = 0;
-    for (int gi = 0; gi < n_groups; ++gi) {
-        n_max = std::max(n_max, meshes[gi]->n);
-        all += cells[gi];
-    }
-    if (threads <= 0) threads = simt_threads(h0, n_max, all);
+    // an evaluation (one group) chooses for itself
+    if (threads <= 0) threads = eval_threads(simt_mesh(h0), cells[0], h0->sm_count);
     // 512 / threads blocks share an SM's shared memory (1 KB of it per block is the system's)
     const int budget = (threads < 512 ? h0->smem_sm / (512 / threads) : h0->smem_optin) - kFixedSmem - 1024;
     for (int gi = 0; gi < n_groups; ++gi) {
@@ -640,7 +622,7 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
             int as = g;
             for (int m = 0; m < n_groups && cells_per_group[g] <= sms; ++m)
                 if (!done[m] && cells_per_group[m] > sms && meshes[m]->n >= meshes[g]->n) as = m;
-            shape[g] = simt_threads(meshes[as], meshes[as]->n, cells_per_group[as]);
+            shape[g] = simt_threads(simt_mesh(meshes[as]), cells_per_group[as], sms);
             dense[g] = meshes[as]->tf.ainv != nullptr;
             if (as != g) joined[g] = 1;
         }
@@ -668,7 +650,7 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
             }
         }
     } else if (n_groups == 1) {
-        shape[0] = simt_threads(meshes[0], meshes[0]->n, left);
+        shape[0] = simt_threads(simt_mesh(meshes[0]), left, sms);
     }
     for (int g0 = 0; g0 < n_groups; ++g0) {
         if (done[g0]) continue;

@@ -34,6 +34,38 @@ NPFEM_HD inline long long carry_rec_elems(int n_pad, int m) { return carry_head_
 // 2.38 / 2.99 ms); above, the factor wins at every count (FP32, dense / sparse: DENSEFIGS).
 constexpr int kDenseVerts = 700;
 
+// Block size of a SIMT group: a mesh's evaluation keeps about n / 32 warps busy and most of
+// its phases are latency-bound, so when every SM has several cells to solve, two blocks of
+// 256 threads or four of 128 per SM overlap each other's phases (vectors that then do not
+// fit in shared memory go to global memory, L2).  Measured, FP32, three steps of 3040
+// cells, 512 / 256 / 128 threads: 66 vertices 296 / 161 / 107 us, 258: 1087 / 688 / 557,
+// 362: 1223 / 830 / 804; 1520 cells: 642: 2048 / 1726 / 1901, 1026: 5235 / 4758 / 6816;
+// 400 cells of 2562: 7677 / 12086.  With at most a cell per SM a cell's own latency counts:
+// 40 cells of 66 vertices 33 / 30 / 31 us, 162: 64 / 66 / 79, 258: 68 / 78 / 105.  FP64 is
+// bound by the FP64 pipe; four blocks hide its latencies best at every size (160 cells of
+// 66 vertices 972 / 705 / 573 us, 258: 5321 / 4846 / 4666).
+//
+// Cells come in rounds of one per resident block, and a pair of cells on an SM takes 1.65
+// (dense inverse), 1.75 (sparse factor) or 1.8 (damped) times one cell's time, so an odd
+// number of rounds of single cells can be the shorter: 512 / 256 threads, two steps, 642 x
+// 310 1260 / 1318 us, 642 x 456 1267 / 1451, 1026 x 400 3230 / 3810, 1026 x 700 5354 / 5683;
+// but 642 x 304 866 / 773, 642 x 620 2067 / 2021, 1026 x 608 4331 / 4017, 1026 x 930 7342 /
+// 7248.
+struct SimtMesh {
+    int n;
+    bool fp64, dense, damped;
+};
+
+inline int simt_threads(const SimtMesh& m, long long cells, long long sms)
+{
+    if (m.fp64) return cells > sms || m.n <= 320 ? 128 : 512;
+    if (m.n <= 384 && cells > 2 * sms) return 128;
+    if (m.n > 1200 || cells <= sms) return 512;
+    const double pair = m.damped ? 1.8 : (m.dense ? 1.65 : 1.75);
+    const long long singles = (cells + sms - 1) / sms, pairs = (cells + 2 * sms - 1) / (2 * sms);
+    return m.n > 384 && (double)singles < pair * (double)pairs ? 512 : 256;
+}
+
 // One group of a call: its mesh, its own handle's L-BFGS window, and whether its cells go to
 // the tensor-core cluster kernel (with its own handle's options).
 struct PlanGroup {
@@ -48,6 +80,15 @@ inline int simt_lead(const std::vector<PlanGroup>& groups)
     for (size_t g = 0; g < groups.size(); ++g)
         if (groups[g].cells > 0 && !groups[g].clusters) return (int)g;
     return -1;
+}
+
+// The same for an evaluation of the objective, which applies no inverse: finer meshes gain
+// nothing from smaller blocks, whose vectors spill (evaluations of 1026 x 160, 400 and 600
+// cells, 512 / 256 threads: 78 / 78, 113 / 138, 147 / 146 us; 786: 69 / 63, 98 / 110, 126 / 114;
+// 642: 54 / 48, 77 / 78, 98 / 84).
+inline int eval_threads(const SimtMesh& m, long long cells, long long sms)
+{
+    return !m.fp64 && m.n > kDenseVerts ? 512 : simt_threads(m, cells, sms);
 }
 
 // Where every group's carried pairs lie in the call's buffer, in elements: its first record and

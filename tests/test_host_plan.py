@@ -36,6 +36,12 @@ int main()
             printf("%lld", c.total);
             for (size_t q = 0; q < c.rec.size(); ++q) printf(" %d %lld %lld", c.window[q], c.off[q], c.rec[q]);
             printf("\n");
+        } else if (!strcmp(what, "threads")) {
+            int n, fp64, dense, damped, eval;
+            long long cells;
+            if (scanf("%d %d %d %d %lld %d", &n, &fp64, &dense, &damped, &cells, &eval) != 6) return 1;
+            const SimtMesh m = {n, fp64 != 0, dense != 0, damped != 0};
+            printf("%d\n", eval ? eval_threads(m, cells, 152) : simt_threads(m, cells, 152));
         } else if (!strcmp(what, "buffers")) {
             // one handle's buffer: "n<bytes>" needs room, "c<bytes>" the same inside a capture of the
             // library, "u<bytes>" inside another one, "g" a graph was made, "d" one is destroyed;
@@ -134,3 +140,20 @@ def test_launches_take_the_planned_records():
 ])
 def test_buffers_of_live_graphs_are_not_freed(plan, ops, want):
     assert " ".join(plan("buffers " + ops + " end")) == want
+
+
+# vertices, FP64, dense inverse, damped, cells, evaluation on 152 SMs: the edges of the rule
+@pytest.mark.parametrize("mesh,want", [
+    ((642, 0, 1, 0, 152, 0), 512), ((642, 0, 1, 0, 153, 0), 256), ((642, 0, 1, 0, 304, 0), 256),
+    ((642, 0, 1, 0, 305, 0), 512), ((642, 0, 1, 0, 456, 0), 512), ((642, 0, 1, 0, 457, 0), 256),
+    ((642, 0, 1, 0, 620, 0), 256), ((642, 0, 1, 0, 16384, 0), 256), ((642, 0, 1, 1, 620, 0), 512),
+    ((642, 0, 1, 1, 1000, 0), 512), ((642, 0, 1, 1, 1400, 0), 256),
+    ((1026, 0, 0, 0, 304, 0), 256), ((1026, 0, 0, 0, 400, 0), 512), ((1026, 0, 0, 0, 700, 0), 512),
+    ((1026, 0, 0, 0, 930, 0), 256), ((2562, 0, 0, 0, 400, 0), 512),
+    ((258, 0, 1, 0, 152, 0), 512), ((258, 0, 1, 0, 304, 0), 256), ((258, 0, 1, 0, 305, 0), 128),
+    ((258, 0, 1, 1, 400, 0), 128), ((384, 0, 1, 0, 400, 0), 128), ((385, 0, 1, 0, 400, 0), 512),
+    ((1026, 0, 0, 0, 304, 1), 512), ((642, 0, 1, 0, 304, 1), 256), ((258, 0, 1, 0, 400, 1), 128),
+    ((320, 1, 0, 0, 1, 0), 128), ((321, 1, 0, 0, 152, 0), 512), ((642, 1, 0, 0, 153, 0), 128), ((1026, 1, 0, 0, 9, 1), 512),
+])
+def test_block_sizes(plan, mesh, want):
+    assert int(plan("threads %d %d %d %d %d %d" % mesh)[0]) == want
