@@ -952,6 +952,11 @@ int npfem_create(const npfem_mesh* mesh, const npfem_material* mat, const npfem_
     h->n = h->host.n;
     h->nt = h->host.nt;
     h->n_pad = (h->n + 3) & ~3;
+    for (int c = 0; c < 3; ++c) {
+        const auto mm = std::minmax_element(h->host.rest_c.begin() + (size_t)c * h->n, h->host.rest_c.begin() + (size_t)(c + 1) * h->n);
+        h->rest_extent += (*mm.second - *mm.first) * (*mm.second - *mm.first) / 3.0;
+    }
+    h->rest_extent = sqrt(h->rest_extent);
     cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, device);
     cudaDeviceGetAttribute(&h->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
     cudaDeviceGetAttribute(&h->smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device);

@@ -139,8 +139,15 @@ __device__ __forceinline__ const IbmGroup& locate(const IbmArgs& a, long long gv
     while (gi + 1 < a.n_groups && gv >= a.g[gi + 1].vert_begin) ++gi;
     const IbmGroup& G = a.g[gi];
     const long long local = gv - G.vert_begin;
-    *cell = local / G.topo.n;
-    *vert = (int)(local - *cell * G.topo.n);
+    if (local <= UINT_MAX) {
+        // every lane divides: in 32 bits wherever the group has fewer vertices
+        const unsigned l = (unsigned)local, n = (unsigned)G.topo.n, c = l / n;
+        *cell = c;
+        *vert = (int)(l - c * n);
+    } else {
+        *cell = local / G.topo.n;
+        *vert = (int)(local - *cell * G.topo.n);
+    }
     return G;
 }
 
@@ -293,34 +300,41 @@ __global__ void __launch_bounds__(256) ibm_forces_kernel(const __grid_constant__
 }
 
 // Stencil sum of a [nodes][4] field (plus dt times a second one, if given), over the
-// four lanes of a vertex.
+// four lanes of a vertex.  Eight rows in flight per lane and four blocks per SM: 642 x 3000,
+// dx 1 um, interpolation 214 us, against 240 with all sixteen rows and three blocks and 344
+// with eight rows and six blocks, whose registers spill.
 __device__ __forceinline__ void gather4(const LatDev& L, const Stencil& s, int q, float wq, const float* F, const float* F2,
                                         float dt, float out[3])
 {
-    float4 u[16];
-#pragma unroll
-    for (int r = 0; r < 16; ++r) {
-        const long long nd = row_node(L, s, q, r & 3, r >> 2);
-        u[r] = nd >= 0 ? __ldg(reinterpret_cast<const float4*>(F) + nd) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    constexpr int R = 8;
     float o[3] = {0.f, 0.f, 0.f};
 #pragma unroll
-    for (int r = 0; r < 16; ++r) {
-        const float wgt = wq * s.w[1][r & 3] * s.w[2][r >> 2];
-        if (F2) {
-            // the corrected lattice velocity u* + dt f (Step 2) is formed on the fly;
-            // F2 is written by an earlier launch, so a plain (coherent) load
-            const long long nd = row_node(L, s, q, r & 3, r >> 2);
-            if (nd >= 0) {
-                const float4 f = reinterpret_cast<const float4*>(F2)[nd];
-                u[r].x += dt * f.x;
-                u[r].y += dt * f.y;
-                u[r].z += dt * f.z;
-            }
+    for (int r0 = 0; r0 < 16; r0 += R) {
+        float4 u[R];
+#pragma unroll
+        for (int h = 0; h < R; ++h) {
+            const long long nd = row_node(L, s, q, (r0 + h) & 3, (r0 + h) >> 2);
+            u[h] = nd >= 0 ? __ldg(reinterpret_cast<const float4*>(F) + nd) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        o[0] += wgt * u[r].x;
-        o[1] += wgt * u[r].y;
-        o[2] += wgt * u[r].z;
+#pragma unroll
+        for (int h = 0; h < R; ++h) {
+            const int r = r0 + h;
+            const float wgt = wq * s.w[1][r & 3] * s.w[2][r >> 2];
+            if (F2) {
+                // the corrected lattice velocity u* + dt f (Step 2) is formed on the fly;
+                // F2 is written by an earlier launch, so a plain (coherent) load
+                const long long nd = row_node(L, s, q, r & 3, r >> 2);
+                if (nd >= 0) {
+                    const float4 f = reinterpret_cast<const float4*>(F2)[nd];
+                    u[h].x += dt * f.x;
+                    u[h].y += dt * f.y;
+                    u[h].z += dt * f.z;
+                }
+            }
+            o[0] += wgt * u[h].x;
+            o[1] += wgt * u[h].y;
+            o[2] += wgt * u[h].z;
+        }
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) out[c] = sum4(o[c]);
@@ -388,7 +402,7 @@ __device__ __forceinline__ void vertex_phase(const IbmArgs& a, const IbmGroup& G
 
 // Velocity interpolation (phase -1) and the phases of the multi-direct forcing, vertex by
 // vertex (few cells, or small ones).
-__global__ void __launch_bounds__(256, 3) ibm_forcing_kernel(const __grid_constant__ IbmArgs a)
+__global__ void __launch_bounds__(256, 4) ibm_forcing_kernel(const __grid_constant__ IbmArgs a)
 {
     for (long long v0 = blockIdx.x * (long long)kVertsPerBlock; v0 < a.total_verts; v0 += (long long)gridDim.x * kVertsPerBlock) {
         const long long gv = v0 + (threadIdx.x >> 2);
@@ -542,14 +556,30 @@ int ibm_grid(const npfem_handle* h, long long verts)
     return (int)std::max<long long>(1, std::min<long long>(blocks, (long long)std::max(h->sm_count, 1) * 8));
 }
 
-// A phase over all vertices: gathers by a block per cell where the cells fill the GPU and a
-// cell's stencils overlap (1024 cells of 642 vertices, whole forcing with FP64 coordinates: 2.14 -> 1.97 ms), else
-// vertex by vertex.
-constexpr long long kBoxMinCells = 128, kBoxMinVerts = 200;
+// A phase over all vertices: gathers by a block per cell where the cells fill the GPU, a cell's
+// stencils overlap enough to pay for its box, and the boxes fit (node_box); else vertex by
+// vertex.  Step 4 reads two fields per node and gains earlier.  Vertex by vertex / box:
+// interpolation of 642 x 160, 250, 1000 and 3000 cells at dx 1 um 24 / 32, 31 / 32, 80 / 72 and
+// 214 / 206 us, of 1026 x 1000 121 / 101, of 258 x 3000 97 / 121; forcing with two cycles, 258 x
+// 1000 394 / 374, 642 x 1000 877 / 793; at dx 0.5 um, where no box fits, 642 x 1000 1017 / 1338.
+constexpr long long kBoxMinCells = 250, kBoxMinVerts = 500, kBoxMinVertsTwo = 200;
+constexpr double kBoxMeanNodes = 2200.0;  // above, tilted cells pass kBoxNodes (dx below 0.82 um)
 
-cudaError_t launch_forcing(const IbmArgs& a, const npfem_handle* h, cudaStream_t s)
+// Nodes of a cell's box at this spacing on average over its orientations (from the mesh's rest
+// extent).
+double node_box(const npfem_handle* h, double dx)
 {
-    if (a.phase != 1 && a.total_cells >= kBoxMinCells && a.total_verts >= kBoxMinVerts * a.total_cells) {
+    const double e = h->rest_extent / dx + 5.0;
+    return e * e * e;
+}
+
+cudaError_t launch_forcing(const IbmArgs& a, npfem_handle* const* meshes, double dx, cudaStream_t s)
+{
+    const npfem_handle* h = meshes[0];
+    bool box = a.phase != 1 && a.total_cells >= kBoxMinCells &&
+               a.total_verts >= (a.phase == 2 ? kBoxMinVertsTwo : kBoxMinVerts) * a.total_cells;
+    for (int g = 0; g < a.n_groups && box; ++g) box = a.g[g].cells == 0 || node_box(meshes[g], dx) <= kBoxMeanNodes;
+    if (box) {
         const int smem = kBoxNodes * (int)sizeof(float4);
         const int grid = (int)std::min<long long>(a.total_cells, (long long)std::max(h->sm_count, 1) * 4);
         ibm_gather_kernel<<<grid, 256, smem, s>>>(a);
@@ -619,7 +649,7 @@ extern "C" int npfem_ibm_interpolate(npfem_handle* const* meshes, int n_groups, 
     a.field = u_lattice;
     a.out = u_vertex;
     a.phase = -1;
-    const cudaError_t e = launch_forcing(a, meshes[0], static_cast<cudaStream_t>(stream));
+    const cudaError_t e = launch_forcing(a, meshes, lattice->dx, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? 0 : launch_err("npfem_ibm_interpolate", e);
 }
 
@@ -646,7 +676,7 @@ extern "C" int npfem_ibm_forcing(npfem_handle* const* meshes, int n_groups, cons
     cudaError_t e = cudaSuccess;
     auto run = [&](int phase) {
         a.phase = phase;
-        return a.total_verts > 0 ? launch_forcing(a, meshes[0], s) : cudaGetLastError();
+        return a.total_verts > 0 ? launch_forcing(a, meshes, lattice->dx, s) : cudaGetLastError();
     };
     e = run(0);  // Step 0: f_0 = (U - u*(X)) / dt
     for (int l = 0; l < cycles && e == cudaSuccess; ++l) {

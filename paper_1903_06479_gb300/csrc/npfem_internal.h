@@ -416,6 +416,7 @@ struct npfem_handle {
     npfem_material mat{};
     npfem::HostTopo host;
     int n = 0, nt = 0, n_pad = 0;
+    double rest_extent = 0.0;   // root mean square of the rest shape's extents along the axes
     std::vector<void*> allocs;  // every device allocation owned by the handle
     npfem::TopoDev<float> tf{};
     npfem::TopoDev<double> td{};
