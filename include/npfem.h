@@ -58,7 +58,7 @@ extern "C" {
 #define NPFEM_PREC_TF32 2 /* as FP32 (the direction is at least as accurate as with a TF32  */
                           /* A^-1 and one refinement sweep, and cheaper: a sparse factor or  */
                           /* the dense inverse in FP32 beats streaming A^-1 through the      */
-                          /* tensor cores)                                                  */
+                          /* tensor cores); npfem_step takes up to 4096 vertices             */
 #define NPFEM_PREC_BF16 3 /* as FP32, but the A^-1 contraction runs on tcgen05 tensor    */
                           /* cores: BF16 A^-1 resident in tensor memory across a cluster */
                           /* of ceil(n/128) SMs, BF16 q, FP32 accumulation, `refine`     */

@@ -1088,6 +1088,10 @@ int npfem_step(npfem_handle* const* meshes, int n_groups, const int32_t* cells_p
     if (int rc = validate_group(meshes, n_groups, cells_per_group)) return rc;
     if (!x || !v || !f_ext) return fail(NPFEM_ERR_INVALID_ARG, "null state pointer");
     if (dt != meshes[0]->dt) return fail(NPFEM_ERR_INVALID_ARG, "dt differs from the handle's dt");
+    // the limit of the TF32 precision, whatever its cells run on
+    for (int g = 0; g < n_groups; ++g)
+        if (meshes[g]->precision == NPFEM_PREC_TF32 && cells_per_group[g] > 0 && meshes[g]->n > kTf32MaxVerts)
+            return fail(NPFEM_ERR_INVALID_ARG, "npfem_step: TF32 handles of at most 4096 vertices");
     DeviceGuard guard(meshes[0]->device);
     std::lock_guard<std::mutex> lk(meshes[0]->mu);
     cudaStream_t s = static_cast<cudaStream_t>(stream);

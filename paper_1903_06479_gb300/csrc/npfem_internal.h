@@ -305,6 +305,7 @@ cudaError_t launch_ws_increments(const npfem_handle* h, int n_cells, const float
 cudaError_t launch_ws_temporal(const npfem_handle* h, int n_cells, const float* x, const float* v, const float* f,
                                const float* f_prev, const float* c1, const float* c2, const float* x_next, float* feat,
                                float* target, float* c_out, float* out, long long stride, cudaStream_t s);
+constexpr int kTf32MaxVerts = 4096;  // largest mesh npfem_step takes on a TF32 handle
 constexpr int kTcThreads = 512;  // block size of the cluster kernel
 // Records msg as the calling thread's last error and returns code (npfem_api.cu).
 int set_error(int code, const std::string& msg);

@@ -226,3 +226,21 @@ def test_idle_sms_are_filled(N, n):
         launches.append(N.launch_count() - before)
     torch.cuda.synchronize()
     assert launches[1] == launches[0] + 1
+
+
+def test_tf32_limit(N):
+    """npfem_step refuses cells of a TF32 mesh above 4096 vertices, also in a group behind others;
+    npfem_step_static and empty groups are not refused."""
+    import torch
+    (small, big), _, (x, v, f) = _call(N, (66, 4098), (2, 1), "tf32")
+    x0 = x.clone()
+    for hs, cells, at in (((small, big), (2, 1), 0), ((big,), (1,), 3 * 66 * 2)):
+        with pytest.raises(N.NpfemError) as e:
+            N.step(hs, cells, x[at:], v[at:], f[at:], DT)
+        assert e.value.code == -1
+    torch.cuda.synchronize()
+    assert torch.equal(x, x0)
+    N.step((small, big), (2, 0), x, v, f, DT)
+    N.step_static((big,), (1,), x[396:], v[396:], f[396:], DT)
+    torch.cuda.synchronize()
+    assert bool(torch.isfinite(x).all()) and not torch.equal(x[:396], x0[:396]) and not torch.equal(x[396:], x0[396:])
