@@ -440,13 +440,14 @@ const char* npfem_last_error(void);
    without the idle-SM SIMT launch (with the handle's temporal warm start, as the steps
    that follow will run).  x, v are not modified.  trial_ms (optional, 5 floats per
    group) receives the mean trial-step time of each candidate: [0] SIMT, [2] clusters +
-   idle-SM blocks, [3] clusters only (-1 where a candidate does not apply; [1] and [4] are
-   not used).  Blocks.  Errors: INVALID_ARG, CUDA, OOM. */
+   idle-SM blocks, [3] clusters only (-1 where a candidate does not apply; [1] and [4],
+   once blocks of 640 threads, always).  Blocks.  Errors: INVALID_ARG, CUDA, OOM. */
 int npfem_autotune(npfem_handle* const* meshes, int n_groups, const int32_t* cells_per_group, const void* x,
                    const void* v, const void* f_ext, double dt, int trial_steps, float* trial_ms);
 
-/* The launch shape a handle uses: *use_tc (cluster kernel), *threads (the largest SIMT
-   block size, 512), *fill_idle_sms.  Errors: INVALID_ARG. */
+/* The launch shape a handle uses: *use_tc (cluster kernel), *threads (block size of the
+   last npfem_step that ran the handle's cells on the SIMT kernel, a trial of the autotuner
+   included; 512 before the first), *fill_idle_sms.  Errors: INVALID_ARG. */
 int npfem_get_tuning(const npfem_handle* h, int* use_tc, int* threads, int* fill_idle_sms);
 
 /* A CUDA graph of `steps` consecutive npfem_step calls on fixed state buffers (the

@@ -679,6 +679,7 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
             if (rc) return rc;
         }
         if (clustered) continue;
+        for (npfem_handle* h : hs) h->simt_block = threads;
         if (prec == NPFEM_PREC_FP64)
             rc = run_cells<double>(hs.data(), (int)hs.size(), cs.data(), (double*)x, (double*)v, (const double*)f_ext,
                                    nullptr, nullptr, nullptr, stats, 0, s, nullptr, so.data(), co.data(), threads,
@@ -807,7 +808,7 @@ int npfem_get_tuning(const npfem_handle* h, int* use_tc, int* threads, int* fill
 {
     if (!h || !use_tc || !threads || !fill_idle_sms) return fail(NPFEM_ERR_INVALID_ARG, "npfem_get_tuning: null argument");
     *use_tc = h->takes_clusters();
-    *threads = 512;
+    *threads = h->simt_block;
     *fill_idle_sms = h->opts.fill_idle_sms;
     return 0;
 }

@@ -439,6 +439,7 @@ struct npfem_handle {
     // what captured graphs hold of the buffers above and of col_table
     std::shared_ptr<npfem::Captures> captures = std::make_shared<npfem::Captures>();
     int sm_count = 0, smem_optin = 0, smem_sm = 0;
+    int simt_block = 512;  // block size of npfem_step's last launch of the handle's cells off the cluster kernel
     int use_tc = 1;     // BF16: use the tensor-core cluster kernel when the mesh fits it
     // buffers of npfem_step_host
     float* mlp = nullptr;       // learned warm start parameters on the device (weights BF16-rounded)

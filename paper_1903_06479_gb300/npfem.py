@@ -302,7 +302,8 @@ def autotune(handles, cells_per_group, x, v, f, dt: float, trial_steps: int = 2)
     ms = np.zeros(5 * len(handles), dtype=np.float32)
     _check(lib().npfem_autotune(arr, len(handles), cells, _addr(x), _addr(v), _addr(f), float(dt), int(trial_steps),
                                 ms.ctypes.data))
-    names = ("simt512", "unused1", "tc_fill512", "tc_only", "unused4")
+    # the slots of 640-thread blocks stay empty: no kernel runs in them
+    names = ("simt512", "simt640", "tc_fill512", "tc_only", "tc_fill640")
     out = []
     for g, h in enumerate(handles):
         t = h.tuning()

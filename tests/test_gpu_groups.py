@@ -244,3 +244,17 @@ def test_tf32_limit(N):
     N.step_static((big,), (1,), x[396:], v[396:], f[396:], DT)
     torch.cuda.synchronize()
     assert bool(torch.isfinite(x).all()) and not torch.equal(x[:396], x0[:396]) and not torch.equal(x[396:], x0[396:])
+
+
+@pytest.mark.parametrize("precision,n,cells,want", [("fp32", 258, 400, 128), ("fp32", 642, 200, 256),
+                                                    ("fp32", 642, 3, 512), ("fp64", 66, 200, 128)])
+def test_tuning_reports_the_block_size(N, precision, n, cells, want):
+    import torch
+    (h,), _, (x, v, f) = _call(N, (n,), (cells,), precision)
+    if precision == "fp64":
+        x, v, f = x.double(), v.double(), f.double()
+    assert h.tuning()["simt_threads"] == 512
+    N.step([h], [cells], x, v, f, DT)
+    assert h.tuning()["simt_threads"] == want
+    shape = N.autotune([h], [cells], x, v, f, DT, trial_steps=1)[0]
+    assert shape["simt_threads"] == want and set(shape["trial_ms"]) == {"simt512"}
