@@ -215,7 +215,8 @@ int npfem_step(npfem_handle* const* meshes, int n_groups, const int32_t* cells_p
    the process exits.  Arguments, layout, results and errors are those of
    npfem_step, with these differences: every group runs the persistent SIMT solver
    kernel (NPFEM_PREC_BF16 handles included, which then apply H~^-1 in FP32 instead of on
-   the tensor cores) in one launch of 512-thread blocks; the temporal warm start
+   the tensor cores) in one launch of 512-thread blocks (small FP64 meshes: 128
+   threads); the temporal warm start
    (opts.warm_history) is not used; with large meshes it may run fewer persistent
    blocks so that their slots fit; and it returns INVALID_ARG when one block's
    scratch exceeds the array.  Every call looks up the array's device address on

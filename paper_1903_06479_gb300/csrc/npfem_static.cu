@@ -59,34 +59,47 @@ int static_base(char** out)
     return 0;
 }
 
-// One persistent SIMT launch over the groups `sel` (all of one block size), with the
-// groups' offsets into the caller's state and stats arrays.
+// One persistent SIMT launch over all groups, concatenated in the caller's state and stats.
+// Blocks of 512 threads, one per SM; FP64 cells of small meshes, bound by their reductions, take
+// four blocks of 128 (512 / 128 threads: 66 x 1 566 / 404 us, 66 x 700 2735 / 1829, 162 x 320
+// 3583 / 2787; but 162 x 40 1356 / 1409, and from 258 vertices on the slots of four blocks per
+// SM pass the array).
+int static_threads(bool fp64, int n, long long cells, long long sms)
+{
+    return fp64 && n <= (cells > sms ? 162 : 66) ? 128 : 512;
+}
+
 template <typename T>
-int run_static(npfem_handle* const* meshes, const std::vector<int>& sel, const int32_t* cells,
-               const std::vector<long long>& soff, const std::vector<long long>& coff, int threads, T* x, T* v,
-               const T* f, npfem_cell_stats* stats, char* base, cudaStream_t stream)
+int run_static(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T* x, T* v, const T* f,
+               npfem_cell_stats* stats, char* base, cudaStream_t stream)
 {
     using namespace npfem;
-    npfem_handle* h0 = meshes[sel[0]];
+    npfem_handle* h0 = meshes[0];
     LaunchArgs<T> a;
     memset(&a, 0, sizeof(a));
-    long long total = 0, slot = 0;
-    int smem_max = 0;
-    const int budget = h0->smem_optin - kFixedSmem - 1024;
-    int ng = 0;
-    for (int gi : sel) {
+    long long total = 0, state = 0, slot = 0;
+    int smem_max = 0, n_max = 0;
+    long long all = 0;
+    for (int gi = 0; gi < n_groups; ++gi) {
+        n_max = std::max(n_max, meshes[gi]->n);
+        all += cells[gi];
+    }
+    const int threads = static_threads(sizeof(T) == 8, n_max, all, h0->sm_count);
+    const int budget = (threads < 512 ? h0->smem_sm / (512 / threads) : h0->smem_optin) - kFixedSmem - 1024;
+    for (int gi = 0; gi < n_groups; ++gi) {
         npfem_handle* h = meshes[gi];
-        GroupDesc<T>& g = a.g[ng++];
+        GroupDesc<T>& g = a.g[gi];
         g.topo = *reinterpret_cast<const TopoDev<T>*>(sizeof(T) == 4 ? (const void*)&h->tf : (const void*)&h->td);
         g.cell_begin = total;
-        g.state_off = soff[gi];
-        g.stats_off = coff[gi];
+        g.state_off = state;
+        g.stats_off = total;
         g.cells = cells[gi];
         long long sb = 0;
         place_vectors(&g, h->n, h->n_pad, h->nt, h->npos(), h0->opts.lbfgs_m, budget, &sb);
         slot = std::max(slot, sb);
         smem_max = std::max(smem_max, g.smem_bytes);
         total += cells[gi];
+        state += 3LL * h->n * cells[gi];
     }
     if (total == 0) return 0;
     const long long capacity = (long long)NPFEM_STATIC_SCRATCH_BYTES - NPFEM_STATIC_COUNTER_BYTES;
@@ -95,7 +108,7 @@ int run_static(npfem_handle* const* meshes, const std::vector<int>& sel, const i
                          "npfem_step_static: one block needs " + std::to_string(slot) +
                              " bytes of scratch, more than the static array's " + std::to_string(capacity) +
                              " bytes (mesh too large for the allocation-free path)");
-    a.n_groups = ng;
+    a.n_groups = n_groups;
     a.total_cells = total;
     a.x = x;
     a.v = v;
@@ -124,35 +137,6 @@ int run_static(npfem_handle* const* meshes, const std::vector<int>& sel, const i
     return 0;
 }
 
-// The groups in launches of one block size each (the tuned SIMT block size of every
-// handle; 512 threads for FP64), in the order npfem_step launches its SIMT groups.
-template <typename T>
-int step_static(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T* x, T* v, const T* f,
-                npfem_cell_stats* stats, char* base, cudaStream_t stream)
-{
-    std::vector<long long> soff(n_groups), coff(n_groups);
-    long long st = 0, ct = 0;
-    for (int g = 0; g < n_groups; ++g) {
-        soff[g] = st;
-        coff[g] = ct;
-        st += 3LL * meshes[g]->n * cells[g];
-        ct += cells[g];
-    }
-    std::vector<char> done(n_groups, 0);
-    for (int g0 = 0; g0 < n_groups; ++g0) {
-        if (done[g0]) continue;
-        const int threads = 512;
-        std::vector<int> sel;
-        for (int g = g0; g < n_groups; ++g) {
-            if (done[g]) continue;
-            sel.push_back(g);
-            done[g] = 1;
-        }
-        if (int rc = run_static<T>(meshes, sel, cells, soff, coff, threads, x, v, f, stats, base, stream)) return rc;
-    }
-    return 0;
-}
-
 }  // namespace
 
 extern "C" int npfem_step_static(npfem_handle* const* meshes, int n_groups, const int32_t* cells_per_group, void* x,
@@ -173,8 +157,7 @@ extern "C" int npfem_step_static(npfem_handle* const* meshes, int n_groups, cons
     if (int rc = static_base(&base)) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (meshes[0]->precision == NPFEM_PREC_FP64)
-        return step_static<double>(meshes, n_groups, cells_per_group, (double*)x, (double*)v, (const double*)f_ext,
-                                   stats, base, s);
-    return step_static<float>(meshes, n_groups, cells_per_group, (float*)x, (float*)v, (const float*)f_ext, stats, base,
-                              s);
+        return run_static<double>(meshes, n_groups, cells_per_group, (double*)x, (double*)v, (const double*)f_ext, stats,
+                                  base, s);
+    return run_static<float>(meshes, n_groups, cells_per_group, (float*)x, (float*)v, (const float*)f_ext, stats, base, s);
 }

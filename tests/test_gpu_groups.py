@@ -258,3 +258,24 @@ def test_tuning_reports_the_block_size(N, precision, n, cells, want):
     assert h.tuning()["simt_threads"] == want
     shape = N.autotune([h], [cells], x, v, f, DT, trial_steps=1)[0]
     assert shape["simt_threads"] == want and set(shape["trial_ms"]) == {"simt512"}
+
+
+@pytest.mark.parametrize("sizes,cells", [((66,), (1,)), ((66,), (700,)), ((162,), (320,)), ((162,), (9,)), ((66, 162), (140, 20)),
+                                         ((66, 258), (3, 2))])
+def test_static_step_of_small_fp64_meshes(N, sizes, cells):
+    """npfem_step_static in 128-thread blocks (66 vertices; 162 with more than a cell per SM) and in
+    512: a fixed number of iterations differs from npfem_step by rounding only."""
+    import torch
+    hs, _, (x, v, f) = _call(N, sizes, cells, "fp64", warm_history=0, max_iter=4, armijo_noise=0.0)
+    for h in hs:
+        h.close()
+    hs = [N.Handle(*W.discocyte(n), N.material(), N.default_opts(precision="fp64", tol=0.0, max_iter=4, warm_history=0,
+                                                               armijo_noise=0.0), dt=DT) for n in sizes]
+    x, v, f = x.double(), v.double(), f.double()
+    xs, vs = x.clone(), v.clone()
+    for _ in range(2):
+        N.step(hs, cells, x, v, f, DT)
+        N.step_static(hs, cells, xs, vs, f, DT)
+    torch.cuda.synchronize()
+    lb = min(h.rest_info()[1]["lbar"] for h in hs)
+    assert float((x - xs).abs().max()) <= 1e-10 * lb and float((v - vs).abs().max()) * DT <= 1e-10 * lb
