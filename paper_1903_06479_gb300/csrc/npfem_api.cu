@@ -266,7 +266,7 @@ int check_opts(const npfem_opts* o)
 // What the block-size rule (npfem_plan.h) asks about a mesh.
 SimtMesh simt_mesh(const npfem_handle* h)
 {
-    return {h->n, h->precision == NPFEM_PREC_FP64, h->tf.ainv != nullptr, h->mat.beta_D > 0.0};
+    return {h->n, h->precision == NPFEM_PREC_FP64, h->n <= kDenseVerts, h->mat.beta_D > 0.0};
 }
 
 // Collision planes of a call (those installed on its first handle), from the first vertex of
@@ -290,7 +290,8 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
     npfem_handle* h0 = lead ? lead : meshes[0];
     LaunchArgs<T> a;
     memset(&a, 0, sizeof(a));
-    long long total = 0, state = 0, slot = 0;
+    long long total = 0, state = 0, slot = 0, all = 0;
+    for (int gi = 0; gi < n_groups; ++gi) all += cells[gi];
     int smem_max = 0;
     // an evaluation (one group) chooses for itself
     if (threads <= 0) threads = eval_threads(simt_mesh(h0), cells[0], h0->sm_count);
@@ -300,6 +301,7 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
         npfem_handle* h = meshes[gi];
         GroupDesc<T>& g = a.g[gi];
         g.topo = *reinterpret_cast<const TopoDev<T>*>(sizeof(T) == 4 ? (const void*)&h->tf : (const void*)&h->td);
+        if (!h->applies_dense(all)) g.topo.ainv = nullptr;
         g.cell_begin = total;
         g.state_off = state_offs ? state_offs[gi] : state;
         g.stats_off = stats_offs ? stats_offs[gi] : total;
@@ -623,7 +625,7 @@ int step_groups(npfem_handle* const* meshes, int n_groups, const int32_t* cells_
             for (int m = 0; m < n_groups && cells_per_group[g] <= sms; ++m)
                 if (!done[m] && cells_per_group[m] > sms && meshes[m]->n >= meshes[g]->n) as = m;
             shape[g] = simt_threads(simt_mesh(meshes[as]), cells_per_group[as], sms);
-            dense[g] = meshes[as]->tf.ainv != nullptr;
+            dense[g] = meshes[as]->applies_dense(left);
             if (as != g) joined[g] = 1;
         }
         // Launches follow one another, so a group that leaves SMs idle costs its own latency
@@ -1007,6 +1009,7 @@ int npfem_create(const npfem_mesh* mesh, const npfem_material* mat, const npfem_
     // of a mesh whose cells apply those; beta_D > 0: M~ is not diagonal, the first guess
     // applies M~^-1 the same way (Eq. preOptimizationNewton)
     const bool damped = mat->beta_D > 0.0, dense = h->precision != NPFEM_PREC_FP64 && n <= kDenseVerts;
+    const bool few = h->applies_dense(1);  // dense at least in launches of few cells
     if ((rc = invert(h->ainv64, H, "H~"))) return bail(rc);
     Factors factors;
     int frc = 0;
@@ -1021,7 +1024,7 @@ int npfem_create(const npfem_mesh* mesh, const npfem_material* mat, const npfem_
     if ((rc = done("H~"))) return bail(rc);
     if (frc) return bail(fail(frc, err));
     float *a32 = nullptr, *m32 = nullptr;
-    if (dense) {
+    if (few) {
         a32 = h->alloc<float>((size_t)np * np, &e);
         if (e) return bail(e);
     }

@@ -76,7 +76,7 @@ struct TopoDev {
     const unsigned short* ring8_idx;  // [n][8]
     const T* ring8_c;                 // [n][8]
     const T* ring8_ct;                // [n][8]
-    const T* ainv;               // FP32, up to kDenseVerts: [n_pad][n_pad] A^-1 (zero padding); else null
+    const T* ainv;               // where applies_dense(): [n_pad][n_pad] A^-1 in FP32 (zero padding); else null
     int dense_p;                 // parts of every 128-row tile's columns (dense_parts)
     SparseDev<T> sp;             // without ainv: sparse block factor of H~ (applied as H~^-1)
     SparseDev<T> spc;            // the same, cut finer, for a cluster's warps (FP64; else null)
@@ -329,7 +329,7 @@ inline void place_vectors(GroupDesc<T>* g, int n, int n_pad, int nt, int npos, i
     const int ws_bytes = ((n_pad + 15) & ~15) * 16 * 4;
     const int slot_bytes8 = 24 * n_pad * (int)sizeof(T);  // [8 slots][3][n_pad] corner gradients
     // and the dense contraction's partial sums (384 floats per item)
-    const int dn_bytes = sizeof(T) == 4 && n <= kTcMaxVerts ? dense_parts(n) * ((n + 127) / 128) * 384 * 4 : 0;
+    const int dn_bytes = sizeof(T) == 4 && n <= kDenseFewVerts ? dense_parts(n) * ((n + 127) / 128) * 384 * 4 : 0;
     int tb = tri_bytes > slot_bytes8 ? tri_bytes : slot_bytes8;
     tb = tb > dn_bytes ? tb : dn_bytes;
     tb = ((tb > ws_bytes ? tb : ws_bytes) + 15) & ~15;
@@ -466,7 +466,12 @@ struct npfem_handle {
     int tev_used = 0;
     std::mutex mu;
 
-    // Positions of the sparse factor (0: the cells apply the dense inverse).
+    // Do its cells apply the dense inverse in a SIMT launch of `cells`?
+    bool applies_dense(long long cells) const
+    {
+        return npfem::applies_dense(precision == NPFEM_PREC_FP64, precision == NPFEM_PREC_FP32, mat.beta_D > 0.0, n, cells);
+    }
+    // Positions of the sparse factor (0: the cells always apply the dense inverse).
     int npos() const { return precision == NPFEM_PREC_FP64 ? td.sp.npos : tf.sp.npos; }
     // Can the tensor-core cluster kernel take this handle's cells?  With beta_D > 0 only those of
     // meshes above kDenseVerts: below, FP32 blocks are as fast or faster (damped, two steps,

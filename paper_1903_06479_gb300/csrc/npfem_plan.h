@@ -27,12 +27,28 @@ NPFEM_HD inline long long carry_head_elems(int m) { return 4 + (((long long)m * 
 NPFEM_HD inline long long carry_rec_elems(int n_pad, int m) { return carry_head_elems(m) + 2LL * m * 3 * n_pad; }
 
 // Meshes whose FP32 cells apply the dense inverse; finer ones (and FP64) apply the sparse
-// factor.  A matter of the mesh alone, so that a cell's arithmetic does not depend on the
-// other cells of its call: the two differ in the order of their sums.  At 642 vertices the
-// inverse is 1.65 MB from L2 in 48.5 K cycles, the factor 0.47 MB in eleven steps in 41 K, and
-// a population takes the same time with either (1520 cells 1869 / 1726 us, 3001 cells of 258
-// 2.38 / 2.99 ms); above, the factor wins at every count (FP32, dense / sparse: DENSEFIGS).
-constexpr int kDenseVerts = 700;
+// factor.  A matter of the mesh, so that a cell's arithmetic does not depend on the other
+// groups of its call: the two differ in the order of their sums.  At 642 vertices the inverse is
+// 1.65 MB from L2 in 48.5 K cycles, the factor 0.47 MB in eleven steps in 41 K, and a population
+// takes the same time with either (1520 cells 1869 / 1726 us, 3001 cells of 258 2.38 / 2.99 ms);
+// at 1026 vertices (37 cells, four steps) 2.65 / 2.24 ms.
+//
+// One exception: launches of at most kDenseFewCells cells of an FP32 handle keep the dense
+// inverse up to kDenseFewVerts vertices, and its time (1026 x 1, four steps, 2418 us; the
+// factor 2095).  Another order of the sums moves velocities by about 6e-8 um/us.  Among many
+// cells that is 3e-6 of the fastest; one slow cell's velocities moved by 1e-4 of their size
+// (1026 x 1 at a low shear rate, where either order is 2e-3 from FP64), and a few cells may all
+// be slow.  Eight cells drawn from the shear rates of 10 to 1000 / s are all below 100 / s once in
+// 10^8.  BF16 and TF32 handles, whose contractions were never these, take the factor.
+constexpr int kDenseVerts = 700, kDenseFewVerts = 1100, kDenseFewCells = 8;
+
+// Do the cells of a mesh of n vertices apply the dense inverse in a SIMT launch of `cells`?
+// (fp64, fp32: the handle's precision is NPFEM_PREC_FP64, NPFEM_PREC_FP32.)
+inline bool applies_dense(bool fp64, bool fp32, bool damped, int n, long long cells)
+{
+    if (fp64 || n > kDenseFewVerts) return false;
+    return n <= kDenseVerts || (fp32 && !damped && cells <= kDenseFewCells);
+}
 
 // Block size of a SIMT group: a mesh's evaluation keeps about n / 32 warps busy and most of
 // its phases are latency-bound, so when every SM has several cells to solve, two blocks of

@@ -90,6 +90,7 @@ int run_static(npfem_handle* const* meshes, int n_groups, const int32_t* cells, 
         npfem_handle* h = meshes[gi];
         GroupDesc<T>& g = a.g[gi];
         g.topo = *reinterpret_cast<const TopoDev<T>*>(sizeof(T) == 4 ? (const void*)&h->tf : (const void*)&h->td);
+        if (!h->applies_dense(all)) g.topo.ainv = nullptr;
         g.cell_begin = total;
         g.state_off = state;
         g.stats_off = total;

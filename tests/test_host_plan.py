@@ -42,6 +42,11 @@ int main()
             if (scanf("%d %d %d %d %lld %d", &n, &fp64, &dense, &damped, &cells, &eval) != 6) return 1;
             const SimtMesh m = {n, fp64 != 0, dense != 0, damped != 0};
             printf("%d\n", eval ? eval_threads(m, cells, 152) : simt_threads(m, cells, 152));
+        } else if (!strcmp(what, "dense")) {
+            int fp64, fp32, damped, n;
+            long long cells;
+            if (scanf("%d %d %d %d %lld", &fp64, &fp32, &damped, &n, &cells) != 5) return 1;
+            printf("%d\n", (int)applies_dense(fp64 != 0, fp32 != 0, damped != 0, n, cells));
         } else if (!strcmp(what, "buffers")) {
             // one handle's buffer: "n<bytes>" needs room, "c<bytes>" the same inside a capture of the
             // library, "u<bytes>" inside another one, "g" a graph was made, "d" one is destroyed;
@@ -157,3 +162,13 @@ def test_buffers_of_live_graphs_are_not_freed(plan, ops, want):
 ])
 def test_block_sizes(plan, mesh, want):
     assert int(plan("threads %d %d %d %d %d %d" % mesh)[0]) == want
+
+
+# FP64, FP32, damped, vertices, cells of the launch (BF16 and TF32 handles are neither FP64 nor FP32)
+@pytest.mark.parametrize("case,want", [
+    ((0, 1, 0, 700, 1), 1), ((0, 1, 0, 700, 16384), 1), ((0, 0, 0, 700, 16384), 1), ((0, 1, 1, 642, 1), 1),
+    ((0, 1, 0, 701, 8), 1), ((0, 1, 0, 701, 9), 0), ((0, 1, 0, 1100, 8), 1), ((0, 1, 0, 1101, 1), 0),
+    ((0, 0, 0, 701, 1), 0), ((0, 1, 1, 701, 1), 0), ((1, 0, 0, 66, 1), 0),
+])
+def test_dense_inverse_by_mesh(plan, case, want):
+    assert int(plan("dense %d %d %d %d %d" % case)[0]) == want
