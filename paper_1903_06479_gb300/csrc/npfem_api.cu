@@ -309,7 +309,8 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
         g.carry_rec = carry_recs ? carry_recs[gi] : 0;
         g.carry_off = carry_offs ? carry_offs[gi] : 0;
         long long sb = 0;
-        place_vectors(&g, h->n, h->n_pad, h->nt, h->npos(), h0->opts.lbfgs_m, budget, &sb);
+        // (an evaluation solves nothing: no room for the solve's vectors)
+        place_vectors(&g, h->n, h->n_pad, h->nt, mode == 1 ? 0 : h->npos(), h0->opts.lbfgs_m, budget, &sb);
         slot = std::max(slot, sb);
         smem_max = std::max(smem_max, g.smem_bytes);
         total += cells[gi];
