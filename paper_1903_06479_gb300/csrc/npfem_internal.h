@@ -281,6 +281,10 @@ cudaError_t symmetrise(double* A, int n, int n_pad, float* out, cudaStream_t s);
 // loads into tensor memory.
 cudaError_t publish_inverse_bf16_blocked(const double* A, int n, int rows_pad, int kpad, void* out, cudaStream_t s);
 
+// Lets a kernel have as much dynamic shared memory as a block can: the same value whoever
+// sets it, so that host threads whose launches need different amounts do not lower each
+// other's limit between setting it and launching.
+cudaError_t allow_smem(const void* kernel);
 template <typename T>
 cudaError_t launch_cells(const LaunchArgs<T>& a, int grid, int block, int smem, cudaStream_t s);
 // Resident blocks per SM of the SIMT launch `a` at this block size and dynamic shared memory.

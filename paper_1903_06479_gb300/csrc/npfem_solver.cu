@@ -78,12 +78,20 @@ cudaLaunchConfig_t tc_config(int cluster, int block, int smem, int grid, cudaStr
 
 }  // namespace
 
+cudaError_t allow_smem(const void* k)
+{
+    int dev = 0, limit = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return e == cudaSuccess ? cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) : e;
+}
+
 template <typename T>
 cudaError_t cells_per_sm(const LaunchArgs<T>& a, int block, int smem, int* n)
 {
     const void* k = simt_kernel(a, block);
     if (!k) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(k);
     return e == cudaSuccess ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k, block, smem) : e;
 }
 
@@ -92,7 +100,7 @@ cudaError_t launch_cells(const LaunchArgs<T>& a, int grid, int block, int smem, 
 {
     const void* k = simt_kernel(a, block);
     if (!k) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(k);
     if (e != cudaSuccess) return e;
     void* args[1] = {const_cast<LaunchArgs<T>*>(&a)};
     e = cudaLaunchKernel(k, dim3(grid), dim3(block), args, smem, s);
@@ -103,7 +111,7 @@ cudaError_t launch_cells(const LaunchArgs<T>& a, int grid, int block, int smem, 
 cudaError_t query_cells_cl(int cluster, int block, int smem, int* max_clusters)
 {
     const void* k = cell_kernel_cl_f64();
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(k);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = tc_config(cluster, block, smem, cluster, nullptr, attr);
@@ -113,7 +121,7 @@ cudaError_t query_cells_cl(int cluster, int block, int smem, int* max_clusters)
 cudaError_t launch_cells_cl(const LaunchArgs<double>& a, int cluster, int clusters, int block, int smem, cudaStream_t s)
 {
     const void* k = cell_kernel_cl_f64();
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(k);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = tc_config(cluster, block, smem, cluster * clusters, s, attr);
@@ -127,7 +135,7 @@ cudaError_t query_cells_tc(int cluster, bool damped, int block, int smem, int* m
 {
     const void* k = tc_kernel(cluster, damped);
     if (!k) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(k);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = tc_config(cluster, block, smem, cluster, nullptr, attr);
@@ -139,13 +147,12 @@ cudaError_t query_cells_tc(int cluster, bool damped, int block, int smem, int* m
     return cudaSuccess;
 }
 
-// Cluster launch of the tensor-core kernel for one mesh group.  Its shared memory is set
-// here as for the other kernels: handles of several meshes share the kernel.
+// Cluster launch of the tensor-core kernel for one mesh group.
 cudaError_t launch_cells_tc(const LaunchArgs<float>& a, int cluster, int block, int smem, int grid, cudaStream_t s)
 {
     const void* k = tc_kernel(cluster, a.g[0].topo.l_ptr != nullptr);
     if (!k) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(k);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = tc_config(cluster, block, smem, grid, s, attr);
