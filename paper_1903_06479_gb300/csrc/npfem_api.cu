@@ -90,6 +90,9 @@ int upload_sparse(npfem_handle* h, const SparseHost& F, SparseDev<T>* sp)
     sp->row = reinterpret_cast<const int2*>(drow);
     sp->npos = F.npos;
     for (int v = 0; v < kSparseScheds; ++v) {
+        sp->sched[v] = nullptr;
+        sp->entries[v] = 0;
+        if (F.sched[v].empty()) continue;
         const int* ds = nullptr;
         if ((rc = upload(h, F.sched[v], &ds))) return rc;
         sp->sched[v] = reinterpret_cast<const int4*>(ds);

@@ -4,10 +4,10 @@
 // instructions per triangle and evaluation); eight share them, and what is left is the
 // latency of one triangle's chain (one 258-vertex cell, four steps: 10.9 ms by one block of
 // 512 threads, 6.18 by eight of 512, 4.64 by eight of 128, which do not run the reductions
-// on warps without data).  In
-// FP32 a block's evaluation is too short to pay for the cluster barriers (one 642-vertex
-// cell, eight steps: 1.31 ms by one block, 1.35 ms by eight), so FP32 stays at a block per
-// cell.  Clusters take the cells in turn.
+// on warps without data).  FP32 stays at a block per cell: with eight blocks of 512 threads and
+// the sparse solve (a cluster barrier per level) one 642-vertex cell took 1.35 ms for eight
+// steps, by one block with the dense inverse 1.31; blocks of 128 threads, or a cluster that
+// only shares the dense contraction, were not tried.  Clusters take the cells in turn.
 #pragma once
 
 #include "npfem_cell.cuh"

@@ -29,7 +29,8 @@ constexpr int kTriRow = 12;
 
 enum Vec { V_XN = 0, V_U = 1, V_UT = 2, V_G = 3, V_GT = 4, V_GC = 5, V_UY = 6, V_D = 7, V_TRI = 8, V_WR = 9, V_SBASE = 10 };
 
-// Schedules of the sparse solve by warps per block.
+// Schedules of the sparse solve by warps: a block per cell has 4 to 16 (the first three), a
+// cluster per cell 8 to 128 (the last five); a factor holds those its launches take.
 constexpr int kSparseScheds = 6;
 NPFEM_HD constexpr int sparse_sched_warps(int v) { return 4 << v; }
 NPFEM_HD constexpr int sparse_sched_of(int warps) { return warps <= 4 ? 0 : (warps <= 8 ? 1 : (warps <= 16 ? 2 : (warps <= 32 ? 3 : (warps <= 64 ? 4 : 5)))); }
@@ -233,7 +234,7 @@ struct SparseHost {
     std::vector<int> rows;              // [rows][2] position written (-1: none), vertex (-1: forward row)
     std::vector<unsigned short> idx;    // [iterations][32] group index: positions 4 g .. 4 g + 3
     std::vector<double> val;            // [iterations][32][4]
-    std::vector<int> sched[kSparseScheds];  // [entries][warps][4]: slice, barrier after it in bit 8 of lg
+    std::vector<int> sched[kSparseScheds];  // (empty where not needed) [entries][warps][4]: slice, barrier after it in bit 8 of lg
 };
 constexpr int kSparseWarps = 16;     // warps a step's work is spread over
 constexpr int kSparseWarpsCluster = 64;  // the same for a cluster per cell

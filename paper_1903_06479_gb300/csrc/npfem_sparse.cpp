@@ -1,6 +1,6 @@
 // Host-side, once-per-topology sparse factorisation of H~ in FP64 (not on the timed
 // path): nested dissection of the mesh and a block LDL^T over its separator tree, laid
-// out for solve_sparse() in npfem_solver.cu.
+// out for solve_sparse() in npfem_cell.cuh.
 //
 // H~ couples a vertex with its two-ring, so a closed surface mesh splits by short rings
 // of vertices (separators): 642 vertices need 92 K factor entries against 412 K of the
@@ -265,7 +265,8 @@ int build_sparse_factor(const HostTopo& H, const double* rest, double mass_scale
     std::vector<std::vector<std::pair<int, int>>> below(n);  // (node, column of W) per boundary vertex
     for (size_t k = 0; k < N.size(); ++k)
         for (size_t j = 0; j < N[k].B.size(); ++j) below[N[k].B[j]].push_back({(int)k, (int)j});
-    auto lay_out = [&](SparseHost* o, int warps) {
+    // for the schedules [sched0, sched1)
+    auto lay_out = [&](SparseHost* o, int warps, int sched0, int sched1) {
     o->rows.clear();
     o->idx.clear();
     o->val.clear();
@@ -388,7 +389,7 @@ int build_sparse_factor(const HostTopo& H, const double* rest, double mass_scale
     }
 
     // schedules: the warps take a step's slices in turn; the last of a step ends in a barrier
-    for (int v = 0; v < kSparseScheds; ++v) {
+    for (int v = sched0; v < sched1; ++v) {
         const int nw = sparse_sched_warps(v);
         std::vector<int>& sc = o->sched[v];
         sc.clear();
@@ -406,11 +407,11 @@ int build_sparse_factor(const HostTopo& H, const double* rest, double mass_scale
         }
     }
     };
-    lay_out(out, kSparseWarps);
+    lay_out(out, kSparseWarps, 0, 3);
     if (out_cluster) {
         out_cluster->npos = out->npos;
         out_cluster->perm = out->perm;
-        lay_out(out_cluster, kSparseWarpsCluster);
+        lay_out(out_cluster, kSparseWarpsCluster, 1, kSparseScheds);
     }
     return 0;
 }
