@@ -12,7 +12,7 @@
 // and unit normal n_k at the current positions; their stencil sums meet in two shuffles.
 // Lattice coordinates are sums of two floats (lattice_base), weights and sums FP32.
 // Measured on 1024 cells of 642 vertices, 121^3 nodes: forcing with three cycles (four
-// spreads and four gathers) 3.0 -> 1.06 ms against one thread per vertex with scalar
+// spreads and four gathers) 3.0 -> 1.02 ms against one thread per vertex with scalar
 // atomics and FP64 coordinates.
 //
 // Conventions (the paper prints the formulas in lattice units, dx = 1):
@@ -371,6 +371,7 @@ __device__ __forceinline__ void take_sum(const IbmArgs& a, long long so, int n, 
 }
 
 // One vertex of a phase straight on the lattice.
+template <bool kSpread>
 __device__ __forceinline__ void vertex_phase(const IbmArgs& a, const IbmGroup& G, long long cell, int i, int q, bool live)
 {
     const LatDev& L = a.lat;
@@ -380,7 +381,7 @@ __device__ __forceinline__ void vertex_phase(const IbmArgs& a, const IbmGroup& G
     Stencil s;
     float wq;
     make_stencil(L, xc, n, i, q, s, &wq);
-    if (a.phase == 1) {
+    if constexpr (kSpread) {
         // Step 1: spread f_k with weight A_k dx / dx^3 per unit stencil weight
         float A;
         area_normal4<false>(G.topo, xc, i, q, &A, nullptr);
@@ -393,16 +394,17 @@ __device__ __forceinline__ void vertex_phase(const IbmArgs& a, const IbmGroup& G
             const float wgt = s.w[1][r & 3] * s.w[2][r >> 2];
             if (live && nd >= 0) red4(a.lat_out + 4 * nd, wgt * f[0], wgt * f[1], wgt * f[2], a.lat_vec);
         }
-        return;
+    } else {
+        float u[3];
+        gather4(L, s, q, wq, a.field, a.phase == 2 ? a.field2 : nullptr, a.dt, u);
+        take_sum(a, so, n, i, q, live, u);
     }
-    float u[3];
-    gather4(L, s, q, wq, a.field, a.phase == 2 ? a.field2 : nullptr, a.dt, u);
-    take_sum(a, so, n, i, q, live, u);
 }
 
 // Velocity interpolation (phase -1) and the phases of the multi-direct forcing, vertex by
-// vertex (few cells, or small ones).
-__global__ void __launch_bounds__(256, 4) ibm_forcing_kernel(const __grid_constant__ IbmArgs a)
+// vertex.  The gathers run with four blocks per SM (gather4), the spread with three.
+template <bool kSpread>
+__global__ void __launch_bounds__(256, kSpread ? 3 : 4) ibm_forcing_kernel(const __grid_constant__ IbmArgs a)
 {
     for (long long v0 = blockIdx.x * (long long)kVertsPerBlock; v0 < a.total_verts; v0 += (long long)gridDim.x * kVertsPerBlock) {
         const long long gv = v0 + (threadIdx.x >> 2);
@@ -410,7 +412,7 @@ __global__ void __launch_bounds__(256, 4) ibm_forcing_kernel(const __grid_consta
         long long cell;
         int i;
         const IbmGroup& G = locate(a, live ? gv : a.total_verts - 1, &cell, &i);
-        vertex_phase(a, G, cell, i, threadIdx.x & 3, live);
+        vertex_phase<kSpread>(a, G, cell, i, threadIdx.x & 3, live);
     }
 }
 
@@ -486,7 +488,7 @@ __global__ void __launch_bounds__(256, 3) ibm_gather_kernel(const __grid_constan
             const bool live = v0 + (tid >> 2) < n;
             const int i = live ? v0 + (tid >> 2) : n - 1;
             if (!fits) {
-                vertex_phase(a, G, cell, i, q, live);
+                vertex_phase<false>(a, G, cell, i, q, live);
                 continue;
             }
             Stencil s;
@@ -584,7 +586,9 @@ cudaError_t launch_forcing(const IbmArgs& a, npfem_handle* const* meshes, double
         const int grid = (int)std::min<long long>(a.total_cells, (long long)std::max(h->sm_count, 1) * 4);
         ibm_gather_kernel<<<grid, 256, smem, s>>>(a);
     } else {
-        ibm_forcing_kernel<<<ibm_grid(h, a.total_verts), 256, 0, s>>>(a);
+        const int grid = ibm_grid(h, a.total_verts);
+        if (a.phase == 1) ibm_forcing_kernel<true><<<grid, 256, 0, s>>>(a);
+        else ibm_forcing_kernel<false><<<grid, 256, 0, s>>>(a);
     }
     count_launch();
     return cudaGetLastError();
