@@ -280,3 +280,17 @@ def test_static_step_of_small_fp64_meshes(N, sizes, cells):
     torch.cuda.synchronize()
     lb = min(h.rest_info()[1]["lbar"] for h in hs)
     assert float((x - xs).abs().max()) <= 1e-10 * lb and float((v - vs).abs().max()) * DT <= 1e-10 * lb
+
+
+def test_stretched_equilibria_of_the_dense_inverse_and_the_factor(N):
+    """A 1026-vertex cell stretched to 200 pN: an FP32 handle alone (dense inverse) and a TF32 handle
+    (the same FP32 path with the sparse factor) reach the same equilibrium, by the tolerance of the
+    equilibria against the oracle (2e-3 of the diameters)."""
+    from paper_1903_06479_gb300 import validation as V
+    forces = (100.0, 200.0)
+    r = {p: V.stretching(sizes=(1026,), forces_pN=forces, precision=p)[1026] for p in ("fp32", "tf32")}
+    for p in r:
+        assert max(r[p]["move"]) < 1e-4, (p, r[p]["move"])  # settled
+    for k in ("DA", "DT"):
+        a, b = np.array(r["fp32"][k]), np.array(r["tf32"][k])
+        assert (np.abs(a - b) <= 2e-3 * a).all(), (k, a, b)
