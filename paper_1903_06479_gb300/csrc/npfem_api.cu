@@ -344,7 +344,7 @@ int run_cells(npfem_handle* const* meshes, int n_groups, const int32_t* cells, T
 
     const int smem = kFixedSmem + smem_max;
     int per_sm = 1;
-    NPFEM_CUDA(cells_per_sm<T>(a, threads, smem, &per_sm));
+    NPFEM_CUDA(cells_per_sm<T>(a, threads, smem, h0->smem_optin, &per_sm));
     per_sm = std::max(per_sm, 1);
     long long grid = std::min<long long>(total, (long long)h0->sm_count * per_sm);
     a.slot_bytes = slot;
@@ -406,7 +406,7 @@ int run_cells_cluster(npfem_handle* const* meshes, int n_groups, const int32_t* 
         const int smem = kFixedSmem + smem_max;
         const int key = smem + (block << 20);
         if (h0->cl_smem[lg] != key) {
-            NPFEM_CUDA(query_cells_cl(C, block, smem, &h0->cl_max[lg]));
+            NPFEM_CUDA(query_cells_cl(C, block, smem, h0->smem_optin, &h0->cl_max[lg]));
             h0->cl_smem[lg] = key;
         }
         if (h0->cl_max[lg] < total) continue;
@@ -484,7 +484,8 @@ int run_cells_tc(npfem_handle* h, int cells, float* x, float* v, const float* f,
     int smem = kFixedSmem + g.smem_bytes;
     smem = std::max(smem, h->smem_optin / 2 + 4096);
     if (h->tc_smem != smem) {
-        NPFEM_CUDA(query_cells_tc(cluster, h->mat.beta_D > 0.0, kTcThreads, smem, &h->tc_max_clusters));
+        NPFEM_CUDA(query_cells_tc(cluster, h->mat.beta_D > 0.0, kTcThreads, smem, h->smem_optin,
+                                  &h->tc_max_clusters));
         h->tc_smem = smem;
     }
     const int max_clusters = h->tc_max_clusters;
@@ -529,6 +530,7 @@ int run_cells_tc(npfem_handle* h, int cells, float* x, float* v, const float* f,
     NPFEM_CUDA(launch_cells_tc(a, cluster, kTcThreads, smem, grid, stream));
     if (helper > 0) {
         cudaError_t e = cudaStreamWaitEvent(h->side_stream, h->ev_fork, 0);
+        if (e == cudaSuccess) e = allow_cells_smem<float>(b, kTcThreads, h->smem_optin);
         if (e == cudaSuccess) e = launch_cells<float>(b, helper, kTcThreads, smem_b, h->side_stream);
         if (e != cudaSuccess) {
             // the clusters alone cannot reset the shared counters: clear them behind

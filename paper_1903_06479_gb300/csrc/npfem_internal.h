@@ -282,21 +282,24 @@ cudaError_t symmetrise(double* A, int n, int n_pad, float* out, cudaStream_t s);
 // loads into tensor memory.
 cudaError_t publish_inverse_bf16_blocked(const double* A, int n, int rows_pad, int kpad, void* out, cudaStream_t s);
 
-// Lets a kernel have as much dynamic shared memory as a block can: the same value whoever
-// sets it, so that host threads whose launches need different amounts do not lower each
-// other's limit between setting it and launching.
-cudaError_t allow_smem(const void* kernel);
+// Lets a kernel have `limit` dynamic shared memory: always the most a block can have on the
+// device (npfem_handle::smem_optin), the same value whoever sets it, so that host threads
+// whose launches need different amounts do not lower each other's.  A launch comes after
+// cells_per_sm, allow_cells_smem or its kernel's query on the same device.
+cudaError_t allow_smem(const void* kernel, int limit);
+template <typename T>
+cudaError_t allow_cells_smem(const LaunchArgs<T>& a, int block, int limit);
 template <typename T>
 cudaError_t launch_cells(const LaunchArgs<T>& a, int grid, int block, int smem, cudaStream_t s);
 // Resident blocks per SM of the SIMT launch `a` at this block size and dynamic shared memory.
 template <typename T>
-cudaError_t cells_per_sm(const LaunchArgs<T>& a, int block, int smem, int* n);
+cudaError_t cells_per_sm(const LaunchArgs<T>& a, int block, int smem, int limit, int* n);
 // Tensor-core kernel (BF16, A^-1 row blocks resident in TMEM across a cluster): sets
 // its shared-memory size and returns how many clusters can be resident at once.
-cudaError_t query_cells_tc(int cluster, bool damped, int block, int smem, int* max_clusters);
+cudaError_t query_cells_tc(int cluster, bool damped, int block, int smem, int limit, int* max_clusters);
 // Cluster kernel for few FP64 cells: how many clusters of this size can be resident at once, and
 // its launch on `clusters` of them.
-cudaError_t query_cells_cl(int cluster, int block, int smem, int* max_clusters);
+cudaError_t query_cells_cl(int cluster, int block, int smem, int limit, int* max_clusters);
 cudaError_t launch_cells_cl(const LaunchArgs<double>& a, int cluster, int clusters, int block, int smem, cudaStream_t s);
 // Launch of one mesh group on `grid` blocks (a multiple of the cluster size).
 cudaError_t launch_cells_tc(const LaunchArgs<float>& a, int cluster, int block, int smem, int grid, cudaStream_t s);

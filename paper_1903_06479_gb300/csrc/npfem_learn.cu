@@ -577,7 +577,7 @@ cudaError_t launch_ws_temporal(const npfem_handle* h, int n_cells, const float* 
     if (n_cells <= 0) return cudaSuccess;
     const int np = h->n_pad, n16 = (h->n + 15) & ~15;
     const int smem = kFixedSmem + 12 * np * (int)sizeof(float) + 16 * n16 * (int)sizeof(float);
-    cudaError_t e = allow_smem(reinterpret_cast<const void*>(&ws_temporal_kernel));
+    cudaError_t e = allow_smem(reinterpret_cast<const void*>(&ws_temporal_kernel), h->smem_optin);
     if (e != cudaSuccess) return e;
     const int per_sm = smem <= h->smem_optin / 2 ? 2 : 1;
     const int grid = std::min(n_cells, per_sm * h->sm_count);
@@ -593,7 +593,7 @@ cudaError_t launch_ws_increments(const npfem_handle* h, int n_cells, const float
     if (n_cells <= 0) return cudaSuccess;
     const int np = h->n_pad, n16 = (h->n + 15) & ~15;
     const int smem = kFixedSmem + 9 * np * (int)sizeof(float) + 16 * n16 * (int)sizeof(float);
-    cudaError_t e = allow_smem(reinterpret_cast<const void*>(&ws_increment_kernel));
+    cudaError_t e = allow_smem(reinterpret_cast<const void*>(&ws_increment_kernel), h->smem_optin);
     if (e != cudaSuccess) return e;
     const int per_sm = smem <= h->smem_optin / 2 ? 2 : 1;
     const int grid = std::min(n_cells, per_sm * h->sm_count);
@@ -667,7 +667,7 @@ int npfem_ws_features(npfem_handle* h, int n_cells, const float* x, const float*
     if (n_cells == 0) return 0;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int smem = kFixedSmem + 3 * 3 * h->n_pad * (int)sizeof(float);
-    cudaError_t e = allow_smem(reinterpret_cast<const void*>(&ws_features_kernel));
+    cudaError_t e = allow_smem(reinterpret_cast<const void*>(&ws_features_kernel), h->smem_optin);
     if (e != cudaSuccess) return set_error(NPFEM_ERR_CUDA, std::string("npfem_ws_features: ") + cudaGetErrorString(e));
     ws_features_kernel<<<std::min(n_cells, 4 * h->sm_count), 256, smem, s>>>(h->tf, n_cells, x, v, f, x_next, feat, target);
     count_launch();
@@ -690,7 +690,7 @@ int npfem_ws_features_temporal(npfem_handle* h, int n_cells, const float* x, con
     if (n_cells == 0) return 0;
     const int np = h->n_pad, n16 = (h->n + 15) & ~15;
     const int smem = kFixedSmem + 12 * np * (int)sizeof(float) + 16 * n16 * (int)sizeof(float);
-    cudaError_t e = allow_smem(reinterpret_cast<const void*>(&ws_temporal_kernel));
+    cudaError_t e = allow_smem(reinterpret_cast<const void*>(&ws_temporal_kernel), h->smem_optin);
     if (e == cudaSuccess) {
         const int grid = std::min(n_cells, 2 * h->sm_count);
         ws_temporal_kernel<<<grid, 512, smem, s>>>(tp, n_cells, x, v, f, f_prev, c1, c2, x_next, feat, target, c_out,

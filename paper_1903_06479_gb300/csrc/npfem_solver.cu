@@ -78,20 +78,24 @@ cudaLaunchConfig_t tc_config(int cluster, int block, int smem, int grid, cudaStr
 
 }  // namespace
 
-cudaError_t allow_smem(const void* k)
+cudaError_t allow_smem(const void* k, int limit)
 {
-    int dev = 0, limit = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    return e == cudaSuccess ? cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) : e;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
 }
 
 template <typename T>
-cudaError_t cells_per_sm(const LaunchArgs<T>& a, int block, int smem, int* n)
+cudaError_t allow_cells_smem(const LaunchArgs<T>& a, int block, int limit)
+{
+    const void* k = simt_kernel(a, block);
+    return k ? allow_smem(k, limit) : cudaErrorInvalidValue;
+}
+
+template <typename T>
+cudaError_t cells_per_sm(const LaunchArgs<T>& a, int block, int smem, int limit, int* n)
 {
     const void* k = simt_kernel(a, block);
     if (!k) return cudaErrorInvalidValue;
-    cudaError_t e = allow_smem(k);
+    cudaError_t e = allow_smem(k, limit);
     return e == cudaSuccess ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k, block, smem) : e;
 }
 
@@ -100,18 +104,16 @@ cudaError_t launch_cells(const LaunchArgs<T>& a, int grid, int block, int smem, 
 {
     const void* k = simt_kernel(a, block);
     if (!k) return cudaErrorInvalidValue;
-    cudaError_t e = allow_smem(k);
-    if (e != cudaSuccess) return e;
     void* args[1] = {const_cast<LaunchArgs<T>*>(&a)};
-    e = cudaLaunchKernel(k, dim3(grid), dim3(block), args, smem, s);
+    const cudaError_t e = cudaLaunchKernel(k, dim3(grid), dim3(block), args, smem, s);
     if (e == cudaSuccess) count_launch();
     return e;
 }
 
-cudaError_t query_cells_cl(int cluster, int block, int smem, int* max_clusters)
+cudaError_t query_cells_cl(int cluster, int block, int smem, int limit, int* max_clusters)
 {
     const void* k = cell_kernel_cl_f64();
-    cudaError_t e = allow_smem(k);
+    cudaError_t e = allow_smem(k, limit);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = tc_config(cluster, block, smem, cluster, nullptr, attr);
@@ -121,21 +123,19 @@ cudaError_t query_cells_cl(int cluster, int block, int smem, int* max_clusters)
 cudaError_t launch_cells_cl(const LaunchArgs<double>& a, int cluster, int clusters, int block, int smem, cudaStream_t s)
 {
     const void* k = cell_kernel_cl_f64();
-    cudaError_t e = allow_smem(k);
-    if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = tc_config(cluster, block, smem, cluster * clusters, s, attr);
     void* args[1] = {const_cast<LaunchArgs<double>*>(&a)};
-    e = cudaLaunchKernelExC(&cfg, k, args);
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, k, args);
     if (e == cudaSuccess) count_launch();
     return e;
 }
 
-cudaError_t query_cells_tc(int cluster, bool damped, int block, int smem, int* max_clusters)
+cudaError_t query_cells_tc(int cluster, bool damped, int block, int smem, int limit, int* max_clusters)
 {
     const void* k = tc_kernel(cluster, damped);
     if (!k) return cudaErrorInvalidValue;
-    cudaError_t e = allow_smem(k);
+    cudaError_t e = allow_smem(k, limit);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = tc_config(cluster, block, smem, cluster, nullptr, attr);
@@ -152,19 +152,18 @@ cudaError_t launch_cells_tc(const LaunchArgs<float>& a, int cluster, int block, 
 {
     const void* k = tc_kernel(cluster, a.g[0].topo.l_ptr != nullptr);
     if (!k) return cudaErrorInvalidValue;
-    cudaError_t e = allow_smem(k);
-    if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = tc_config(cluster, block, smem, grid, s, attr);
     void* args[1] = {const_cast<LaunchArgs<float>*>(&a)};
-    e = cudaLaunchKernelExC(&cfg, k, args);
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, k, args);
     if (e == cudaSuccess) count_launch();
     return e;
 }
 
 template cudaError_t launch_cells<float>(const LaunchArgs<float>&, int, int, int, cudaStream_t);
 template cudaError_t launch_cells<double>(const LaunchArgs<double>&, int, int, int, cudaStream_t);
-template cudaError_t cells_per_sm<float>(const LaunchArgs<float>&, int, int, int*);
-template cudaError_t cells_per_sm<double>(const LaunchArgs<double>&, int, int, int*);
+template cudaError_t allow_cells_smem<float>(const LaunchArgs<float>&, int, int);
+template cudaError_t cells_per_sm<float>(const LaunchArgs<float>&, int, int, int, int*);
+template cudaError_t cells_per_sm<double>(const LaunchArgs<double>&, int, int, int, int*);
 
 }  // namespace npfem

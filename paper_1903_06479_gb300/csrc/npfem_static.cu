@@ -127,7 +127,7 @@ int run_static(npfem_handle* const* meshes, int n_groups, const int32_t* cells, 
 
     const int smem = kFixedSmem + smem_max;
     int per_sm = 1;
-    cudaError_t e = cells_per_sm<T>(a, threads, smem, &per_sm);
+    cudaError_t e = cells_per_sm<T>(a, threads, smem, h0->smem_optin, &per_sm);
     if (e != cudaSuccess) return set_error(NPFEM_ERR_CUDA, std::string("npfem_step_static: ") + cudaGetErrorString(e));
     per_sm = std::max(per_sm, 1);
     long long grid = std::min<long long>(total, (long long)h0->sm_count * per_sm);
