@@ -294,8 +294,8 @@ cudaError_t launch_cells(const LaunchArgs<T>& a, int grid, int block, int smem, 
 // Resident blocks per SM of the SIMT launch `a` at this block size and dynamic shared memory.
 template <typename T>
 cudaError_t cells_per_sm(const LaunchArgs<T>& a, int block, int smem, int limit, int* n);
-// Tensor-core kernel (BF16, A^-1 row blocks resident in TMEM across a cluster): sets
-// its shared-memory size and returns how many clusters can be resident at once.
+// Tensor-core kernel (BF16, A^-1 row blocks resident in TMEM across a cluster): how many
+// clusters can be resident at once at this shared memory.
 cudaError_t query_cells_tc(int cluster, bool damped, int block, int smem, int limit, int* max_clusters);
 // Cluster kernel for few FP64 cells: how many clusters of this size can be resident at once, and
 // its launch on `clusters` of them.

@@ -82,6 +82,15 @@ inline int simt_threads(const SimtMesh& m, long long cells, long long sms)
     return m.n > 384 && (double)singles < pair * (double)pairs ? 512 : 256;
 }
 
+// The same for an evaluation of the objective, which applies no inverse: finer meshes gain
+// nothing from smaller blocks, whose vectors spill (evaluations of 1026 x 160, 400 and 600
+// cells, 512 / 256 threads: 78 / 78, 113 / 138, 147 / 146 us; 786: 69 / 63, 98 / 110, 126 / 114;
+// 642: 54 / 48, 77 / 78, 98 / 84).
+inline int eval_threads(const SimtMesh& m, long long cells, long long sms)
+{
+    return !m.fp64 && m.n > kDenseVerts ? 512 : simt_threads(m, cells, sms);
+}
+
 // One group of a call: its mesh, its own handle's L-BFGS window, and whether its cells go to
 // the tensor-core cluster kernel (with its own handle's options).
 struct PlanGroup {
@@ -96,15 +105,6 @@ inline int simt_lead(const std::vector<PlanGroup>& groups)
     for (size_t g = 0; g < groups.size(); ++g)
         if (groups[g].cells > 0 && !groups[g].clusters) return (int)g;
     return -1;
-}
-
-// The same for an evaluation of the objective, which applies no inverse: finer meshes gain
-// nothing from smaller blocks, whose vectors spill (evaluations of 1026 x 160, 400 and 600
-// cells, 512 / 256 threads: 78 / 78, 113 / 138, 147 / 146 us; 786: 69 / 63, 98 / 110, 126 / 114;
-// 642: 54 / 48, 77 / 78, 98 / 84).
-inline int eval_threads(const SimtMesh& m, long long cells, long long sms)
-{
-    return !m.fp64 && m.n > kDenseVerts ? 512 : simt_threads(m, cells, sms);
 }
 
 // Where every group's carried pairs lie in the call's buffer, in elements: its first record and
